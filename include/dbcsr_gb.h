@@ -84,7 +84,7 @@ typedef struct {
     /* BF16 products (the tensor-core tier on groups of atom blocks): */
     double flops_tensor;       /* executed MMA flops, 2 M N K per MMA, padding and every split product counted */
     double bytes_tensor;       /* bytes its bulk copies move from global into shared memory */
-    int64_t n_tiles;           /* group tiles of C formed */
+    int64_t n_tiles;           /* group tiles of C formed (FP64 products too: 0 without tensor cores) */
 } dbcsr_mult_stats;
 
 /* Options of the sign iteration. */
@@ -303,8 +303,8 @@ dbcsr_status dbcsr_multiply(double alpha, dbcsr_matrix A, dbcsr_matrix B, double
  *     queue (an atomic counter over the shape lists) and run the single-warp kernel of each
  *     block's shape (K-split where m n = 32 EF + 1).  Products with a shape of more than 17
  *     element slots per lane (m n > 544) keep the per-shape launches.
- * Every C element is summed in the same order either way; the block norms differ only in
- * rounding where the per-shape schedule uses warp pairs.  Library-wide; not from the paper.
+ * It concerns the blocks the FP64 units compute (dbcsr_multiply).  Every C element is summed in
+ * the same order either way; the block norms differ only in rounding where the per-shape schedule uses warp pairs.  Library-wide; not from the paper.
  * Errors: EINVAL (unknown mode).
  */
 #define DBCSR_SCHEDULE_PER_SHAPE 0

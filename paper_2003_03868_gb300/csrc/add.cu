@@ -164,6 +164,7 @@ void add(dbcsr_matrix_* A, double alpha, const dbcsr_matrix_* B, double beta) {
     A->data = std::move(data);
     A->nnzb = nb;
     A->nel = nel;
+    A->exact_sym = A->exact_sym && B->exact_sym;
     A->norms_valid = false;
 }
 

@@ -363,6 +363,7 @@ dbcsr_status sign_iterate_batched(int32_t nsys, dbcsr_matrix_* const* H, const d
             nbs.insert(nbs.end(), cur_bs.begin() + act_beg[a], cur_bs.begin() + act_beg[a + 1]);
             nbeg.push_back((int32_t)nbs.size());
         }
+        std::shared_ptr<Groups> kept_groups;
         auto rebuild = [&](const dbcsr_matrix_* m, const std::vector<int64_t>& b, const std::vector<int64_t>& e) {
             int64_t nnzb_new = 0, nel_new = 0;
             for (size_t a = 0; a < na; ++a)
@@ -389,9 +390,20 @@ dbcsr_status sign_iterate_batched(int32_t nsys, dbcsr_matrix_* const* H, const d
             y->nel = nel_new;
             y->norms_valid = false;
             y->finalized = true;
+            y->exact_sym = m->exact_sym;
+            y->groups = kept_groups;
             return y;
         };
         if (!nact.empty()) {
+            // the block groups stay those of the first product, so that a system's later products
+            // are the same sums as without the batch
+            if (X->groups) {
+                std::vector<int32_t> rows;
+                for (size_t a = 0; a < na; ++a)
+                    if (!leave[a])
+                        for (int32_t i = act_beg[a]; i < act_beg[a + 1]; ++i) rows.push_back(i);
+                kept_groups = groups_of_rows(*X->groups, rows, nbs, st);
+            }
             // each old matrix is freed (stream-ordered, after its copies) before the next is rebuilt
             X = rebuild(X.get(), xb, xe);
             if (x2) X2 = rebuild(x2, yb, ye);

@@ -146,7 +146,8 @@ constexpr int kGroupMembers = 16;
 constexpr int32_t kMaxBlockRowsLt = 262144;
 struct Groups {
     int32_t ngrp = 0, nblk = 0, max_members = 0;
-    std::vector<int32_t> h_w;            // host copy of the widths
+    std::vector<int32_t> h_w;            // host copies of the widths and of g_of
+    std::vector<int32_t> h_of;
     DBuf<int32_t> g_of;                  // [nblk] group of every block
     DBuf<int32_t> g_pos;                 // [nblk] first row of the block inside its group
     DBuf<int32_t> g_ptr;                 // [ngrp + 1] members of group k: g_mem[g_ptr[k] .. g_ptr[k+1])
@@ -176,6 +177,10 @@ struct dbcsr_matrix_ {
     dbg::DBuf<double> data;              // [nel] blocks row-major, packed in CSR order
     dbg::DBuf<double> norms;             // [nnzb] Frobenius norms (valid iff norms_valid)
     bool norms_valid = false;
+
+    // values and pattern known to be exactly symmetric (results of products of the sign
+    // iteration and what keeps the property); false only means not known
+    bool exact_sym = false;
 
     int plans = 0;                       // live multiply plans that use this matrix's arrays
 
@@ -207,6 +212,7 @@ void det_sum_into(const double* v, int64_t n, double* partials, double* out, cud
 void check_finalized(const dbcsr_matrix_* m);
 void ensure_norms(dbcsr_matrix_* m);
 void compute_block_norms(const dbcsr_matrix_* m, double* norms, double* dev2);
+void block_norms(const dbcsr_matrix_* m, double* norms, cudaStream_t s);
 void copy_matrix(dbcsr_matrix_* dst, const dbcsr_matrix_* src);
 void scale_shift(dbcsr_matrix_* m, double scale, double shift);
 // Keeps the blocks whose flag is nonzero (norms, when given, are compacted too).
@@ -239,8 +245,13 @@ void trace_product_parts_into(dbcsr_matrix_* a, dbcsr_matrix_* b, double* part, 
 //                (for operands that commute only approximately, e.g. BF16 products).
 constexpr int kSymNone = 0, kSymMirror = 1, kSymAverage = 2;
 struct LowTierPlan;
+struct F64TcPlan;
+// One-off and planned products below this many flops (counted over both triangles) stay on the FP64
+// pipe: such a product is launch-bound on either path, and the tensor cores' needs more launches.
+constexpr double kTcMinFlops = 64e6;
 // m <- (m + m^T) / 2 on the blocks that have a twin; blocks without one are dropped.
 void symmetrize(dbcsr_matrix_* m);
+void mark_if_symmetric(dbcsr_matrix_* m);
 // A planned product C = alpha A B on fixed patterns: the buffers its numeric phase needs
 // and that phase captured as one CUDA graph (dbcsr_multiply_plan).
 struct MultPlan {
@@ -256,12 +267,17 @@ struct MultPlan {
     std::vector<DBuf<__nv_bfloat16>> bufs_bf16;
     std::vector<DBuf<uint8_t>> bufs_u8;
     LowTierPlan* lt = nullptr;           // BF16 products: the tensor-core tier's symbolic results
+    F64TcPlan* tc = nullptr;             // FP64 products: the digit tiles of the tensor-core blocks
     ~MultPlan();
 };
+// tc_min_flops: FP64 products of fewer flops do not use the tensor cores.  The iterations leave it
+// at 0: the choice then depends on each tile alone, and a system's products are the same sums in
+// a batch as on their own.
 // plan: build a plan instead of a one-off product (beta = 0, C distinct from A and B, no
 // symmetric result); C then holds the formed pattern with blocks under eps zeroed.
 void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbcsr_matrix_* C, double eps,
-              int prec, dbcsr_mult_stats* stats, bool want_dev2, int sym_result = kSymNone, MultPlan* plan = nullptr);
+              int prec, dbcsr_mult_stats* stats, bool want_dev2, int sym_result = kSymNone, MultPlan* plan = nullptr,
+              double tc_min_flops = 0.0);
 void execute_plan(MultPlan* plan);
 // Fails with DBCSR_ESTATE when a live plan uses m's arrays (they must not be replaced).
 void check_unplanned(const dbcsr_matrix_* m, const char* where);
@@ -269,6 +285,10 @@ void check_unplanned(const dbcsr_matrix_* m, const char* where);
 // ---- lowtier.cu
 // Groups of neighbouring blocks from the strongest couplings (block norms) of m.
 std::shared_ptr<Groups> build_groups(dbcsr_matrix_* m);
+std::shared_ptr<Groups> groups_of(const std::vector<int32_t>& root, const std::vector<int32_t>& bs, cudaStream_t s);
+// g restricted to the given block rows (ascending, whole groups), renumbered; bs: their edges.
+std::shared_ptr<Groups> groups_of_rows(const Groups& g, const std::vector<int32_t>& rows, const std::vector<int32_t>& bs,
+                                       cudaStream_t s);
 // Where the tensor-core tier writes: the formed blocks of the product (CSR over block rows,
 // computed flags, element offsets, C input) and the result arrays.
 struct LowTierOut {
@@ -297,6 +317,35 @@ int64_t lowtier_tiles(const LowTierPlan& L);
 // its bulk copies move into shared memory.
 double lowtier_tensor_flops(const LowTierPlan& L);
 double lowtier_copy_bytes(const LowTierPlan& L);
+
+// ---- fp64tc.cu
+// The formed blocks of an FP64 product and their choice between the FP64 pipe and the tensor cores.
+struct F64TcBlocks {
+    const int32_t* row; const int32_t* col; const int64_t* mirror; const int32_t* ksum;
+    const float* max_term;               // largest |alpha| ||A_IK|| ||B_KJ|| of every block
+    uint8_t* comp;                       // out: 0 copied or dropped, 1 FP64 pipe, 2 tensor cores
+    int sym, by_group;                   // as block_role's
+};
+void f64tc_delete(F64TcPlan* p);
+// Tile patterns, stacks and digit tiles of C = alpha A B and the blocks the tensor cores take;
+// null when the product does not fit them (then comp is not complete).
+std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A, dbcsr_matrix_* B,
+                                                               std::shared_ptr<Groups> groups, int64_t nform,
+                                                               const int64_t* f_rp, const F64TcBlocks& f, double alpha,
+                                                               cudaStream_t s);
+// The current values into the digit tiles (f64tc_prepare has done it for its values).
+void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s);
+// After f64tc_pack of a planned product's new values: the flag returned (device) becomes nonzero when
+// a tensor-core block needs the FP64 pipe with them.  an, bn: room for the operands' block norms.
+const int* f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, double* an, double* bn,
+                         int64_t nform, const F64TcBlocks& f, const int64_t* f_pbeg, const int32_t* prod_a,
+                         const int32_t* prod_b, double alpha, cudaStream_t s);
+void f64tc_run(F64TcPlan& L, const LowTierOut& o, cudaStream_t s);
+void f64tc_norms(int64_t nform, const uint8_t* comp, const int32_t* row, const int32_t* col, const int32_t* bs,
+                 const int64_t* off, const double* data, double* norms, double* dev2, cudaStream_t s);
+int64_t f64tc_tiles(const F64TcPlan& L);
+// Fails with DBCSR_ETIMEOUT when a bounded wait of the kernel ran out (synchronises s).
+void f64tc_check(F64TcPlan& L, cudaStream_t s);
 
 // ---- dense.cu
 // C[b] = alpha A[b] B[b] + beta C[b] for nb row-major n x n matrices (b < 65536): FP64 on the

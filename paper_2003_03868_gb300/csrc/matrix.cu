@@ -276,6 +276,13 @@ __global__ void k_compact_data(int64_t nb, const int32_t* __restrict__ keep, con
 
 }  // namespace
 
+void block_norms(const dbcsr_matrix_* m, double* norms, cudaStream_t s) {
+    if (m->nnzb == 0) return;
+    k_block_norms<<<grid_for(m->nnzb, 8), 256, 0, s>>>(m->nnzb, m->row.p, m->col.p, m->bs.p, m->off.p, m->data.p, norms,
+                                                       nullptr);
+    DBG_LAUNCH_CK();
+}
+
 void compute_block_norms(const dbcsr_matrix_* m, double* norms, double* dev2) {
     if (m->nnzb == 0) return;
     k_block_norms<<<grid_for(m->nnzb, 8), 256, 0, m->stream>>>(m->nnzb, m->row.p, m->col.p, m->bs.p, m->off.p,
@@ -311,6 +318,7 @@ void copy_matrix(dbcsr_matrix_* dst, const dbcsr_matrix_* src) {
     if (src->nel) DBG_CK(cudaMemcpyAsync(dst->data.p, src->data.p, sizeof(double) * src->nel, cudaMemcpyDeviceToDevice, s));
     dst->nnzb = src->nnzb;
     dst->nel = src->nel;
+    dst->exact_sym = src->exact_sym;
     dst->norms_valid = false;
     if (src->norms_valid && src->nnzb) {
         dst->norms.alloc(src->nnzb, s);
@@ -397,6 +405,8 @@ void filter_matrix(dbcsr_matrix_* m, double eps, const double* norms_in) {
     keep.alloc(m->nnzb, s);
     k_keep_norm<<<grid_for(m->nnzb, 256), 256, 0, s>>>(m->nnzb, m->row.p, m->col.p, norms_in, eps, keep.p);
     DBG_LAUNCH_CK();
+    // a block and its transpose sum their norms in another order: the kept pattern may lose its twins
+    m->exact_sym = false;
     // norms_in may be owned by m: compact() replaces m->norms only after reading it
     compact(m, keep.p, norms_in);
 }
@@ -597,6 +607,7 @@ dbcsr_status dbcsr_put_values(dbcsr_matrix m, const double* data, int on_device)
             DBG_CK(cudaMemcpyAsync(m->data.p, data, sizeof(double) * m->nel,
                                    on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, m->stream));
         if (!on_device) DBG_CK(cudaStreamSynchronize(m->stream));
+        m->exact_sym = false;
         m->norms_valid = false;
     });
 }
@@ -855,7 +866,8 @@ dbcsr_status dbcsr_filter(dbcsr_matrix m, double eps) {
 
 dbcsr_status dbcsr_multiply(double alpha, dbcsr_matrix A, dbcsr_matrix B, double beta, dbcsr_matrix C,
                             double eps_filter, int32_t prec, dbcsr_mult_stats* stats) {
-    return guarded([&] { dbg::multiply(alpha, A, B, beta, C, eps_filter, prec, stats, stats != nullptr); });
+    return guarded([&] { dbg::multiply(alpha, A, B, beta, C, eps_filter, prec, stats, stats != nullptr, dbg::kSymNone, nullptr,
+                                        dbg::kTcMinFlops); });
 }
 
 dbcsr_status dbcsr_trace(dbcsr_matrix A, double* out) {

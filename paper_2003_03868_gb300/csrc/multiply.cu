@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "grouptiles.cuh"
 #include "smm.cuh"
 
 namespace dbg {
@@ -144,6 +145,8 @@ struct BoundArgs {
     int use_smem;
     int use_fast;            // FP32 upper bound with atomics (needs use_smem and < 4096 terms per candidate)
     const float* b_norm_ru;  // use_fast: B's norms rounded up to FP32, once per block
+    float* max_term;         // per candidate (nullable): its largest |alpha| ||A_IK|| ||B_KJ||
+    unsigned long long* flops;   // sum of 2 m n k over the kept candidates
 };
 
 // B's block norms rounded up to FP32 for the fast bound: one conversion per block instead of one
@@ -170,10 +173,16 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
     for (int32_t I = blockIdx.x; I < nblk; I += gridDim.x) {
         const int nc = build_row(P, I, bm, wpre, nwords, sh_scan);
         const int64_t cb = B.coff[I];
+        // per candidate in shared memory: use_fast the FP32 bound, the packed counters (terms,
+        // below 4096, in the low 12 bits, the sum of k above) and the largest term, 12 bytes;
+        // otherwise the FP64 bound, the two counters and the largest term
         double* bnd = B.use_smem ? sh_bound : B.bound + cb;
         int32_t* pc = B.use_smem ? (int32_t*)(sh_bound + nc) : B.pcnt + cb;
         int32_t* ks = B.use_smem ? pc + nc : B.ksum + cb;
-        float* fb = (float*)(pc + 2 * nc);      // use_fast: FP32 bounds after the counters
+        float* fb = (float*)sh_bound;
+        unsigned* pk = (unsigned*)(fb + nc);
+        float* mx = B.use_fast ? (float*)(pk + nc) : B.use_smem ? (float*)(ks + nc) : B.max_term + cb;
+        const bool want_max = B.max_term != nullptr;
         // candidates in ascending J
         for (int w = threadIdx.x; w < nwords; w += blockDim.x) {
             uint32_t bits = bm[w];
@@ -183,10 +192,15 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
                 bits &= bits - 1u;
                 B.cand_col[cb + r] = 32 * w + b;
                 B.cand_row[cb + r] = I;
-                bnd[r] = 0.0;
-                pc[r] = 0;
-                ks[r] = 0;
-                if (B.use_fast) fb[r] = 0.f;
+                if (B.use_fast) {
+                    fb[r] = 0.f;
+                    pk[r] = 0u;
+                } else {
+                    bnd[r] = 0.0;
+                    pc[r] = 0;
+                    ks[r] = 0;
+                }
+                if (want_max) mx[r] = 0.f;
                 if (B.cin) B.cin[cb + r] = -1;
                 ++r;
             }
@@ -199,17 +213,18 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
             // warps over K, lanes over the blocks of B's row K, no barrier
             for (int64_t p = P.a_rp[I] + warp; p < P.a_rp[I + 1]; p += nw) {
                 const int32_t K = P.a_col[p];
-                const float na = (float)(B.abs_alpha * B.a_norm[p]) * 1.0009765625f;
-                const int kk = B.bs[K];
+                const float na = __fmul_ru(__double2float_ru(B.abs_alpha * B.a_norm[p]), 1.0009765625f);
+                const unsigned kk = ((unsigned)B.bs[K] << 12) | 1u;
                 for (int64_t q = P.b_rp[K] + lane; q < P.b_rp[K + 1]; q += 32) {
                     const int r = rank_of(bm, wpre, P.b_col[q]);
-                    atomicAdd(&fb[r], __fmul_ru(na, B.b_norm_ru[q]));
-                    atomicAdd(&pc[r], 1);
-                    atomicAdd(&ks[r], kk);
+                    // (a norm past FP32's range is infinite here; times a zero norm it is still zero)
+                    const float nb = B.b_norm_ru[q];
+                    const float term = na == 0.f || nb == 0.f ? 0.f : __fmul_ru(na, nb);
+                    atomicAdd(&fb[r], term);
+                    atomicAdd(&pk[r], kk);
+                    if (want_max) atomicMax((int*)&mx[r], __float_as_int(term));
                 }
             }
-            __syncthreads();
-            for (int r = threadIdx.x; r < nc; r += blockDim.x) bnd[r] = (double)fb[r] * 1.0009765625;
         } else {
             __syncthreads();
             // ascending K, one K at a time: every accumulator is updated in a fixed order
@@ -219,25 +234,36 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
                 const int kk = B.bs[K];
                 for (int64_t q = P.b_rp[K] + threadIdx.x; q < P.b_rp[K + 1]; q += blockDim.x) {
                     const int r = rank_of(bm, wpre, P.b_col[q]);
-                    bnd[r] = bnd[r] + na * B.b_norm[q];
+                    const double term = na * B.b_norm[q];
+                    bnd[r] = bnd[r] + term;
                     pc[r] += 1;
                     ks[r] += kk;
+                    if (want_max) mx[r] = fmaxf(mx[r], (float)term);
                 }
                 __syncthreads();
             }
         }
         __syncthreads();
+        unsigned long long fl = 0;
+        const int mI = B.bs[I];
         for (int r = threadIdx.x; r < nc; r += blockDim.x) {
-            double b = bnd[r];
+            double b = B.use_fast ? (double)fb[r] * 1.0009765625 : bnd[r];
             const int64_t ci = B.cin ? B.cin[cb + r] : -1;
             if (ci >= 0) b += B.abs_beta * B.c_norm[ci];
             const int32_t J = B.cand_col[cb + r];
-            B.keep[cb + r] = (J == I || b >= B.eps_lo) ? 1 : 0;
+            const int keep = (J == I || b >= B.eps_lo) ? 1 : 0;
+            B.keep[cb + r] = keep;
+            const int k = B.use_fast ? (int)(pk[r] >> 12) : ks[r];
             if (B.use_smem) {
-                B.pcnt[cb + r] = pc[r];
-                B.ksum[cb + r] = ks[r];
+                B.pcnt[cb + r] = B.use_fast ? (int)(pk[r] & 4095u) : pc[r];
+                B.ksum[cb + r] = k;
+                if (want_max) B.max_term[cb + r] = mx[r];
             }
+            if (keep) fl += 2ull * (unsigned long long)(mI * B.bs[J]) * (unsigned long long)k;
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) fl += __shfl_xor_sync(0xffffffffu, fl, o);
+        if (lane == 0 && fl) atomicAdd(B.flops, fl);
         __syncthreads();
     }
 }
@@ -254,7 +280,8 @@ __global__ void k_form_meta(int64_t ncand, const int32_t* __restrict__ keep, con
                             const int32_t* __restrict__ pcnt, const int32_t* __restrict__ ksum,
                             const int64_t* __restrict__ cin, const int32_t* __restrict__ bs,
                             int32_t* __restrict__ f_row, int32_t* __restrict__ f_col, int64_t* __restrict__ f_area,
-                            int64_t* __restrict__ f_np, int64_t* __restrict__ f_cin, int32_t* __restrict__ f_ksum) {
+                            int64_t* __restrict__ f_np, int64_t* __restrict__ f_cin, int32_t* __restrict__ f_ksum,
+                            const float* __restrict__ max_term, float* __restrict__ f_max) {
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncand; c += (int64_t)gridDim.x * blockDim.x) {
         if (!keep[c]) continue;
         const int64_t k = kidx[c];
@@ -265,6 +292,7 @@ __global__ void k_form_meta(int64_t ncand, const int32_t* __restrict__ keep, con
         f_np[k] = pcnt[c];
         f_cin[k] = cin ? cin[c] : -1;
         f_ksum[k] = ksum[c];
+        if (f_max) f_max[k] = max_term[c];
     }
 }
 
@@ -292,20 +320,6 @@ __global__ void k_find_mirror(int64_t nform, const int32_t* __restrict__ f_row, 
         }
         mirror[k] = src;
     }
-}
-
-// role of formed block k: 0 computed, 1 copied from its twin, 2 dropped.
-// sym = 1 (mirror): I < J computed, I > J copied; sym = 2 (average): both twins
-// computed and then replaced by their symmetric mean; blocks without a formed twin
-// are dropped in both modes.
-// grp (BF16 products, nullable): blocks are ordered by their group first, so that all the
-// computed blocks between two groups lie in one group tile of the tensor-core tier.
-__device__ __forceinline__ int block_role(int sym, int32_t I, int32_t J, int64_t mirror, const int32_t* grp) {
-    if (!sym || I == J) return 0;
-    if (mirror < 0) return 2;
-    if (sym == 2) return 0;
-    const bool first = grp ? (grp[I] < grp[J] || (grp[I] == grp[J] && I < J)) : I < J;
-    return first ? 0 : 1;
 }
 
 // One warp: the m x m block P becomes (P + P^T) / 2 in place; *sq and *d receive the
@@ -409,35 +423,38 @@ __global__ void k_sym_average(int64_t nform, const int64_t* __restrict__ mirror,
 }
 
 // Work of the blocks that are computed (not mirrored): flops, products, and a
-// histogram by block shape (m, n).  Blocks that are copied or dropped get no product
-// stack (f_np = 0, comp = 0).
+// histogram by block shape (m, n) of those the FP64 pipe takes.  Blocks that are copied or
+// dropped get no product stack (f_np = 0, comp = 0).  tc: comp is given (f64tc_prepare), 2 for
+// the blocks the tensor cores take; they count as work, their stacks are kept only for a plan's
+// fallback (keep_tc), and their shapes go to a second histogram.
 __global__ void k_form_stats(int64_t nform, const int32_t* __restrict__ f_row, const int32_t* __restrict__ f_col,
                              int64_t* __restrict__ f_np, const int32_t* __restrict__ f_ksum,
                              const int64_t* __restrict__ mirror, int sym, const int32_t* __restrict__ bs,
                              unsigned long long* __restrict__ flops, unsigned long long* __restrict__ nprod,
                              unsigned long long* __restrict__ shape_cnt, uint8_t* __restrict__ comp,
-                             const int32_t* __restrict__ grp) {
+                             const int32_t* __restrict__ grp, int by_group, int tc, int keep_tc) {
     // the shape histogram is gathered per CTA in shared memory (a few shapes take every block,
     // so global atomics per block would serialise on them) and added once per nonzero bin
     constexpr int kBins = (kMaxBlock + 1) * (kMaxBlock + 1);
-    __shared__ unsigned int hist[kBins];
-    for (int t = threadIdx.x; t < kBins; t += blockDim.x) hist[t] = 0;
+    __shared__ unsigned int hist[2 * kBins];
+    for (int t = threadIdx.x; t < 2 * kBins; t += blockDim.x) hist[t] = 0;
     __syncthreads();
     unsigned long long lf = 0, lp = 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nform; k += (int64_t)gridDim.x * blockDim.x) {
-        const bool computed = block_role(sym, f_row[k], f_col[k], mirror[k], grp) == 0;
-        comp[k] = computed ? 1 : 0;
-        if (!computed) {
+        const int c = tc ? comp[k] : block_role(sym, f_row[k], f_col[k], mirror[k], grp, by_group) == 0 ? 1 : 0;
+        if (!tc) comp[k] = (uint8_t)c;
+        if (!c) {
             f_np[k] = 0;
             continue;
         }
         const int m = bs[f_row[k]], n = bs[f_col[k]];
         lf += 2ull * (unsigned long long)m * (unsigned long long)n * (unsigned long long)f_ksum[k];
         lp += (unsigned long long)f_np[k];
-        atomicAdd(&hist[m * (kMaxBlock + 1) + n], 1u);
+        if (c == 2 && !keep_tc) f_np[k] = 0;
+        atomicAdd(&hist[(c == 2 ? kBins : 0) + m * (kMaxBlock + 1) + n], 1u);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < kBins; t += blockDim.x)
+    for (int t = threadIdx.x; t < (tc ? 2 : 1) * kBins; t += blockDim.x)
         if (hist[t]) atomicAdd(shape_cnt + t, (unsigned long long)hist[t]);
     for (int o = 16; o > 0; o >>= 1) {
         lf += __shfl_xor_sync(0xffffffffu, lf, o);
@@ -456,11 +473,11 @@ __global__ void k_mirror_copy(int64_t nform, int sym, const int64_t* __restrict_
                               const int32_t* __restrict__ f_row, const int32_t* __restrict__ f_col,
                               const int64_t* __restrict__ f_off, const int32_t* __restrict__ bs,
                               double* __restrict__ c_data, double* __restrict__ c_norm, double* __restrict__ c_dev2,
-                              const int32_t* __restrict__ grp) {
+                              const int32_t* __restrict__ grp, int by_group) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < nform; k += warps) {
-        const int role = block_role(sym, f_row[k], f_col[k], mirror[k], grp);
+        const int role = block_role(sym, f_row[k], f_col[k], mirror[k], grp, by_group);
         if (role == 0) continue;
         if (role == 2) {
             if (lane == 0) {
@@ -503,7 +520,8 @@ __global__ void k_form_rp(int32_t nblk, const int64_t* __restrict__ coff, const 
 struct FillArgs {
     const int64_t* coff;
     const int32_t* keep;
-    const uint8_t* comp;     // per formed block: 1 if computed (only those get stack entries)
+    const uint8_t* comp;     // per formed block: 1 if the FP64 pipe computes it, 2 the tensor cores
+    int comp_max;            // blocks with 1 <= comp <= comp_max get stack entries
     const int64_t* kidx;
     const int64_t* pbeg;
     int32_t* cursor;
@@ -525,7 +543,8 @@ __global__ void k_fill_stack(int32_t nblk, RowPattern P, int nwords, FillArgs F)
             int32_t* cur = (int32_t*)(sh_base + nc);
             for (int r = threadIdx.x; r < nc; r += blockDim.x) {
                 const int64_t c = cb + r;
-                sh_base[r] = (F.keep[c] && F.comp[F.kidx[c]]) ? F.pbeg[F.kidx[c]] : -1;
+                const int cp = F.keep[c] ? F.comp[F.kidx[c]] : 0;
+                sh_base[r] = (cp && cp <= F.comp_max) ? F.pbeg[F.kidx[c]] : -1;
                 cur[r] = 0;
             }
             __syncthreads();
@@ -554,7 +573,7 @@ __global__ void k_fill_stack(int32_t nblk, RowPattern P, int nwords, FillArgs F)
                     const int64_t c = cb + rank_of(bm, wpre, P.b_col[q]);
                     if (!F.keep[c]) continue;
                     const int64_t k = F.kidx[c];
-                    if (!F.comp[k]) continue;
+                    if (!F.comp[k] || F.comp[k] > F.comp_max) continue;
                     const int32_t at = cur[k - kb];
                     cur[k - kb] = at + 1;
                     const int64_t pos = F.pbeg[k] + at;
@@ -690,6 +709,7 @@ __global__ void __launch_bounds__(256) k_smm_f64(int64_t nlist, const int64_t* _
     // element slots, so a large block needs half the registers per thread; the halves'
     // norm sums meet in shared memory behind a 64-thread named barrier of the pair.
     __shared__ double sh_part[PAIR ? 4 : 1][2][2];
+    if (S.gate && *S.gate == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = PAIR ? (warp & 1) : 0, pair = PAIR ? (warp >> 1) : warp;
     const int per_cta = PAIR ? (blockDim.x >> 6) : (blockDim.x >> 5);
@@ -794,6 +814,7 @@ __device__ __forceinline__ void smm_block_ks(int64_t k, const SmmArgs& S, int la
 
 template <int EF, int R>
 __global__ void __launch_bounds__(256) k_smm_f64_ks(int64_t nlist, const int64_t* __restrict__ list, SmmArgs S) {
+    if (S.gate && *S.gate == 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps)
@@ -804,6 +825,7 @@ __global__ void __launch_bounds__(256) k_smm_f64_ks(int64_t nlist, const int64_t
 // CTAs of 256 threads per SM (80 registers, no spills): at the uncapped 98 registers only two
 // fit, and the operand loads' latency showed (FP64 pipe 72% busy).
 __global__ void __launch_bounds__(256, 3) k_smm_f64_ks5(int64_t nlist, const int64_t* __restrict__ list, SmmArgs S) {
+    if (S.gate && *S.gate == 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps)
@@ -854,14 +876,12 @@ __global__ void __launch_bounds__(256, 2) k_smm_f64_queue(int64_t nlist, const i
 }
 
 
-// Stable partition of the formed blocks by shape: flag[k] = (block k is m x n).
+// Stable partition of the formed blocks by shape: flag[k] = (block k is m x n and comp[k] == want).
 __global__ void k_shape_flags(int64_t nform, const int32_t* __restrict__ f_row, const int32_t* __restrict__ f_col,
-                              const int32_t* __restrict__ bs, const int64_t* __restrict__ mirror, int sym, int m, int n,
+                              const int32_t* __restrict__ bs, const uint8_t* __restrict__ comp, int want, int m, int n,
                               int32_t* __restrict__ flag) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nform; k += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t I = f_row[k], J = f_col[k];
-        flag[k] = (bs[I] == m && bs[J] == n && block_role(sym, I, J, mirror[k], nullptr) == 0) ? 1 : 0;
-    }
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nform; k += (int64_t)gridDim.x * blockDim.x)
+        flag[k] = (comp[k] == want && bs[f_row[k]] == m && bs[f_col[k]] == n) ? 1 : 0;
 }
 
 __global__ void k_class_scatter(int64_t nform, const int32_t* __restrict__ flag, const int64_t* __restrict__ pos,
@@ -949,6 +969,35 @@ struct EventSet {
 
 int sym_grid(int32_t nblk) { return std::min<int32_t>(nblk, num_sms() * 8); }
 
+// Counts the blocks on or above the diagonal that differ from their twin's transpose, and those below
+// it without a twin (one warp per block).
+__global__ void k_asymmetric(int64_t nb, const int32_t* __restrict__ row, const int32_t* __restrict__ col,
+                             const int64_t* __restrict__ rp, const int64_t* __restrict__ off,
+                             const int32_t* __restrict__ bs, const double* __restrict__ data,
+                             unsigned long long* __restrict__ diff) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < nb; k += warps) {
+        const int32_t I = row[k], J = col[k];
+        int64_t lo = rp[J], hi = rp[J + 1];
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (col[mid] < I) lo = mid + 1; else hi = mid;
+        }
+        bool same = lo < rp[J + 1] && col[lo] == I;
+        if (same && I <= J) {
+            const int m = bs[I], n = bs[J];
+            const long long* P = reinterpret_cast<const long long*>(data + off[k]);
+            const long long* Q = reinterpret_cast<const long long*>(data + off[lo]);
+            for (int e = lane; e < m * n; e += 32) {
+                const int i = e / n, j = e - i * n;
+                same = same && P[e] == Q[j * m + i];
+            }
+        }
+        if (!__all_sync(0xffffffffu, same) && lane == 0) atomicAdd(diff, 1ull);
+    }
+}
+
 __global__ void k_keep_twinned(int64_t nb, const int64_t* __restrict__ mirror, int32_t* __restrict__ keep) {
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x)
         keep[b] = mirror[b] >= 0 ? 1 : 0;
@@ -1016,6 +1065,19 @@ void launch_smm_shape(int m, int n, int64_t cnt, const int64_t* list, const SmmA
     DBG_LAUNCH_CK();
 }
 
+// Sets m->exact_sym when m equals its transpose, values (bit for bit) and pattern.
+void mark_if_symmetric(dbcsr_matrix_* m) {
+    cudaStream_t s = m->stream;
+    if (m->nnzb == 0) return;
+    DBuf<int64_t> diff;
+    diff.alloc(1, s);
+    diff.zero();
+    k_asymmetric<<<grid_for(m->nnzb, 8), 256, 0, s>>>(m->nnzb, m->row.p, m->col.p, m->rp.p, m->off.p, m->bs.p, m->data.p,
+                                                      (unsigned long long*)diff.p);
+    DBG_LAUNCH_CK();
+    m->exact_sym = read_i64(diff.p, s) == 0;
+}
+
 void symmetrize(dbcsr_matrix_* m) {
     check_finalized(m);
     check_unplanned(m, "symmetrize");
@@ -1037,10 +1099,11 @@ void symmetrize(dbcsr_matrix_* m) {
     k_keep_twinned<<<grid_for(nb, 256), 256, 0, s>>>(nb, mirror.p, keep.p);
     DBG_LAUNCH_CK();
     compact(m, keep.p, nullptr);
+    m->exact_sym = true;
 }
 
 void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbcsr_matrix_* C, double eps, int prec,
-              dbcsr_mult_stats* stats, bool want_dev2, int sym_result, MultPlan* plan) {
+              dbcsr_mult_stats* stats, bool want_dev2, int sym_result, MultPlan* plan, double tc_min_flops) {
     check_finalized(A);
     check_finalized(B);
     if (!C) fail(DBCSR_EINVAL, "multiply: null C");
@@ -1074,7 +1137,6 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         A->groups = groups;
     }
     if (groups && groups->nblk != nblk) groups.reset();
-    const int32_t* grp = bf16 ? groups->g_of.p : nullptr;
 
     EventSet ev;
     DBG_CK(cudaEventRecord(ev.e[0], s));
@@ -1086,11 +1148,13 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     const size_t sm_rank = (size_t)2 * ((nwords + 1) & ~1) * sizeof(uint32_t);
     RowPattern P{A->rp.p, A->col.p, B->rp.p, B->col.p, use_c ? C->rp.p : nullptr, use_c ? C->col.p : nullptr};
 
+    if (sym_result == kSymMirror && !bf16 && A == B && !A->exact_sym) mark_if_symmetric(A);
+
     // 1. candidate counts
     DBuf<int64_t> ccnt, coff, maxrow;
     ccnt.alloc(nblk, s);
     coff.alloc(nblk + 1, s);
-    maxrow.alloc(2, s);                   // largest candidate count and largest A row of a block row
+    maxrow.alloc(3, s);                   // largest candidate count and A row of a block row; flops of the kept
     maxrow.zero();
     {
         const size_t sm = sm_rank;
@@ -1118,10 +1182,14 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     keep.alloc(nc1, s);
     kidx.alloc(ncand + 1, s);
     if (use_c) cin.alloc(nc1, s);
-    const size_t sm_acc = sm_rank + (size_t)max_row * (sizeof(double) + 2 * sizeof(int32_t) + sizeof(float));
-    const bool acc_smem = sm_acc <= (size_t)kSymSmemBudget;
     // a candidate's bound has at most (largest A row) terms: the FP32 margin covers 4095
-    const bool fast_bound = acc_smem && max_arow < 4096;
+    const bool few_terms = max_arow < 4096;
+    const size_t sm_acc = sm_rank + (size_t)max_row * (few_terms ? 2 * sizeof(float) + sizeof(unsigned)
+                                                                 : sizeof(double) + 2 * sizeof(int32_t) + sizeof(float));
+    const bool acc_smem = sm_acc <= (size_t)kSymSmemBudget;
+    const bool fast_bound = acc_smem && few_terms;
+    DBuf<float> max_term;                 // FP64 products: for the choice between the FP64 pipe and the tensor cores
+    if (!bf16) max_term.alloc(nc1, s);
     if (!acc_smem) bound.alloc(nc1, s);
     if (ncand) {
         DBuf<float> b_norm_ru;
@@ -1133,20 +1201,39 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         BoundArgs ba{std::fabs(alpha), std::fabs(beta), eps * (1.0 - 1e-12), A->norms.p, B->norms.p,
                      use_c ? C->norms.p : nullptr, A->bs.p, coff.p, cand_row.p, cand_col.p,
                      bound.p, pcnt.p, ksum.p, use_c ? cin.p : nullptr, keep.p, acc_smem ? 1 : 0,
-                     fast_bound ? 1 : 0, b_norm_ru.p};
+                     fast_bound ? 1 : 0, b_norm_ru.p, max_term.p, (unsigned long long*)maxrow.p + 2};
         const size_t sm = acc_smem ? sm_acc : sm_rank;
         allow_dyn_smem(k_cand_bound, sm);
         k_cand_bound<<<sym_grid(nblk), kSymThreads, sm, s>>>(nblk, P, nwords, ba);
         DBG_LAUNCH_CK();
     }
     scan_exclusive(keep.p, kidx.p, ncand, s);
-    const int64_t nform = read_i64(kidx.p + ncand, s);
+    int64_t hk[2];
+    {
+        const int64_t* src[2] = {kidx.p + ncand, maxrow.p + 2};
+        read_i64s(src, 2, hk, s);
+    }
+    const int64_t nform = hk[0];
+    // FP64 products of at least tc_min_flops may use the tensor cores (fp64tc.cu decides per block)
+    bool tc = !bf16 && nform && (double)(unsigned long long)hk[1] >= tc_min_flops;
+    if (tc && !groups) {
+        groups = build_groups(A);
+        A->groups = groups;
+    }
+    const int32_t* grp = (bf16 || tc) ? groups->g_of.p : nullptr;
+    // which twin of a mirrored pair is computed.  In X X with X exactly symmetric both are the same
+    // sums, and in the BF16 tier they differ by less than its rounding: those that fill a tile.  Else
+    // (X X2 in FP64: X2 is filtered, so the twins differ by the filter's truncation) it is the block
+    // I < J on any path, and tiles (G, G') and (G', G) are both formed, each with its half.
+    const int by_group = bf16 || (tc && A == B && A->exact_sym) ? 1 : 0;
 
     // 3. formed-block metadata
     const int64_t nf1 = std::max<int64_t>(nform, 1);
     DBuf<int32_t> f_row, f_col, f_ksum;
     DBuf<uint8_t> f_comp;                 // 1: the block is computed (0: copied from its twin or dropped)
     DBuf<int64_t> f_area, f_np, f_cin, f_off, f_pbeg, f_rp, flops, nprod_exec, shape_cnt, mirror;
+    DBuf<float> f_max;
+    if (tc) f_max.alloc(nf1, s);
     f_ksum.alloc(nf1, s);
     f_comp.alloc(nf1, s);
     mirror.alloc(nf1, s);
@@ -1163,14 +1250,15 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     flops.alloc(1, s);
     flops.zero();
     constexpr int kShapes = (kMaxBlock + 1) * (kMaxBlock + 1);     // histogram of formed blocks by (m, n)
-    shape_cnt.alloc(kShapes, s);
+    shape_cnt.alloc(2 * kShapes, s);
     shape_cnt.zero();
     if (ncand) {
         k_form_meta<<<grid_for(ncand, 256), 256, 0, s>>>(ncand, keep.p, kidx.p, cand_row.p, cand_col.p, pcnt.p, ksum.p,
                                                          use_c ? cin.p : nullptr, A->bs.p, f_row.p, f_col.p, f_area.p,
-                                                         f_np.p, f_cin.p, f_ksum.p);
+                                                         f_np.p, f_cin.p, f_ksum.p, max_term.p, f_max.p);
         DBG_LAUNCH_CK();
     }
+    std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> tcp(nullptr, f64tc_delete);
     k_form_rp<<<grid_for(nblk + 1, 256), 256, 0, s>>>(nblk, coff.p, kidx.p, f_rp.p);
     DBG_LAUNCH_CK();
     if (nform) {
@@ -1180,20 +1268,27 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         } else {
             DBG_CK(cudaMemsetAsync(mirror.p, 0xff, sizeof(int64_t) * nform, s));   // -1 (unused without sym)
         }
+        if (tc) {
+            // group tile patterns, digit tiles and the blocks the tensor cores take (f_comp = 2)
+            tcp = f64tc_prepare(A, B, groups, nform, f_rp.p,
+                                F64TcBlocks{f_row.p, f_col.p, mirror.p, f_ksum.p, f_max.p, f_comp.p, sym_result, by_group}, alpha, s);
+            tc = tcp != nullptr;
+        }
         k_form_stats<<<grid_for(nform, 256, (int64_t)num_sms() * 8), 256, 0, s>>>(nform, f_row.p, f_col.p, f_np.p, f_ksum.p, mirror.p,
                                                           sym_result, A->bs.p,
                                                           (unsigned long long*)flops.p,
                                                           (unsigned long long*)nprod_exec.p,
-                                                          (unsigned long long*)shape_cnt.p, f_comp.p, grp);
+                                                          (unsigned long long*)shape_cnt.p, f_comp.p, grp, by_group, tc ? 1 : 0,
+                                                          plan ? 1 : 0);
         DBG_LAUNCH_CK();
     }
     scan_exclusive(f_area.p, f_off.p, nform, s);
     scan_exclusive(f_np.p, f_pbeg.p, nform, s);
     int64_t h3[4];
-    std::vector<int64_t> shapes(kShapes);
+    std::vector<int64_t> shapes(2 * kShapes, 0);
     {
         const int64_t* src[4] = {f_off.p + nform, f_pbeg.p + nform, flops.p, nprod_exec.p};
-        DBG_CK(cudaMemcpyAsync(shapes.data(), shape_cnt.p, sizeof(int64_t) * kShapes, cudaMemcpyDeviceToHost, s));
+        DBG_CK(cudaMemcpyAsync(shapes.data(), shape_cnt.p, sizeof(int64_t) * 2 * kShapes, cudaMemcpyDeviceToHost, s));
         read_i64s(src, 4, h3, s);
     }
     const int64_t nel = h3[0], nprod = h3[1];
@@ -1208,7 +1303,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     const bool fill_smem = sm_fill <= (size_t)kSymSmemBudget;
     if (!fill_smem && !bf16) cursor.alloc(nf1, s);
     if (nprod && !bf16) {
-        FillArgs fa{coff.p, keep.p, f_comp.p, kidx.p, f_pbeg.p, cursor.p, prod_a.p, prod_b.p, fill_smem ? 1 : 0};
+        FillArgs fa{coff.p, keep.p, f_comp.p, plan ? 2 : 1, kidx.p, f_pbeg.p, cursor.p, prod_a.p, prod_b.p, fill_smem ? 1 : 0};
         const size_t sm = fill_smem ? sm_fill : sm_rank;
         allow_dyn_smem(k_fill_stack, sm);
         k_fill_stack<<<sym_grid(nblk), kSymThreads, sm, s>>>(nblk, P, nwords, fa);
@@ -1216,6 +1311,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     }
     // the candidate arrays are no longer needed
     cand_row.release(); cand_col.release(); pcnt.release(); ksum.release(); bound.release(); cursor.release();
+    max_term.release(); f_max.release();
     if (!nform) DBG_CK(cudaEventRecord(ev.e[1], s));
 
     // 5. numeric
@@ -1226,7 +1322,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     // kept by a plan: the shape lists, the tensor-core tier's patterns and the launch sequence
     DBuf<int64_t> list;
     SmmArgs sa{};
-    struct ShapeLaunch { int m, n; int64_t cnt; };
+    struct ShapeLaunch { int m, n; int64_t cnt; bool fallback; };
     std::vector<ShapeLaunch> launches;
     std::unique_ptr<LowTierPlan, void (*)(LowTierPlan*)> lt(nullptr, lowtier_plan_delete);
     LowTierOut lto{};
@@ -1246,25 +1342,32 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         }
         // with the one-launch schedule, the shapes the work queue takes come first in the list
         const bool queue = !bf16 && g_fp64_schedule.load() == 1;
-        int64_t at = 0, at_q = 0;
-        for (int pass = 0; pass < 2; ++pass)
+        int64_t at = 0, at_q = 0, n_tc = 0;
+        // passes 0 and 1: the blocks of the FP64 pipe; pass 2: those of the tensor cores, listed
+        // only for a plan (whose executions fall back to the FP64 pipe when new values need it)
+        for (int pass = 0; pass < 3; ++pass)
         for (int m = 1; m <= kMaxBlock; ++m)
             for (int n = 1; n <= kMaxBlock; ++n) {
-                const int64_t cnt = shapes[m * (kMaxBlock + 1) + n];
+                const int64_t cnt = shapes[(pass == 2 ? kShapes : 0) + m * (kMaxBlock + 1) + n];
                 if (!cnt) continue;
-                if ((queue && ((m * n + 31) >> 5) <= kQueueMaxE) != (pass == 0)) continue;
+                if (pass < 2 && (queue && ((m * n + 31) >> 5) <= kQueueMaxE) != (pass == 0)) continue;
                 bytes_min += 8.0 * (double)cnt * m * n;
-                if (bf16) continue;
-                k_shape_flags<<<grid_for(nform, 256), 256, 0, s>>>(nform, f_row.p, f_col.p, A->bs.p, mirror.p,
-                                                                   sym_result, m, n, flag.p);
+                if (pass == 2) n_tc += cnt;
+                if (bf16 || (pass == 2 && !plan)) continue;
+                k_shape_flags<<<grid_for(nform, 256), 256, 0, s>>>(nform, f_row.p, f_col.p, A->bs.p, f_comp.p,
+                                                                   pass == 2 ? 2 : 1, m, n, flag.p);
                 DBG_LAUNCH_CK();
                 scan_exclusive(flag.p, pos.p, nform, s);
                 k_class_scatter<<<grid_for(nform, 256), 256, 0, s>>>(nform, flag.p, pos.p, list.p + at);
                 DBG_LAUNCH_CK();
                 if (pass == 0) at_q += cnt;
-                launches.push_back({m, n, cnt});
+                launches.push_back({m, n, cnt, pass == 2});
                 at += cnt;
             }
+        if (tc && !n_tc) {
+            tcp.reset();
+            tc = false;
+        }
         if (bf16) {
             // the tensor-core tier on groups of blocks: group tile patterns and stacks, then the
             // operands packed (split) into tiles -- all counted with the symbolic phase
@@ -1283,7 +1386,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         }
         if (at_q > 0) {
             // the queue's shapes in one launch, replacing their per-shape entries
-            std::vector<ShapeLaunch> rest{{0, 0, at_q}};
+            std::vector<ShapeLaunch> rest{{0, 0, at_q, false}};
             int64_t q = 0;
             for (const ShapeLaunch& L : launches) {
                 if (q < at_q) q += L.cnt;
@@ -1294,15 +1397,24 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         }
         at = 0;
         for (const ShapeLaunch& L : launches) {
+            if (L.fallback) continue;
             if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, s);
             else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, sa, tune_lookup(prec, L.m, L.n, kmax), s);
             at += L.cnt;
+            if (!bf16) ++n_smm_launches;
         }
-        if (!bf16)         n_smm_launches = (int32_t)launches.size();
+        if (tc) {
+            lto = LowTierOut{f_rp.p, f_col.p, f_comp.p, f_off.p, use_c ? f_cin.p : nullptr,
+                             use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, alpha, beta,
+                             c_data.p, c_norm.p, c_dev2.p};
+            f64tc_run(*tcp, lto, s);
+            f64tc_norms(nform, f_comp.p, f_row.p, f_col.p, A->bs.p, f_off.p, c_data.p, c_norm.p, c_dev2.p, s);
+            ++n_smm_launches;
+        }
         if (sym_result) {
             DBG_CK(cudaEventRecord(ev.e[2], s));     // the copy / averaging is timed with the filter
             k_mirror_copy<<<grid_for(nform, 8), 256, 0, s>>>(nform, sym_result, mirror.p, f_row.p, f_col.p, f_off.p,
-                                                            A->bs.p, c_data.p, c_norm.p, c_dev2.p, grp);
+                                                            A->bs.p, c_data.p, c_norm.p, c_dev2.p, grp, by_group);
             DBG_LAUNCH_CK();
             if (sym_result == 2) {
                 k_sym_average<<<grid_for(nform, 8), 256, 0, s>>>(nform, mirror.p, f_row.p, f_col.p, f_off.p, A->bs.p,
@@ -1333,6 +1445,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     C->norms_valid = true;
     C->finalized = true;
     if (groups) C->groups = groups;
+    C->exact_sym = sym_result != kSymNone;
 
     if (plan) {
         // 6'. a plan keeps the formed pattern: blocks under eps are zeroed, not removed, so
@@ -1345,6 +1458,12 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             DBG_LAUNCH_CK();
         };
         zero_small(s);
+        DBuf<double> an, bn;                       // the operands' block norms at an execution
+        const F64TcBlocks f64tc_blocks{C->row.p, C->col.p, mirror.p, f_ksum.p, nullptr, f_comp.p, sym_result, by_group};
+        if (tc) {
+            an.alloc(std::max<int64_t>(A->nnzb, 1), s);
+            bn.alloc(std::max<int64_t>(B->nnzb, 1), s);
+        }
         // captured on a private stream (the legacy default stream cannot be captured); the
         // graph is launched on C's stream
         cudaStream_t cs = nullptr;
@@ -1357,10 +1476,20 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                 lowtier_pack(*lt, A, B, cs);
                 lowtier_run(*lt, A, lto, cs);
             }
+            SmmArgs fb = sa;
+            if (tc) {
+                // the tensor cores' blocks with the current values; the FP64 pipe repeats them all
+                // when these need it (f64tc_recheck)
+                f64tc_pack(*tcp, A, B, cs);
+                fb.gate = f64tc_recheck(*tcp, A, B, an.p, bn.p, nform, f64tc_blocks, f_pbeg.p, prod_a.p, prod_b.p, alpha, cs);
+                f64tc_run(*tcp, lto, cs);
+                f64tc_norms(nform, f_comp.p, C->row.p, C->col.p, C->bs.p, C->off.p, C->data.p, C->norms.p, c_dev2.p, cs);
+            }
             int64_t at = 0;
             for (const ShapeLaunch& L : launches) {
                 if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, cs);
-                else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, sa, tune_lookup(prec, L.m, L.n, kmax), cs);
+                else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, L.fallback ? fb : sa,
+                                      tune_lookup(prec, L.m, L.n, kmax), cs);
                 at += L.cnt;
             }
             zero_small(cs);
@@ -1395,7 +1524,10 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         plan->bufs_f64.push_back(std::move(c_dev2));
         plan->bufs_i64.push_back(std::move(qcounter));
         plan->bufs_u8.push_back(std::move(f_comp));
+        plan->bufs_f64.push_back(std::move(an));
+        plan->bufs_f64.push_back(std::move(bn));
         plan->lt = lt.release();
+        plan->tc = tcp.release();
         A->plans++;
         B->plans++;
         C->plans++;
@@ -1414,7 +1546,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             stats->n_launches = n_smm_launches;
             stats->flops_tensor = plan->lt ? lowtier_tensor_flops(*plan->lt) : 0.0;
             stats->bytes_tensor = plan->lt ? lowtier_copy_bytes(*plan->lt) : 0.0;
-            stats->n_tiles = plan->lt ? lowtier_tiles(*plan->lt) : 0;
+            stats->n_tiles = plan->lt ? lowtier_tiles(*plan->lt) : plan->tc ? f64tc_tiles(*plan->tc) : 0;
         }
         return;
     }
@@ -1434,6 +1566,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     compact(C, keep2.p, C->norms.p);
     DBG_CK(cudaEventRecord(ev.e[3], s));
     if (lt) lowtier_check(*lt, s);
+    if (tcp) f64tc_check(*tcp, s);
 
     if (stats) {
         DBG_CK(cudaStreamSynchronize(s));
@@ -1450,7 +1583,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         stats->n_launches = n_smm_launches;
         stats->flops_tensor = lt ? lowtier_tensor_flops(*lt) : 0.0;
         stats->bytes_tensor = lt ? lowtier_copy_bytes(*lt) : 0.0;
-        stats->n_tiles = lt ? lowtier_tiles(*lt) : 0;
+        stats->n_tiles = lt ? lowtier_tiles(*lt) : tcp ? f64tc_tiles(*tcp) : 0;
     }
 }
 
@@ -1471,6 +1604,7 @@ MultPlan::~MultPlan() {
         cudaGraphExecDestroy(exec);
     }
     if (lt) lowtier_plan_delete(lt);
+    if (tc) f64tc_delete(tc);
     if (A) A->plans--;
     if (B) B->plans--;
     if (C) C->plans--;
@@ -1506,7 +1640,7 @@ dbcsr_status dbcsr_multiply_plan(double alpha, dbcsr_matrix A, dbcsr_matrix B, d
     auto* p = new dbcsr_plan_();
     try {
         if (!A || !B) dbg::fail(DBCSR_EINVAL, "multiply_plan: null handle");
-        dbg::multiply(alpha, A, B, 0.0, C, eps_filter, prec, stats, false, dbg::kSymNone, &p->plan);
+        dbg::multiply(alpha, A, B, 0.0, C, eps_filter, prec, stats, false, dbg::kSymNone, &p->plan, dbg::kTcMinFlops);
         *out = p;
         dbg::set_last_error("");
         return DBCSR_OK;

@@ -295,6 +295,14 @@ dbcsr_status sign_iterate_resume(dbcsr_matrix_* H, dbcsr_matrix_* X0, const dbcs
     const auto t0 = std::chrono::steady_clock::now();
     auto X = make_like(H, H->stream);
     copy_matrix(X.get(), X0);
+    if (prev->alpha > 0 && std::isfinite(prev->alpha)) {
+        // the block groups of the tensor-core products are those of the run's first X (its couplings
+        // off the diagonal, which do not depend on mu), so that the products continue as the same sums
+        auto first = make_like(H, H->stream);
+        copy_matrix(first.get(), H);
+        scale_shift(first.get(), 1.0 / prev->alpha, 0.0);
+        X->groups = build_groups(first.get());
+    }
     const int it = prev->iterations;
     int first_fp64 = prev->fp64_from;
     if (S.o.prec == DBCSR_FP64) first_fp64 = std::max(1, first_fp64 ? first_fp64 : 1);

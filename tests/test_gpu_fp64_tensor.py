@@ -1,0 +1,172 @@
+"""FP64 products on the tensor cores (eight-digit splitting): at the edges of the tiles and slices,
+with badly scaled and non-finite operands, and in planned products whose values change.
+
+Every block is compared with a doubled-precision sum of the same terms within the bound that any summation of
+n rounded FP64 terms keeps, ||error|| <= n 2^-53 (sum_K ||A_IK|| ||B_KJ|| + |beta| ||C_IJ||), n the
+matrix dimension plus 4 (two scalings, a C input, the last rounding)."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import bsr
+
+pytestmark = pytest.mark.gpu
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def gb():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2003_03868_gb300 as m
+    m.lib()
+    return m
+
+
+def _product(a, b):
+    """a @ b in about twice FP64's precision (Dekker's products, Knuth's sums): (high, low)."""
+    def split(x):
+        c = 134217729.0 * x
+        h = c - (c - x)
+        return h, x - h
+    hi, lo = np.zeros((a.shape[0], b.shape[1])), np.zeros((a.shape[0], b.shape[1]))
+    (ah, al), (bh, bl) = split(a), split(b)
+    for k in range(a.shape[1]):
+        p = np.multiply.outer(a[:, k], b[k])
+        e = ((np.multiply.outer(ah[:, k], bh[k]) - p) + np.multiply.outer(ah[:, k], bl[k])
+             + np.multiply.outer(al[:, k], bh[k])) + np.multiply.outer(al[:, k], bl[k])
+        s = hi + p
+        z = s - hi
+        lo += ((hi - (s - z)) + (p - z)) + e
+        hi = s
+    return hi, lo
+
+
+def _norms(d, start):
+    """Frobenius norms of the blocks of d, each scaled by its largest element before squaring."""
+    n = np.maximum.reduceat(np.maximum.reduceat(np.abs(d), start[:-1], 0), start[:-1], 1)
+    q = np.where(n > 0, n, 1.0)
+    reps = np.diff(start)
+    big = np.repeat(np.repeat(q, reps, 0), reps, 1)
+    return np.where(n > 0, q * np.sqrt(np.add.reduceat(np.add.reduceat((d / big) ** 2, start[:-1], 0), start[:-1], 1)),
+                    0.0)
+
+
+def _check(C, Ao, Bo, alpha=1.0, beta=0.0, Co=None):
+    bs = np.asarray(Ao.bs)
+    start = np.concatenate([[0], np.cumsum(bs)])
+    a, b = bsr.to_dense(Ao), bsr.to_dense(Bo)
+    hi, lo = _product(a, b)
+    rp, col, data = C.export()
+    got = bsr.to_dense(bsr.Mat(bs, rp, col, data))
+    mag = abs(alpha) * (_norms(a, start) @ _norms(b, start))
+    # alpha and beta are short dyadic fractions: alpha * hi and beta * c round to FP64 at most
+    diff = (got - alpha * hi) - alpha * lo
+    if Co is not None:
+        c = bsr.to_dense(Co)
+        diff = ((got - beta * c) - alpha * hi) - alpha * lo
+        mag = mag + abs(beta) * _norms(c, start)
+    err = _norms(diff, start)
+    assert np.all(err <= (start[-1] + 4) * U * mag + 1e-300)
+
+
+# widths of the block groups (at most 112 rows, 16 blocks) and of the 32-column slices: full tiles
+# (16 x 7, 112 = 4 x 28), one row short or over, one block per tile, slices cut inside a block
+SIZES = [[7] * 64, [28] * 16, [31] * 15, [32] * 14, [23, 7, 7] * 12, [13, 5, 5] * 20, [1] * 90 + [32] * 10,
+         list(range(1, 33)), [17, 16, 15, 9, 8, 24] * 5]
+
+
+@pytest.mark.parametrize("si", range(len(SIZES)))
+@pytest.mark.parametrize("density", [0.45, 1.0])
+def test_products_at_tile_edges(gb, si, density):
+    bs = SIZES[si]
+    a = synth.random_block_matrix(bs, density, 1200 + si)
+    b = synth.random_block_matrix(bs, density, 1300 + si)
+    c = synth.random_block_matrix(bs, 0.3, 1400 + si)
+    A, B, C = (gb.Matrix.of(x) for x in (a, b, c))
+    st = gb.multiply(-0.75, A, B, 1.25, C, 0.0)
+    if st.flops >= 64e6 and density == 1.0 and min(bs) > 1:
+        assert st.n_tiles > 0
+    _check(C, bsr.Mat.of(a), bsr.Mat.of(b), -0.75, 1.25, bsr.Mat.of(c))
+
+
+def _scaled(m, f, seed):
+    """m with every block multiplied by 10 to a uniform power in [-f, f]."""
+    out = m.copy()
+    rng = np.random.default_rng(seed)
+    off, rows = out.blk_off(), out.rows()
+    for k in range(out.nnzb):
+        n = int(out.blk_size[rows[k]]) * int(out.blk_size[out.col[k]])
+        out.data[off[k]:off[k] + n] *= 10.0 ** rng.uniform(-f, f)
+    return out
+
+
+@pytest.mark.parametrize("f", [2.0, 8.0, 60.0, 150.0])
+def test_badly_scaled_blocks_keep_the_bound(gb, f):
+    bs = [13, 5, 5] * 20
+    a = _scaled(synth.random_block_matrix(bs, 0.9, 1500), f, 1)
+    b = _scaled(synth.random_block_matrix(bs, 0.9, 1501), f, 2)
+    A, B = gb.Matrix.of(a), gb.Matrix.of(b)
+    C = gb.Matrix(A.blk_size, A.stream)
+    gb.multiply(1.0, A, B, 0.0, C, 0.0)
+    _check(C, bsr.Mat.of(a), bsr.Mat.of(b))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, 1e200, 1e-200, 5e-324])
+def test_values_outside_the_scales(gb, bad):
+    bs = [23, 7, 7] * 10
+    a = synth.random_block_matrix(bs, 0.8, 1600)
+    if abs(bad) < 1:
+        a.data[a.blk_off()[0]:a.blk_off()[0] + 23 * 23] = bad        # a whole block
+    else:
+        a.data[1234] = bad
+    b = synth.random_block_matrix(bs, 0.8, 1601)
+    A, B = gb.Matrix.of(a), gb.Matrix.of(b)
+    C = gb.Matrix(A.blk_size, A.stream)
+    gb.multiply(1.0, A, B, 0.0, C, 0.0)
+    ref = bsr.multiply(1.0, bsr.Mat.of(a), bsr.Mat.of(b))
+    _, col, data = C.export()
+    assert np.array_equal(col, ref.col)
+    assert np.array_equal(np.isnan(data), np.isnan(ref.data))
+    assert np.array_equal(np.isinf(data), np.isinf(ref.data))
+    if np.isfinite(bad):
+        _check(C, bsr.Mat.of(a), bsr.Mat.of(b))
+
+
+def test_plan_with_values_that_need_the_fp64_units(gb):
+    bs = [13, 5, 5] * 20
+    a = synth.random_block_matrix(bs, 0.9, 1700)
+    A, B = gb.Matrix.of(a), gb.Matrix.of(a)
+    C = gb.Matrix(A.blk_size, A.stream)
+    plan = gb.Plan(1.0, A, B, C, 0.0)
+    assert plan.stats.n_tiles > 0
+    for values in (a.data * 3.0, _scaled(a, 8.0, 3).data, _scaled(a, 140.0, 4).data, a.data):
+        A.put_values(values)
+        plan.execute()
+        m = a.copy()
+        m.data = values
+        _check(C, bsr.Mat.of(m), bsr.Mat.of(a))
+    v = a.data.copy()
+    v[77] = np.nan
+    A.put_values(v)
+    plan.execute()
+    m = a.copy()
+    m.data = v
+    got = bsr.to_dense(bsr.Mat(C.blk_size, *C.export()))
+    # its row of the product, in the columns where B has a block
+    hit = np.isnan(bsr.to_dense(bsr.Mat.of(m))).astype(float)
+    there = bsr.to_dense(bsr.Mat(a.blk_size, a.row_ptr, a.col, np.ones_like(a.data)))
+    assert np.array_equal(np.isnan(got), hit @ there > 0)
+    plan.close()
+
+
+def test_symmetric_square_equals_its_transpose_and_the_bound(gb):
+    # A A of an exactly symmetric A: the mirrored products of the sign iteration, one step
+    h = synth.build_hamiltonian(synth.small(40, seed=1800))
+    X = gb.sign_iterate(gb.Matrix.of(h.H), 0.0, 0.0, 1e-13, max_iter=1, return_x=True).P
+    D = bsr.to_dense(bsr.Mat(X.blk_size, *X.export()))
+    assert np.array_equal(D, D.T)
+    C = gb.Matrix(X.blk_size, X.stream)
+    gb.multiply(1.0, X, X, 0.0, C, 0.0)
+    _check(C, bsr.Mat(X.blk_size, *X.export()), bsr.Mat(X.blk_size, *X.export()))

@@ -22,7 +22,7 @@
 // chunks of 128 x 8 BF16.  One CTA per SM runs a persistent loop over C tiles with
 // specialised warps: warp 0 streams the A and B steps of the tile's stack into a ring of
 // shared-memory stages with bulk copies, warp 1 issues the MMAs (M = 128, N = the column
-// group's width rounded up to 16, K = 16) into one of two TMEM accumulators, and warps 2-5
+// group's width rounded up to 16, K = 16) into one of four TMEM accumulators, and warps 2-9
 // read the finished accumulator back and write the atom blocks.  Every wait is bounded: a
 // wait that runs out sets an error flag and the kernel winds down.
 #include <algorithm>
@@ -534,74 +534,77 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                 if (!tc::mbar_wait(&S.full[stage], phase, kWaitLimit)) lt_fail(A, S);
             }
     } else if (warp == 1) {
-        // ---------------- MMA issuer (lane 0): the same runs as the producer, np MMAs per K step
-        // (hi*hi, then hi*lo and lo*hi for split operands); the warp fetches 32 entries' masks at once
+        // ---------------- MMA issuer (the whole warp, every lane with the same values, see
+        // tc::elect_one): the same runs as the producer, np MMAs per K step (hi*hi, then hi*lo and
+        // lo*hi for split operands); the warp fetches 32 entries' masks at once
+        // (behind `if (lane == 0)` the issue was the kernel's bound: H H of 512 waters with 23/7
+        // blocks 3.59 -> 2.78 ms, with 13/5 blocks 2.34 -> 1.75 ms, the same bits)
         int stage = 0;
         uint32_t phase = 0;
         int it = 0;
-        bool stop = false;
-        for (int64_t t = blockIdx.x; t < A.ntiles && !stop; t += gridDim.x, ++it) {
+        bool ok = true;
+        constexpr uint64_t dhi = ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);   // 8-row groups 128 bytes apart
+        const uint32_t s_base = tc::smem_u32(S.stage[0]) >> 4;
+        for (int64_t t = blockIdx.x; t < A.ntiles && ok; t += gridDim.x, ++it) {
             const int acc = it % kAccs;
             const uint32_t acc_phase = (uint32_t)(it / kAccs) & 1u;
             const int wc = A.g.g_w[A.c_tcol[t]];
-            const int ra = lt_rows(A.g.g_w[A.c_trow[t]]), rb = lt_rows(wc);
-            const int sa_bytes = np * 2 * ra * 16, sb_bytes = np * 2 * rb * 16;
-            const uint32_t idesc = tc::instr_desc(1, kTileRows, ((wc + 15) >> 4) << 4);
-            const uint32_t d_tmem = tmem + (uint32_t)(acc * 128);
-            if (lane == 0) {
-                if (!tc::mbar_wait(&S.acc_empty[acc], acc_phase ^ 1u, kWaitLimit)) lt_fail(A, S);
-                tc::fence_after_sync();
-            }
-            stop = __shfl_sync(0xffffffffu, lt_aborted(S), 0) != 0;
+            const uint32_t ra = tc::uniform((uint32_t)lt_rows(A.g.g_w[A.c_trow[t]])), rb = tc::uniform((uint32_t)lt_rows(wc));
+            // in 16-byte units: rows of a chunk; a K step is np x 2 chunks
+            const uint32_t sa_step = (uint32_t)np * 2u * ra, sb_step = (uint32_t)np * 2u * rb;
+            const uint32_t idesc = tc::uniform(tc::instr_desc(1, kTileRows, ((wc + 15) >> 4) << 4));
+            const uint32_t d_tmem = tc::uniform(tmem + (uint32_t)(acc * 128));
+            ok = tc::mbar_wait(&S.acc_empty[acc], acc_phase ^ 1u, kWaitLimit);
+            tc::fence_after_sync();
             uint32_t accumulate = 0;
             const int64_t e0 = A.s_ptr[t], e1 = A.s_ptr[t + 1];
-            for (int64_t eb0 = e0; eb0 < e1 && !stop; eb0 += 32) {
+            for (int64_t eb0 = e0; eb0 < e1 && ok; eb0 += 32) {
                 const int64_t my = eb0 + lane;
                 const unsigned mym = my < e1 ? (unsigned)(A.ea[my] & 255) : 0u;
-                const int cnt = (int)min((int64_t)32, e1 - eb0);
-                for (int x = 0; x < cnt && !stop; ++x) {
+                unsigned live = __ballot_sync(0xffffffffu, mym != 0u);
+                while (live && ok) {
+                    const int x = __ffs(live) - 1;
+                    live &= live - 1;
                     unsigned mask = __shfl_sync(0xffffffffu, mym, x);
-                    if (lane == 0) {
-                        while (mask) {
-                            int len;
-                            lt_next_run(mask, len);
-                            if (!tc::mbar_wait(&S.full[stage], phase, kWaitLimit)) {
-                                lt_fail(A, S);
-                                break;
-                            }
-                            tc::fence_after_sync();
-                            const uint32_t s0 = tc::smem_u32(S.stage[stage]);
-                            for (int j = 0; j < len; ++j) {
-                                const uint32_t sa = s0 + (uint32_t)(j * sa_bytes);
-                                const uint32_t sb = s0 + (uint32_t)(len * sa_bytes + j * sb_bytes);
-                                const uint64_t ah = tc::smem_desc(sa, ra * 16, 128);
-                                const uint64_t bh = tc::smem_desc(sb, rb * 16, 128);
-                                tc::mma_f16(d_tmem, ah, bh, idesc, accumulate);
-                                accumulate = 1;
+                    while (mask) {
+                        int len;
+                        lt_next_run(mask, len);
+                        ok = tc::mbar_wait(&S.full[stage], phase, kWaitLimit);
+                        if (!ok) break;
+                        tc::fence_after_sync();
+                        const uint32_t s0 = tc::uniform(s_base + (uint32_t)stage * (kStageBytesMax / 16));
+                        const uint32_t n = tc::uniform((uint32_t)len);
+                        if (tc::elect_one()) {
+                            for (uint32_t j = 0; j < n; ++j) {
+                                const uint32_t ah = (s0 + j * sa_step) | (ra << 16);
+                                const uint32_t bh = (s0 + n * sa_step + j * sb_step) | (rb << 16);
+                                tc::mma_f16(d_tmem, dhi | ah, dhi | bh, idesc, accumulate | j);
                                 if (np == 2) {
-                                    const uint64_t al = tc::smem_desc(sa + 2 * ra * 16, ra * 16, 128);
-                                    const uint64_t bl = tc::smem_desc(sb + 2 * rb * 16, rb * 16, 128);
-                                    tc::mma_f16(d_tmem, ah, bl, idesc, 1);
-                                    tc::mma_f16(d_tmem, al, bh, idesc, 1);
+                                    tc::mma_f16_acc<true>(d_tmem, dhi | ah, dhi | (bh + 2u * rb), idesc);
+                                    tc::mma_f16_acc<true>(d_tmem, dhi | (ah + 2u * ra), dhi | bh, idesc);
                                 }
                             }
                             tc::mma_commit(&S.empty[stage]);         // the stage is free once these MMAs ran
-                            if (++stage == kStages) {
-                                stage = 0;
-                                phase ^= 1u;
-                            }
+                        }
+                        __syncwarp();
+                        accumulate = 1;
+                        if (++stage == kStages) {
+                            stage = 0;
+                            phase ^= 1u;
                         }
                     }
-                    stop = __shfl_sync(0xffffffffu, lt_aborted(S), 0) != 0;
                 }
             }
-            if (lane == 0) tc::mma_commit(&S.acc_full[acc]);      // the accumulator is complete
+            ok = __all_sync(0xffffffffu, ok) && !__shfl_sync(0xffffffffu, lt_aborted(S), 0);
+            if (!ok && lane == 0) lt_fail(A, S);
+            if (tc::elect_one()) tc::mma_commit(&S.acc_full[acc]);    // the accumulator is complete
+            __syncwarp();
         }
-        // every MMA this thread issued has completed before the TMEM is released
-        if (lane == 0) {
-            tc::mma_commit(&S.fin);
-            if (!tc::mbar_wait(&S.fin, 0, kWaitLimit)) lt_fail(A, S);
-        }
+        // every MMA this warp issued has completed before the TMEM is released
+        if (tc::elect_one()) tc::mma_commit(&S.fin);
+        __syncwarp();
+        if (!tc::mbar_wait(&S.fin, 0, kWaitLimit) && lane == 0) lt_fail(A, S);
+        __syncwarp();
     } else if (warp == kLoaderWarp) {
         // ---------------- table loader: the tables of the epilogue's next tile, while it writes
         // the current one (every lane fetches 8 of the 256 member pairs, loads batched by level)

@@ -348,13 +348,22 @@ int64_t f64tc_tiles(const F64TcPlan& L);
 void f64tc_check(F64TcPlan& L, cudaStream_t s);
 
 // ---- dense.cu
-// C[b] = alpha A[b] B[b] + beta C[b] for nb row-major n x n matrices (b < 65536): FP64 on the
+// C[b] = alpha A[b] B[b] + beta Cin[b] (Cin may be C) for nb row-major n x n matrices (b < 65536): FP64 on the
 // FP64 pipe; FP32 storage on the TF32 tensor cores (split: three products of TF32 halves,
 // close to FP32 arithmetic).  C must not alias A or B.
-void dense_gemm_f64(int64_t nb, int n, double alpha, const double* A, const double* B, double beta, double* C,
-                    cudaStream_t s);
-void dense_gemm_tf32(int64_t nb, int n, float alpha, const float* A, const float* B, float beta, float* C, bool split,
-                     cudaStream_t s);
+void dense_gemm_f64(int64_t nb, int n, double alpha, const double* A, const double* B, double beta, const double* Cin,
+                    double* C, cudaStream_t s);
+// Workspace of the TF32 products of one caller on one stream, kept from product to product: B
+// transposed, A with padded rows (where needed), and the flag of a wait that ran out.
+struct DenseScratch {
+    DBuf<float> bt, a;
+    DBuf<int> err;
+    explicit DenseScratch(cudaStream_t s);
+    // Synchronises; fails with DBCSR_ETIMEOUT when a bounded wait of any product since then ran out.
+    void check(cudaStream_t s);
+};
+void dense_gemm_tf32(int64_t nb, int n, float alpha, const float* A, const float* B, float beta, const float* Cin,
+                     float* C, bool split, DenseScratch& w, cudaStream_t s);
 
 // ---- submatrix.cu
 dbcsr_status submatrix_sign(dbcsr_matrix_* H, double mu, const dbcsr_sign_opts* opts, dbcsr_matrix_* P,

@@ -5,11 +5,9 @@
 //   * FP32 storage on the 5th-generation tensor cores (tcgen05.mma kind::tf32, FP32
 //     accumulators in tensor memory).  Plain TF32 keeps 10 stored bits of each operand (the
 //     tensor cores drop the low 13); split TF32 (hi = x so truncated, lo = x - hi likewise,
-//     three products hi*hi + hi*lo + lo*hi) carries about 20 bits, close to FP32 arithmetic.  Operands are first packed into the K-major
-//     no-swizzle layout of tc05.cuh (B transposed), 128-row tiles of A and up-to-256-row tiles
-//     of B, K in steps of 8; one CTA per C tile streams K in stages of two steps with bulk
-//     copies, one thread issues the MMAs (M = 128, N = the B tile's rows, K = 8), and four
-//     warps write the accumulator back (one row each).
+//     three products hi*hi + hi*lo + lo*hi) carries about 20 bits, close to FP32 arithmetic.
+//     The operands come straight from the matrices through tensor maps (B transposed once;
+//     A through a copy with padded rows when its rows do not start on 16-byte boundaries).
 //   * FP64 storage on the FP64 pipe: 64 x 64 C tiles, 16-wide K slices in shared memory, a
 //     4 x 4 register tile per thread.  GB300's FP64 rate is low enough (about 3.5 flops per
 //     SM cycle) that the FMA loop, not memory, bounds it.
@@ -28,247 +26,82 @@ namespace {
 constexpr int kDM = 128;                 // M of the MMA and rows of an A tile
 constexpr int kDNMax = 256;              // rows of the widest B tile (N of the MMA)
 constexpr int kDStepK = 8;               // TF32 elements per MMA K step (32 bytes)
-constexpr int kDRunParts = 2;            // K steps x parts per stage: two steps plain, one step split
-constexpr int kDStages = 4;
-constexpr int kDStageBytes = kDRunParts * 2 * (kDM + kDNMax) * 16;   // 24 KB: two CTAs fit an SM
-constexpr int kDEpiCols = 64;            // accumulator columns staged per pass of the epilogue
-constexpr int kDThreads = 128;
+constexpr int kTK = 16;                  // K columns per stage (64-byte rows)
+constexpr int kTStageBytes = (kDM + kDNMax) * kTK * 4;  // 24 KB: A 8 KB, B up to 16 KB
+constexpr int kDEpiCols = 32;            // accumulator columns staged per pass of an epilogue warp
+constexpr int kDEpiWarps = 8;            // two per TMEM lane quadrant, every other pass each
+constexpr int kTConvWarps = 8;           // split operands: warps that write the low parts
 constexpr long long kDWaitLimit = 4000000000ll;
 
 // TF32 as the tensor cores read an FP32 operand: the 13 low mantissa bits dropped (truncation
-// toward zero).  Both paths store operands this way, so a stored value is what is multiplied.
+// toward zero).
 __device__ __forceinline__ float to_tf32(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
-
-// Packs a batch of n x n row-major matrices into tiles: tile (b, t) holds rows
-// [t R, t R + R) of M[b] (transpose = 0) or of M[b]^T (transpose = 1), all K = kpad columns,
-// as K steps of 8: per step np parts (hi, lo) x 2 chunks x R rows x 16 bytes.  Zero outside n.
-// A thread writes one 16-byte chunk row (4 consecutive K elements of one row), threads in the
-// order of the packed layout, so the writes are contiguous.
-__global__ void k_dense_pack(int64_t total, int n, int kpad, int R, int ntiles, int np, int transpose,
-                             const float* __restrict__ M, float* __restrict__ out) {
-    const int nsteps = kpad / kDStepK;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        // e enumerates (b, t, step, chunk, row r) with r fastest
-        const int r = (int)(e % R);
-        int64_t rest = e / R;
-        const int ch = (int)(rest % 2);
-        rest /= 2;
-        const int st = (int)(rest % nsteps);
-        rest /= nsteps;
-        const int t = (int)(rest % ntiles);
-        const int64_t b = rest / ntiles;
-        const int row = t * R + r, c0 = st * kDStepK + ch * 4;
-        float x[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = c0 + q;
-            x[q] = (row < n && c < n) ? (transpose ? M[b * n * n + (int64_t)c * n + row] : M[b * n * n + (int64_t)row * n + c])
-                                      : 0.f;
-        }
-        const int64_t step_bytes = (int64_t)np * 2 * R * 16;
-        uint8_t* base = reinterpret_cast<uint8_t*>(out) + ((b * ntiles + t) * nsteps + st) * step_bytes + ch * (R * 16) +
-                        r * 16;
-        float4 hi = make_float4(to_tf32(x[0]), to_tf32(x[1]), to_tf32(x[2]), to_tf32(x[3]));
-        *reinterpret_cast<float4*>(base) = hi;
-        if (np == 2)
-            *reinterpret_cast<float4*>(base + 2 * R * 16) =
-                make_float4(to_tf32(x[0] - hi.x), to_tf32(x[1] - hi.y), to_tf32(x[2] - hi.z), to_tf32(x[3] - hi.w));
-    }
-}
-
-struct DenseArgs {
-    int n, kpad, ntm, ntn, NT, np;       // NT: rows of every B tile (N of the MMA)
-    const uint8_t* a_pack; const uint8_t* b_pack;
-    float alpha, beta;
-    float* C;
-    int* err;
-};
-
-struct DenseShared {
-    alignas(1024) uint8_t stage[kDStages][kDStageBytes];   // after the K loop: the epilogue's staging
-    uint64_t full[kDStages], empty[kDStages], done;
-    uint32_t tmem_base;
-};
-
-__global__ void __launch_bounds__(kDThreads, 2) k_dense_tf32(DenseArgs D) {
-    extern __shared__ __align__(1024) uint8_t d_dyn[];
-    DenseShared& S = *reinterpret_cast<DenseShared*>((reinterpret_cast<uintptr_t>(d_dyn) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tm = blockIdx.x, tn = blockIdx.y;
-    const int64_t b = blockIdx.z;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kDStages; ++i) {
-            tc::mbar_init(&S.full[i], 1);
-            tc::mbar_init(&S.empty[i], 1);
-        }
-        tc::mbar_init(&S.done, 1);
-        tc::fence_barrier_init();
-    }
-    if (warp == 0) {
-        tc::tmem_alloc(&S.tmem_base, kDNMax);
-        tc::tmem_relinquish();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = S.tmem_base;
-    const int np = D.np, NT = D.NT;
-    const int64_t sa_step = (int64_t)np * 2 * kDM * 16, sb_step = (int64_t)np * 2 * NT * 16;
-    const int nk = D.kpad / kDStepK;
-    const int run = kDRunParts / np;                      // K steps per stage
-    const int nstage = (nk + run - 1) / run;
-    const uint8_t* pa = D.a_pack + (b * D.ntm + tm) * (int64_t)nk * sa_step;
-    const uint8_t* pb = D.b_pack + (b * D.ntn + tn) * (int64_t)nk * sb_step;
-    bool ok = true;
-    if (threadIdx.x == 0) {
-        // one thread streams the K stages and issues the MMAs; a stage is refilled once the
-        // MMAs that read it have completed
-        int issued = 0;
-        auto issue = [&](int s) {
-            const int slot = s % kDStages;
-            issued = s + 1;
-            const int k0 = s * run, len = min(run, nk - k0);
-            tc::mbar_arrive_expect_tx(&S.full[slot], (uint32_t)(len * (sa_step + sb_step)));
-            tc::bulk_g2s(S.stage[slot], pa + k0 * sa_step, (uint32_t)(len * sa_step), &S.full[slot]);
-            tc::bulk_g2s(S.stage[slot] + len * sa_step, pb + k0 * sb_step, (uint32_t)(len * sb_step), &S.full[slot]);
-        };
-        for (int s = 0; s < min(kDStages, nstage); ++s) issue(s);
-        const uint32_t idesc = tc::instr_desc(2, kDM, NT);
-        uint32_t accumulate = 0;
-        for (int s = 0; s < nstage && ok; ++s) {
-            const int slot = s % kDStages;
-            const uint32_t phase = (uint32_t)(s / kDStages) & 1u;
-            if (!tc::mbar_wait(&S.full[slot], phase, kDWaitLimit)) {
-                ok = false;
-                break;
-            }
-            tc::fence_after_sync();
-            const int len = min(run, nk - s * run);
-            const uint32_t s0 = tc::smem_u32(S.stage[slot]);
-            for (int j = 0; j < len; ++j) {
-                const uint32_t sa = s0 + (uint32_t)(j * sa_step), sb = s0 + (uint32_t)(len * sa_step + j * sb_step);
-                const uint64_t ah = tc::smem_desc(sa, kDM * 16, 128), bh = tc::smem_desc(sb, NT * 16, 128);
-                tc::mma_tf32(tmem, ah, bh, idesc, accumulate);
-                accumulate = 1;
-                if (np == 2) {
-                    const uint64_t al = tc::smem_desc(sa + 2 * kDM * 16, kDM * 16, 128);
-                    const uint64_t bl = tc::smem_desc(sb + 2 * NT * 16, NT * 16, 128);
-                    tc::mma_tf32(tmem, ah, bl, idesc, 1);
-                    tc::mma_tf32(tmem, al, bh, idesc, 1);
-                }
-            }
-            tc::mma_commit(&S.empty[slot]);
-            // refill the previous stage's slot: its MMAs ran before these, which keep the tensor
-            // cores busy while this thread waits
-            const int pr = s - 1;
-            if (pr >= 0 && pr + kDStages < nstage) {
-                const int pslot = pr % kDStages;
-                if (!tc::mbar_wait(&S.empty[pslot], (uint32_t)(pr / kDStages) & 1u, kDWaitLimit)) {
-                    ok = false;
-                    break;
-                }
-                issue(pr + kDStages);
-            }
-        }
-        tc::mma_commit(&S.done);
-        if (!tc::mbar_wait(&S.done, 0, kDWaitLimit)) ok = false;
-        // copies still landing (after a wait that ran out) are waited for, bounded, before exit
-        for (int s = max(0, issued - kDStages); s < issued; ++s) {
-            const int slot = s % kDStages;
-            tc::mbar_wait(&S.full[slot], (uint32_t)(s / kDStages) & 1u, kDWaitLimit);
-        }
-        if (!ok) atomicExch(D.err, 1);
-    }
-    __syncthreads();
-    tc::fence_after_sync();
-    // epilogue, kDEpiCols columns per pass: thread r reads row r of the accumulator (TMEM lane
-    // r) into shared memory (the stage ring is idle now: every copy landed and every MMA
-    // completed), then each warp writes whole row segments, lanes over consecutive columns
-    float* T = reinterpret_cast<float*>(S.stage[0]);
-    constexpr int kTS = kDEpiCols + 1;                    // odd stride: no bank conflicts
-    float* Cb = D.C + b * D.n * D.n;
-    const int r0 = tm * kDM;
-    for (int c0 = 0; c0 < NT; c0 += kDEpiCols) {
-        const int cw = min(kDEpiCols, NT - c0);
-        for (int c = 0; c < cw; c += 16) {
-            float v[16];
-            tc::tmem_ld16(tmem + (uint32_t)(c0 + c) + ((uint32_t)(32 * warp) << 16), v);
-#pragma unroll
-            for (int x = 0; x < 16; ++x) T[threadIdx.x * kTS + c + x] = v[x];
-        }
-        __syncthreads();
-        const int col0 = tn * NT + c0;
-        const int ncol = min(cw, D.n - col0);
-        for (int r = warp; r < kDM; r += kDThreads / 32) {
-            const int row = r0 + r;
-            if (row >= D.n) break;
-            float* out = Cb + (int64_t)row * D.n + col0;
-            for (int c = lane; c < ncol; c += 32) {
-                const float v = D.alpha * T[r * kTS + c];
-                out[c] = D.beta == 0.f ? v : v + D.beta * out[c];
-            }
-        }
-        __syncthreads();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) {
-        tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kDNMax);
-    }
-}
-
-// ---------------------------------------------------------------- TF32 from tensor-map loads
-// For n a multiple of 4 the operands need no pack pass: a 3-D tensor map (columns, rows,
-// matrix) over A and one over B^T (B transposed once per product) bring 16 K columns of a
-// 128-row A tile and of an N-row B tile per stage straight from the FP32 matrices, in the
-// 64-byte swizzled K-major layout, and the MMAs read them as they are (as TF32).  For split
-// operands four converter warps write lo = x - tf32(x) of every stage into a second buffer;
-// one thread issues the MMAs (two K = 8 steps per stage); the four warps then write the
-// accumulator back.
-constexpr int kTK = 16;                                  // K columns per stage (64-byte rows)
-constexpr int kTStages = 4;
-constexpr int kTStageBytes = (kDM + kDNMax) * kTK * 4;  // 24 KB: A 8 KB, B up to 16 KB
-constexpr int kTThreads = 192;                           // producer, MMA, 4 converter / epilogue warps
 
 template <bool SPLIT>
 struct TmaShared {
-    alignas(1024) uint8_t x[kTStages][kTStageBytes];
-    alignas(1024) uint8_t lo[SPLIT ? kTStages : 1][SPLIT ? kTStageBytes : 16];
-    uint64_t full[kTStages], conv[kTStages], empty[kTStages], done;
+    static constexpr int kStages = SPLIT ? 4 : 7;
+    alignas(1024) uint8_t x[kStages][kTStageBytes];
+    alignas(1024) uint8_t lo[SPLIT ? kStages : 1][SPLIT ? kTStageBytes : 16];
+    float out[kDEpiWarps][32][kDEpiCols + 1];   // odd stride: no bank conflicts
+    uint64_t full[kStages], conv[kStages], empty[kStages], acc_full[2], acc_empty[2], fin;
     uint32_t tmem_base;
     int abort;
 };
 
 struct TmaArgs {
-    int n, ntm, ntn, NT;
+    int n, ntm, ntn, NT;                 // NT: rows of every B tile (N of the MMA)
+    int64_t ntiles;
     float alpha, beta;
+    const float* Cin;                    // beta's C (may be C)
     float* C;
     int* err;
 };
 
+// One persistent CTA per SM over the 128 x NT tiles of C, the row tiles of a matrix next to each other
+// so that the CTAs running at one time share its B tiles in L2.  Warp 0 streams 16 K columns per
+// stage of the A and B^T tiles into a ring (3-D tensor maps, 64-byte swizzled K-major rows, read by the
+// MMAs as they are: as TF32); for split operands eight converter warps write lo = x - tf32(x) of every
+// stage, four of them every other stage (the write, the proxy fence and the arrival take a stage's
+// time, so two stages are converted at once); warp 1 issues the MMAs (two K = 8 steps per stage,
+// three MMAs each when split) into one of two TMEM accumulators, and eight warps write the other one
+// back meanwhile, 32 rows and 32 columns at a time.
+// On 400 matrices of 400 x 400 the earlier kernel (one CTA per tile, four converter warps that also
+// wrote the result back, MMAs issued behind lane 0) took 0.63 ms split and 0.27 ms plain with the
+// tensor cores 28% and 22% busy: loads, products and the write-back followed one another in a CTA.
+// Now 0.33 ms (55% busy; the low parts' writes bound it) and 0.17 ms (bytes: 0.11 ms at copy rate).
 template <bool SPLIT>
-__global__ void __launch_bounds__(kTThreads, 1)
-    k_dense_tf32_tma(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_bt, TmaArgs D) {
+__global__ void __launch_bounds__(32 * (2 + (SPLIT ? kTConvWarps : 0) + kDEpiWarps), 1)
+    k_dense_tf32(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_bt, TmaArgs D) {
     extern __shared__ __align__(1024) uint8_t t_dyn[];
-    auto& S = *reinterpret_cast<TmaShared<SPLIT>*>((reinterpret_cast<uintptr_t>(t_dyn) + 1023) & ~(uintptr_t)1023);
+    using Sh = TmaShared<SPLIT>;
+    constexpr int ST = Sh::kStages;
+    auto& S = *reinterpret_cast<Sh*>((reinterpret_cast<uintptr_t>(t_dyn) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tm = blockIdx.x, tn = blockIdx.y, b = blockIdx.z;
+    constexpr int epi0 = SPLIT ? 2 + kTConvWarps : 2;
     const int NT = D.NT;
     const int a_bytes = kDM * kTK * 4, b_bytes = NT * kTK * 4;
     const int nstage = (D.n + kTK - 1) / kTK;
+    auto failed = [&] {
+        *(volatile int*)&S.abort = 1;
+        atomicExch(D.err, 1);
+    };
+    auto aborted = [&] { return *(volatile const int*)&S.abort != 0; };
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kTStages; ++i) {
+        for (int i = 0; i < ST; ++i) {
             tc::mbar_init(&S.full[i], 1);
-            tc::mbar_init(&S.conv[i], 128);
+            tc::mbar_init(&S.conv[i], kTConvWarps / 2);
             tc::mbar_init(&S.empty[i], 1);
         }
-        tc::mbar_init(&S.done, 1);
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&S.acc_full[i], 1);
+            tc::mbar_init(&S.acc_empty[i], kDEpiWarps);
+        }
+        tc::mbar_init(&S.fin, 1);
         S.abort = 0;
         tc::fence_barrier_init();
     }
     if (warp == 1) {
-        tc::tmem_alloc(&S.tmem_base, kDNMax);
+        tc::tmem_alloc(&S.tmem_base, 2 * kDNMax);
         tc::tmem_relinquish();
     }
     tc::fence_before_sync();
@@ -278,149 +111,235 @@ __global__ void __launch_bounds__(kTThreads, 1)
     if (warp == 0) {
         // ---- producer (lane 0): a stage is refilled once the MMAs that read it completed
         if (lane == 0) {
-            int issued = 0;
-            for (int s = 0; s < nstage; ++s) {
-                const int slot = s % kTStages;
-                if (s >= kTStages &&
-                    !tc::mbar_wait(&S.empty[slot], (uint32_t)((s / kTStages) - 1) & 1u, kDWaitLimit)) {
-                    *(volatile int*)&S.abort = 1;
-                    atomicExch(D.err, 1);
-                    break;
-                }
-                if (*(volatile int*)&S.abort) break;
-                tc::mbar_arrive_expect_tx(&S.full[slot], (uint32_t)(a_bytes + b_bytes));
-                tc::tma_load3d(S.x[slot], &map_a, s * kTK, tm * kDM, b, &S.full[slot]);
-                tc::tma_load3d(S.x[slot] + a_bytes, &map_bt, s * kTK, tn * NT, b, &S.full[slot]);
-                issued = s + 1;
-            }
-            // no copy may still be landing when the CTA exits
-            for (int s = max(0, issued - kTStages); s < issued; ++s)
-                tc::mbar_wait(&S.full[s % kTStages], (uint32_t)(s / kTStages) & 1u, kDWaitLimit);
-        }
-    } else if (warp == 1) {
-        // ---- MMA issuer (lane 0)
-        if (lane == 0) {
-            const uint32_t idesc = tc::instr_desc(2, kDM, NT);
+            int slot = 0;
+            uint32_t phase = 0;
+            int64_t issued = 0;
             bool ok = true;
-            for (int s = 0; s < nstage && ok; ++s) {
-                const int slot = s % kTStages;
-                const uint32_t ph = (uint32_t)(s / kTStages) & 1u;
-                if (!tc::mbar_wait(SPLIT ? &S.conv[slot] : &S.full[slot], ph, kDWaitLimit) || *(volatile int*)&S.abort) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t xa = tc::smem_u32(S.x[slot]), xb = xa + (uint32_t)a_bytes;
-#pragma unroll
-                for (int j = 0; j < kTK / kDStepK; ++j) {
-                    const uint32_t ko = (uint32_t)(j * kDStepK * 4);     // 32 bytes per K = 8 step
-                    const uint64_t ah = tc::smem_desc_sw64(xa + ko), bh = tc::smem_desc_sw64(xb + ko);
-                    tc::mma_tf32(tmem, ah, bh, idesc, (s | j) ? 1u : 0u);
-                    if (SPLIT) {
-                        const uint32_t la = tc::smem_u32(S.lo[slot]), lb = la + (uint32_t)a_bytes;
-                        tc::mma_tf32(tmem, ah, tc::smem_desc_sw64(lb + ko), idesc, 1);
-                        tc::mma_tf32(tmem, tc::smem_desc_sw64(la + ko), bh, idesc, 1);
+            for (int64_t tile = blockIdx.x; tile < D.ntiles && ok; tile += gridDim.x) {
+                const int64_t rest = tile / D.ntm;
+                const int tm = (int)(tile - rest * D.ntm), b = (int)(rest / D.ntn), tn = (int)(rest - (int64_t)b * D.ntn);
+                for (int s = 0; s < nstage; ++s) {
+                    if (!tc::mbar_wait(&S.empty[slot], phase ^ 1u, kDWaitLimit)) failed();
+                    if (aborted()) {
+                        ok = false;
+                        break;
+                    }
+                    tc::mbar_arrive_expect_tx(&S.full[slot], (uint32_t)(a_bytes + b_bytes));
+                    tc::tma_load3d(S.x[slot], &map_a, s * kTK, tm * kDM, b, &S.full[slot]);
+                    tc::tma_load3d(S.x[slot] + a_bytes, &map_bt, s * kTK, tn * NT, b, &S.full[slot]);
+                    ++issued;
+                    if (++slot == ST) {
+                        slot = 0;
+                        phase ^= 1u;
                     }
                 }
-                tc::mma_commit(&S.empty[slot]);
             }
-            if (!ok) {
-                *(volatile int*)&S.abort = 1;
-                atomicExch(D.err, 1);
-            }
-            tc::mma_commit(&S.done);
-        }
-    } else {
-        // ---- converters (warps 2-5, split operands): lo = x - tf32(x) of every stage
-        const int ct = threadIdx.x - 64;
-        for (int s = 0; SPLIT && s < nstage; ++s) {
-            const int slot = s % kTStages;
-            const uint32_t ph = (uint32_t)(s / kTStages) & 1u;
-            const bool ok = tc::mbar_wait(&S.full[slot], ph, kDWaitLimit) && !*(volatile int*)&S.abort;
-            if (ok) {
-                const float4* xs = reinterpret_cast<const float4*>(S.x[slot]);
-                float4* ls = reinterpret_cast<float4*>(S.lo[slot]);
-                const int n4 = (a_bytes + b_bytes) / 16;
-                for (int i = ct; i < n4; i += 128) {
-                    const float4 v = xs[i];
-                    ls[i] = make_float4(v.x - to_tf32(v.x), v.y - to_tf32(v.y), v.z - to_tf32(v.z), v.w - to_tf32(v.w));
+            // no copy may still be landing when the CTA exits
+            for (int64_t x = 0; x < issued && x < ST; ++x) {
+                if (--slot < 0) {
+                    slot = ST - 1;
+                    phase ^= 1u;
                 }
-            } else if (ct == 0) {
-                *(volatile int*)&S.abort = 1;
-                atomicExch(D.err, 1);
+                if (!tc::mbar_wait(&S.full[slot], phase, kDWaitLimit)) failed();
             }
-            tc::fence_proxy_async();                          // the tensor cores read what was written
-            tc::mbar_arrive(&S.conv[slot]);
-            if (!ok) break;
         }
-    }
-    // ---- epilogue (warps 2-5): TMEM lane quadrant warp % 4 holds rows 32 (warp % 4) ..
-    const bool epi = warp >= 2;
-    bool fin = true;
-    if (threadIdx.x == 64) fin = tc::mbar_wait(&S.done, 0, kDWaitLimit);
-    if (threadIdx.x == 64 && !fin) atomicExch(D.err, 1);
-    __syncthreads();                                         // also: every stage is idle now
-    tc::fence_after_sync();
-    float* T = reinterpret_cast<float*>(S.x[0]);
-    constexpr int kTS = kDEpiCols + 1;
-    float* Cb = D.C + (int64_t)b * D.n * D.n;
-    const int q = warp & 3, et = threadIdx.x - 64;
-    for (int c0 = 0; c0 < NT; c0 += kDEpiCols) {
-        const int cw = min(kDEpiCols, NT - c0);
-        if (epi) {
-            for (int c = 0; c < cw; c += 16) {
-                float v[16];
-                tc::tmem_ld16(tmem + (uint32_t)(c0 + c) + ((uint32_t)(32 * q) << 16), v);
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---- MMA issuer (the whole warp, every lane with the same values)
+        const uint32_t idesc = tc::uniform(tc::instr_desc(2, kDM, NT));
+        const uint64_t hi = tc::smem_desc_sw64(0);    // all but the start address
+        const uint32_t x0 = tc::smem_u32(S.x[0]) >> 4, l0 = SPLIT ? tc::smem_u32(S.lo[0]) >> 4 : 0;
+        int slot = 0;
+        uint32_t phase = 0, k = 0;
+        bool ok = true;
+        for (int64_t tile = blockIdx.x; tile < D.ntiles && ok; tile += gridDim.x, ++k) {
+            const uint32_t buf = k & 1u;
+            const uint32_t d = tc::uniform(tmem + buf * kDNMax);
+            ok = tc::mbar_wait(&S.acc_empty[buf], ((k >> 1) & 1u) ^ 1u, kDWaitLimit);
+            uint32_t acc = 0;
+            for (int s = 0; s < nstage && ok; ++s) {
+                ok = tc::mbar_wait(SPLIT ? &S.conv[slot] : &S.full[slot], phase, kDWaitLimit) && !aborted();
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint32_t xa = tc::uniform(x0 + (uint32_t)slot * (kTStageBytes / 16));
+                const uint32_t la = SPLIT ? tc::uniform(l0 + (uint32_t)slot * (kTStageBytes / 16)) : 0;
+                constexpr uint32_t ab = kDM * kTK * 4 / 16;
+                if (tc::elect_one()) {
 #pragma unroll
-                for (int x = 0; x < 16; ++x) T[(32 * q + lane) * kTS + c + x] = v[x];
-            }
-        }
-        __syncthreads();
-        if (epi) {
-            const int col0 = tn * NT + c0;
-            const int ncol = min(cw, D.n - col0);
-            for (int r = et >> 5; r < kDM; r += 4) {
-                const int row = tm * kDM + r;
-                if (row >= D.n) break;
-                float* out = Cb + (int64_t)row * D.n + col0;
-                for (int c = lane; c < ncol; c += 32) {
-                    const float v = D.alpha * T[r * kTS + c];
-                    out[c] = D.beta == 0.f ? v : v + D.beta * out[c];
+                    for (uint32_t j = 0; j < kTK / kDStepK; ++j) {
+                        const uint32_t ko = j * (kDStepK * 4 / 16);          // 32 bytes per K = 8 step
+                        tc::mma_tf32(d, hi | (xa + ko), hi | (xa + ab + ko), idesc, j ? 1u : acc);
+                        if (SPLIT) {
+                            tc::mma_tf32(d, hi | (xa + ko), hi | (la + ab + ko), idesc, 1);
+                            tc::mma_tf32(d, hi | (la + ko), hi | (xa + ab + ko), idesc, 1);
+                        }
+                    }
+                    tc::mma_commit(&S.empty[slot]);
+                    if (s == nstage - 1) tc::mma_commit(&S.acc_full[buf]);
+                }
+                __syncwarp();
+                acc = 1;
+                if (++slot == ST) {
+                    slot = 0;
+                    phase ^= 1u;
                 }
             }
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok && lane == 0) failed();
         }
-        __syncthreads();
+        // every MMA has completed before the TMEM is released
+        if (tc::elect_one()) tc::mma_commit(&S.fin);
+        __syncwarp();
+        if (!tc::mbar_wait(&S.fin, 0, kDWaitLimit) && lane == 0) failed();
+        __syncwarp();
+    } else if (SPLIT && warp < epi0) {
+        // ---- converters (split operands): lo = x - tf32(x) of every other stage
+        constexpr int kConvThreads = 16 * kTConvWarps, kBatch = 6;
+        const int ct = (threadIdx.x - 64) % kConvThreads, group = (threadIdx.x - 64) / kConvThreads;
+        const int n4 = (a_bytes + b_bytes) / 16;
+        int slot = 0, turn = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int64_t tile = blockIdx.x; tile < D.ntiles && ok; tile += gridDim.x)
+            for (int s = 0; s < nstage && ok; ++s, turn ^= 1) {
+                if (turn == group) {
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(&S.full[slot], phase, kDWaitLimit) && !aborted());
+                    if (!ok) {
+                        if (lane == 0) failed();
+                        break;
+                    }
+                    const float4* xs = reinterpret_cast<const float4*>(S.x[slot]);
+                    float4* ls = reinterpret_cast<float4*>(S.lo[SPLIT ? slot : 0]);
+                    for (int i0 = ct; i0 < n4; i0 += kBatch * kConvThreads) {
+                        float4 v[kBatch];
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u)
+                            if (i0 + u * kConvThreads < n4) v[u] = xs[i0 + u * kConvThreads];
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u)
+                            if (i0 + u * kConvThreads < n4)
+                                ls[i0 + u * kConvThreads] =
+                                    make_float4(v[u].x - to_tf32(v[u].x), v[u].y - to_tf32(v[u].y),
+                                                v[u].z - to_tf32(v[u].z), v[u].w - to_tf32(v[u].w));
+                    }
+                    tc::fence_proxy_async();              // the tensor cores read what was written
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&S.conv[slot]);
+                }
+                if (++slot == ST) {
+                    slot = 0;
+                    phase ^= 1u;
+                }
+            }
+    } else {
+        // ---- epilogue: TMEM lane quadrant warp % 4 holds rows 32 (warp % 4) ..; kDEpiCols columns per
+        // pass through this warp's staging, then whole row segments, eight rows in flight
+        const int q = warp & 3, ew = warp - epi0, half = ew >> 2;
+        uint32_t k = 0;
+        for (int64_t tile = blockIdx.x; tile < D.ntiles; tile += gridDim.x, ++k) {
+            const int64_t rest = tile / D.ntm;
+            const int tm = (int)(tile - rest * D.ntm), tn = (int)(rest % D.ntn);
+            const int64_t b = rest / D.ntn;
+            const uint32_t buf = k & 1u;
+            const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&S.acc_full[buf], (k >> 1) & 1u, kDWaitLimit) &&
+                                                        !aborted());
+            if (!ok) {
+                if (lane == 0) failed();
+                break;
+            }
+            tc::fence_after_sync();
+            float* Cb = D.C + b * D.n * D.n;
+            const float* Ib = D.Cin + b * D.n * D.n;
+            const int r0 = tm * kDM + 32 * q;
+            const int rows = min(32, D.n - r0);
+            for (int c0 = kDEpiCols * half; c0 < NT; c0 += 2 * kDEpiCols) {
+                const int cw = min(kDEpiCols, NT - c0);
+                __syncwarp();                             // the last pass's rows are written
+                for (int c = 0; c < cw; c += 16) {
+                    float v[16];
+                    tc::tmem_ld16(tmem + buf * kDNMax + (uint32_t)(c0 + c) + ((uint32_t)(32 * q) << 16), v);
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) S.out[ew][lane][c + x] = v[x];
+                }
+                if (c0 + 2 * kDEpiCols >= NT) {           // this warp's part of the accumulator is read
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&S.acc_empty[buf]);
+                }
+                __syncwarp();
+                const int col = tn * NT + c0 + lane;
+                if (lane < cw && col < D.n) {
+                    const int64_t o = (int64_t)r0 * D.n + col;
+                    for (int rb = 0; rb < rows; rb += 8) {
+                        float v[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) v[u] = D.alpha * S.out[ew][rb + u][lane];
+                        if (D.beta != 0.f) {
+                            float ci[8];
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) ci[u] = rb + u < rows ? Ib[o + (int64_t)(rb + u) * D.n] : 0.f;
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) v[u] = v[u] + D.beta * ci[u];
+                        }
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (rb + u < rows) Cb[o + (int64_t)(rb + u) * D.n] = v[u];
+                    }
+                }
+            }
+            if (kDEpiCols * half >= NT) {                 // (a narrow tile leaves this warp no pass)
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&S.acc_empty[buf]);
+            }
+        }
     }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kDNMax);
+        tc::tmem_dealloc(tmem, 2 * kDNMax);
     }
 }
 
-// B^T of every matrix of a batch (32 x 32 tiles through shared memory).
-__global__ void k_dense_transpose(int64_t nb, int n, const float* __restrict__ B, float* __restrict__ Bt) {
-    __shared__ float t[32][33];
-    const int tiles = (n + 31) / 32;
+// A batch of n x n matrices with rows of ld floats (a multiple of 4, so that tensor maps can read
+// them): transposed (64 x 64 tiles through shared memory, 16 loads in flight per thread) or copied.
+__global__ void __launch_bounds__(256) k_dense_transpose(int64_t nb, int n, int ld, const float* __restrict__ B,
+                                                         float* __restrict__ Bt) {
+    __shared__ float t[64][65];
+    const int tiles = (n + 63) / 64, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     const int64_t total = nb * tiles * tiles;
     for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
         const int64_t m = w / ((int64_t)tiles * tiles);
         const int rest = (int)(w - m * tiles * tiles);
         const int ti = rest / tiles, tj = rest - ti * tiles;
         const float* src = B + m * n * n;
-        float* dst = Bt + m * n * n;
-        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-            const int i = ti * 32 + r, j = tj * 32 + threadIdx.x;
-            t[r][threadIdx.x] = (i < n && j < n) ? src[(int64_t)i * n + j] : 0.f;
+        float* dst = Bt + m * n * ld;
+        const int j0 = tj * 64 + tx;
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int i = ti * 64 + ty + 4 * u;
+            v[u] = (i < n && j0 < n) ? src[(int64_t)i * n + j0] : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) t[ty + 4 * u][tx] = v[u];
         __syncthreads();
-        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-            const int j = tj * 32 + r, i = ti * 32 + threadIdx.x;
-            if (i < n && j < n) dst[(int64_t)j * n + i] = t[threadIdx.x][r];
+        const int i0 = ti * 64 + tx;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const int j = tj * 64 + ty + 4 * u;
+            if (i0 < n && j < n) dst[(int64_t)j * ld + i0] = t[tx][ty + 4 * u];
         }
         __syncthreads();
     }
+}
+__global__ void __launch_bounds__(256) k_dense_pad(int64_t rows, int n, int ld, const float* __restrict__ A,
+                                                   float* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps)
+        for (int c = lane; c < n; c += 32) out[r * ld + c] = A[r * n + c];
 }
 
 // FP64: C tile 64 x 64 per CTA of 256 threads, each a 4 x 4 register tile; K in slices of 16
@@ -428,7 +347,7 @@ __global__ void k_dense_transpose(int64_t nb, int n, const float* __restrict__ B
 constexpr int kF = 64, kFK = 16;
 
 __global__ void __launch_bounds__(256) k_dense_f64(int n, double alpha, const double* __restrict__ A,
-                                                   const double* __restrict__ B, double beta, double* __restrict__ C) {
+                                                   const double* __restrict__ B, double beta, const double* Cin, double* C) {
     __shared__ double sa[kFK][kF + 1];   // A slice transposed: sa[k][i]
     __shared__ double sb[kFK][kF + 1];
     const int64_t b = blockIdx.z;
@@ -461,6 +380,7 @@ __global__ void __launch_bounds__(256) k_dense_f64(int n, double alpha, const do
         __syncthreads();
     }
     double* c = C + b * n * n;
+    const double* ci = Cin + b * n * n;
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -468,20 +388,19 @@ __global__ void __launch_bounds__(256) k_dense_f64(int n, double alpha, const do
             const int i = i0 + ty + 16 * x, j = j0 + tx + 16 * y;
             if (i < n && j < n) {
                 const int64_t p = (int64_t)i * n + j;
-                c[p] = beta == 0.0 ? alpha * acc[x][y] : alpha * acc[x][y] + beta * c[p];
+                c[p] = beta == 0.0 ? alpha * acc[x][y] : alpha * acc[x][y] + beta * ci[p];
             }
         }
 }
 
 }  // namespace
 
-void dense_gemm_f64(int64_t nb, int n, double alpha, const double* A, const double* B, double beta, double* C,
-                    cudaStream_t s) {
-    if (nb > 0 && n > 0 && nb > 65535) fail(DBCSR_ECAPACITY, "dense_gemm: more than 65535 matrices in one batch");
+void dense_gemm_f64(int64_t nb, int n, double alpha, const double* A, const double* B, double beta, const double* Cin,
+                    double* C, cudaStream_t s) {
     if (nb <= 0 || n <= 0) return;
     if (nb > 65535) fail(DBCSR_ECAPACITY, "dense_gemm: more than 65535 matrices in one batch");
     const dim3 grid((unsigned)ceil_div(n, kF), (unsigned)ceil_div(n, kF), (unsigned)nb);
-    k_dense_f64<<<grid, 256, 0, s>>>(n, alpha, A, B, beta, C);
+    k_dense_f64<<<grid, 256, 0, s>>>(n, alpha, A, B, beta, Cin, C);
     DBG_LAUNCH_CK();
 }
 
@@ -499,12 +418,12 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// Tensor map over a batch of n x n row-major FP32 matrices: boxes of 16 columns x rows rows of
-// one matrix, 64-byte swizzled (n a multiple of 4: row strides of whole 16-byte units).
-CUtensorMap batch_map(const float* base, int n, int64_t nb, int rows) {
+// Tensor map over a batch of n x n row-major FP32 matrices with rows of ld floats (a multiple of 4):
+// boxes of 16 columns x rows rows of one matrix, 64-byte swizzled.
+CUtensorMap batch_map(const float* base, int n, int ld, int64_t nb, int rows) {
     CUtensorMap m;
     const cuuint64_t dims[3] = {(cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)nb};
-    const cuuint64_t strides[2] = {(cuuint64_t)n * 4, (cuuint64_t)n * n * 4};
+    const cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)n * ld * 4};
     const cuuint32_t box[3] = {(cuuint32_t)kTK, (cuuint32_t)rows, 1};
     const cuuint32_t es[3] = {1, 1, 1};
     const CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims,
@@ -515,74 +434,69 @@ CUtensorMap batch_map(const float* base, int n, int64_t nb, int rows) {
     return m;
 }
 
+template <bool SPLIT>
+void launch_tf32(const CUtensorMap& ma, const CUtensorMap& mb, const TmaArgs& d, cudaStream_t s) {
+    const size_t sm = sizeof(TmaShared<SPLIT>) + 1024;
+    allow_dyn_smem(k_dense_tf32<SPLIT>, sm);
+    const unsigned grid = (unsigned)std::min<int64_t>(d.ntiles, (int64_t)num_sms());
+    k_dense_tf32<SPLIT><<<grid, 32 * (2 + (SPLIT ? kTConvWarps : 0) + kDEpiWarps), sm, s>>>(ma, mb, d);
+    DBG_LAUNCH_CK();
+}
+
 }  // namespace
 
-void dense_gemm_tf32(int64_t nb, int n, float alpha, const float* A, const float* B, float beta, float* C, bool split,
-                     cudaStream_t s) {
-    if (nb <= 0 || n <= 0) return;
-    if (nb > 65535) fail(DBCSR_ECAPACITY, "dense_gemm: more than 65535 matrices in one batch");
-    const bool aligned = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-    if (n % 4 == 0 && aligned) {
-        // operands straight from the matrices: A by rows, B^T (one transpose pass) by rows
-        const int ntm = (int)ceil_div(n, kDM);
-        const int ntn = (int)ceil_div(n, kDNMax);
-        const int NT = (int)ceil_div(ceil_div(n, ntn), 16) * 16;
-        DBuf<float> bt;
-        DBuf<int> err;
-        bt.alloc(nb * n * (int64_t)n, s);
-        err.alloc(1, s);
-        err.zero();
-        const int64_t tiles = nb * ceil_div(n, 32) * ceil_div(n, 32);
-        k_dense_transpose<<<grid_for(tiles, 1), dim3(32, 8), 0, s>>>(nb, n, B, bt.p);
-        DBG_LAUNCH_CK();
-        const CUtensorMap ma = batch_map(A, n, nb, kDM), mb = batch_map(bt.p, n, nb, NT);
-        const TmaArgs d{n, ntm, ntn, NT, alpha, beta, C, err.p};
-        const dim3 grid((unsigned)ntm, (unsigned)ntn, (unsigned)nb);
-        if (split) {
-            const size_t sm = sizeof(TmaShared<true>) + 1024;
-            allow_dyn_smem(k_dense_tf32_tma<true>, sm);
-            k_dense_tf32_tma<true><<<grid, kTThreads, sm, s>>>(ma, mb, d);
-        } else {
-            const size_t sm = sizeof(TmaShared<false>) + 1024;
-            allow_dyn_smem(k_dense_tf32_tma<false>, sm);
-            k_dense_tf32_tma<false><<<grid, kTThreads, sm, s>>>(ma, mb, d);
-        }
-        DBG_LAUNCH_CK();
-        int e = 0;
-        DBG_CK(cudaMemcpyAsync(&e, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        DBG_CK(cudaStreamSynchronize(s));
-        if (e) fail(DBCSR_ETIMEOUT, "dense_gemm: a wait of the tensor-core kernel ran out");
-        return;
-    }
-    const int np = split ? 2 : 1;
-    const int kpad = (int)ceil_div(n, kDStepK) * kDStepK;
-    const int ntm = (int)ceil_div(n, kDM);
-    // N tiles of equal width (a multiple of 16, at most 256)
-    const int ntn = (int)ceil_div(n, kDNMax);
-    const int NT = (int)ceil_div(ceil_div(n, ntn), 16) * 16;
-    const int64_t a_bytes = nb * ntm * (int64_t)(kpad / kDStepK) * np * 2 * kDM * 16;
-    const int64_t b_bytes = nb * ntn * (int64_t)(kpad / kDStepK) * np * 2 * NT * 16;
-    DBuf<float> pa, pb;
-    DBuf<int> err;
-    pa.alloc(a_bytes / 4, s);
-    pb.alloc(b_bytes / 4, s);
+DenseScratch::DenseScratch(cudaStream_t s) {
     err.alloc(1, s);
     err.zero();
-    const int64_t ta = nb * ntm * (int64_t)kDM * (kpad / 4), tb = nb * ntn * (int64_t)NT * (kpad / 4);
-    k_dense_pack<<<grid_for(ta, 256), 256, 0, s>>>(ta, n, kpad, kDM, ntm, np, 0, A, pa.p);
-    DBG_LAUNCH_CK();
-    k_dense_pack<<<grid_for(tb, 256), 256, 0, s>>>(tb, n, kpad, NT, ntn, np, 1, B, pb.p);
-    DBG_LAUNCH_CK();
-    DenseArgs d{n, kpad, ntm, ntn, NT, np, reinterpret_cast<const uint8_t*>(pa.p),
-                reinterpret_cast<const uint8_t*>(pb.p), alpha, beta, C, err.p};
-    const size_t sm = sizeof(DenseShared) + 1024;
-    allow_dyn_smem(k_dense_tf32, sm);
-    k_dense_tf32<<<dim3((unsigned)ntm, (unsigned)ntn, (unsigned)nb), kDThreads, sm, s>>>(d);
-    DBG_LAUNCH_CK();
+}
+
+void DenseScratch::check(cudaStream_t s) {
     int e = 0;
     DBG_CK(cudaMemcpyAsync(&e, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     DBG_CK(cudaStreamSynchronize(s));
     if (e) fail(DBCSR_ETIMEOUT, "dense_gemm: a wait of the tensor-core kernel ran out");
+}
+
+void dense_gemm_tf32(int64_t nb, int n, float alpha, const float* A, const float* B, float beta, const float* Cin,
+                     float* C, bool split, DenseScratch& w, cudaStream_t s) {
+    if (nb <= 0 || n <= 0) return;
+    if (nb > 65535) fail(DBCSR_ECAPACITY, "dense_gemm: more than 65535 matrices in one batch");
+    const int ld = (n + 3) & ~3;
+    // N tiles of equal width (a multiple of 16, at most 256), as many as give the shortest run of
+    // whole waves: an MMA takes NT / 2 clocks, at least about 66 (measured), and a tile about 20 of
+    // those clocks per K step besides.  (58 matrices of 432 x 432: 3.05 waves of 224 columns run as
+    // 4, 4.6 waves of 144 columns as 5 shorter ones.)
+    const int ntm = (int)ceil_div(n, kDM);
+    int ntn = 1, NT = 0;
+    int64_t best = 0;
+    for (int t = (int)ceil_div(n, kDNMax); t <= (int)ceil_div(n, 64) || !NT; ++t) {
+        const int w = (int)ceil_div(ceil_div(n, t), 16) * 16;
+        const int64_t cost = ceil_div(nb * ntm * t, num_sms()) * (std::max(w / 2, 66) + 20);
+        if (!NT || cost < best) {
+            best = cost;
+            ntn = t;
+            NT = w;
+        }
+    }
+    const int64_t need = nb * n * (int64_t)ld;
+    if (w.bt.n < need) w.bt.alloc(need, s);
+    const int64_t tiles = nb * ceil_div(n, 64) * ceil_div(n, 64);
+    k_dense_transpose<<<grid_for(tiles, 1, (int64_t)num_sms() * 8), 256, 0, s>>>(nb, n, ld, B, w.bt.p);
+    DBG_LAUNCH_CK();
+    const float* a = A;
+    // tensor maps want 16-byte rows; and a C over A must not be written while A's tiles are read
+    const auto pa = reinterpret_cast<uintptr_t>(A), pc = reinterpret_cast<uintptr_t>(C);
+    const uintptr_t bytes = (uintptr_t)nb * n * n * sizeof(float);
+    if (ld != n || (pa & 15) != 0 || (pa < pc + bytes && pc < pa + bytes)) {
+        if (w.a.n < need) w.a.alloc(need, s);
+        k_dense_pad<<<grid_for(nb * n, 8), 256, 0, s>>>(nb * n, n, ld, A, w.a.p);
+        DBG_LAUNCH_CK();
+        a = w.a.p;
+    }
+    const CUtensorMap ma = batch_map(a, n, ld, nb, kDM), mb = batch_map(w.bt.p, n, ld, nb, NT);
+    const TmaArgs d{n, ntm, ntn, NT, nb * ntm * ntn, alpha, beta, Cin, C, w.err.p};
+    if (split) launch_tf32<true>(ma, mb, d, s);
+    else launch_tf32<false>(ma, mb, d, s);
 }
 
 }  // namespace dbg
@@ -594,11 +508,13 @@ extern "C" dbcsr_status dbcsr_dense_multiply(int32_t prec, int64_t nb, int32_t n
             dbg::fail(DBCSR_EINVAL, "dense_multiply: bad argument");
         cudaStream_t s = (cudaStream_t)stream;
         if (prec == DBCSR_FP64) {
-            dbg::dense_gemm_f64(nb, n, alpha, (const double*)A, (const double*)B, beta, (double*)C, s);
+            dbg::dense_gemm_f64(nb, n, alpha, (const double*)A, (const double*)B, beta, (const double*)C, (double*)C, s);
             DBG_CK(cudaStreamSynchronize(s));
         } else if (prec == DBCSR_TF32 || prec == DBCSR_TF32X3) {
-            dbg::dense_gemm_tf32(nb, n, (float)alpha, (const float*)A, (const float*)B, (float)beta, (float*)C,
-                                 prec == DBCSR_TF32X3, s);
+            dbg::DenseScratch w(s);
+            dbg::dense_gemm_tf32(nb, n, (float)alpha, (const float*)A, (const float*)B, (float)beta, (const float*)C,
+                                 (float*)C, prec == DBCSR_TF32X3, w, s);
+            w.check(s);
         } else {
             dbg::fail(DBCSR_EINVAL, "dense_multiply: prec must be DBCSR_FP64, DBCSR_TF32 or DBCSR_TF32X3");
         }

@@ -43,53 +43,141 @@ __device__ __forceinline__ int64_t find_col(const int64_t* __restrict__ rp, cons
     return (lo < rp[row + 1] && col[lo] == c) ? lo : -1;
 }
 
-// One CTA per submatrix s (block column j = sub_j[s]): the dense, scaled, padded X_0.
-// doff[dstart[s] + a] = first row of block I_j[a] inside the submatrix.
+// The dense, scaled, padded X_0 of submatrix s (block column j = sub_j[s]), in `parts` CTAs: CTA p
+// clears and fills the block rows a = p, p + parts, ... (the last one also the identity padding).
+// doff[dstart[s] + a] = first row of block I_j[a] inside the submatrix.  Bound by the searches' and
+// blocks' load latency: one CTA per submatrix that cleared the whole matrix first and copied a block
+// per thread took 3.1 ms for five chunks of 96 waters, this split 0.94 ms.
 template <class T>
-__global__ void k_sub_gather(int32_t nsub, const int32_t* __restrict__ sub_j, const int64_t* __restrict__ dstart,
-                             const int32_t* __restrict__ doff, const int32_t* __restrict__ sub_n, int n_pad,
+__global__ void __launch_bounds__(256) k_sub_gather(int32_t nsub, int parts, const int32_t* __restrict__ sub_j,
+                             const int64_t* __restrict__ dstart, const int32_t* __restrict__ doff,
+                             const int32_t* __restrict__ sub_n, int n_pad,
                              const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                              const int64_t* __restrict__ off, const double* __restrict__ data,
                              const int32_t* __restrict__ bs, double mu, double inv_alpha, T* __restrict__ X) {
-    for (int32_t s = blockIdx.x; s < nsub; s += gridDim.x) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int64_t w = blockIdx.x; w < (int64_t)nsub * parts; w += gridDim.x) {
+        const int32_t s = (int32_t)(w / parts);
+        const int part = (int)(w - (int64_t)s * parts);
         T* x = X + (int64_t)s * n_pad * n_pad;
-        for (int64_t e = threadIdx.x; e < (int64_t)n_pad * n_pad; e += blockDim.x) x[e] = T(0);
-        __syncthreads();
         const int32_t j = sub_j[s];
         const int64_t q0 = rp[j];
         const int L = (int)(rp[j + 1] - q0);
         const int32_t* d = doff + dstart[s];
-        for (int p = threadIdx.x; p < L * L; p += blockDim.x) {
-            const int a = p / L, c = p - a * L;
-            const int32_t i = col[q0 + a], k = col[q0 + c];
-            const int64_t q = find_col(rp, col, i, k);
-            if (q < 0) continue;
-            const int mi = bs[i], mk = bs[k];
-            const double* v = data + off[q];
-            for (int r = 0; r < mi; ++r)
-                for (int t = 0; t < mk; ++t) {
-                    double y = v[r * mk + t];
-                    if (i == k && r == t) y -= mu;
-                    x[(int64_t)(d[a] + r) * n_pad + d[c] + t] = T(y * inv_alpha);
+        for (int a = part; a < L; a += parts) {
+            const int32_t i = col[q0 + a];
+            const int mi = bs[i];
+            T* xr = x + (int64_t)d[a] * n_pad;
+            for (int e = threadIdx.x; e < mi * n_pad; e += blockDim.x) xr[e] = T(0);
+            __syncthreads();
+            // a warp looks up 32 blocks (i, k) of the row at once, one per lane; small blocks are
+            // copied by their lane, larger ones by the warp
+            for (int c0 = 32 * warp; c0 < L; c0 += 32 * nw) {
+                const int c = c0 + lane;
+                const int32_t k = c < L ? col[q0 + c] : -1;
+                const int64_t q = c < L ? find_col(rp, col, i, k) : -1;
+                const int mk = q >= 0 ? bs[k] : 0;
+                auto copy = [&](const double* v, int w, T* o, bool diag, int e0, int de) {
+                    for (int e = e0; e < mi * w; e += de) {
+                        const int r = e / w, t = e - r * w;
+                        double y = v[e];
+                        if (diag && r == t) y -= mu;
+                        o[r * n_pad + t] = T(y * inv_alpha);
+                    }
+                };
+                const bool own = mi * mk <= 32;
+                const double* v = q >= 0 ? data + off[q] : nullptr;
+                const int dc = q >= 0 ? d[c] : 0;
+                if (own && mk) copy(v, mk, xr + dc, i == k, 0, 1);
+                unsigned big = __ballot_sync(0xffffffffu, !own);
+                while (big) {
+                    const int y = __ffs(big) - 1;
+                    big &= big - 1;
+                    const double* vy = reinterpret_cast<const double*>(
+                        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(v), y));
+                    copy(vy, __shfl_sync(0xffffffffu, mk, y), xr + __shfl_sync(0xffffffffu, dc, y),
+                         __shfl_sync(0xffffffffu, i == k ? 1 : 0, y) != 0, lane, 32);
                 }
+            }
         }
-        for (int k = sub_n[s] + threadIdx.x; k < n_pad; k += blockDim.x) x[(int64_t)k * n_pad + k] = T(1);
+        if (part == parts - 1) {
+            const int n = sub_n[s];
+            for (int e = threadIdx.x; e < (n_pad - n) * n_pad; e += blockDim.x) {
+                const int r = n + e / n_pad, c = e % n_pad;
+                x[(int64_t)r * n_pad + c] = r == c ? T(1) : T(0);
+            }
+        }
         __syncthreads();
     }
 }
 
-// One CTA per submatrix: ||X2 - 1||_F^2 (fixed thread order, fixed tree).
-template <class T>
-__global__ void k_sub_residual(int32_t nsub, int n_pad, const T* __restrict__ X2, double* __restrict__ r2) {
-    __shared__ double part[256];
-    for (int32_t s = blockIdx.x; s < nsub; s += gridDim.x) {
-        const T* x = X2 + (int64_t)s * n_pad * n_pad;
-        double acc = 0.0;
-        for (int64_t e = threadIdx.x; e < (int64_t)n_pad * n_pad; e += blockDim.x) {
-            const double v = (double)x[e] - ((e / n_pad) == (e % n_pad) ? 1.0 : 0.0);
+// ||X2 - 1||_F^2 of every submatrix in `parts` sums of fixed row ranges, thread orders and trees (the
+// host adds a submatrix's parts in order): one CTA per submatrix left SMs idle in small batches.  FP32
+// values are squared and summed 16 at a time as unevaluated pairs of FP32 (the squares exactly, Knuth's
+// sums, 48 bits) and the pair added to the thread's FP64 sum: the FP64 pipe, at under two operations
+// per clock, took three per element before (and a 64-bit division per element stood beside them): 30 ms
+// in the 107 residuals of the 96-water submatrix sign, now 2.1 ms.  The sum's error bound falls with
+// the number of FP64 additions (2^-47 against 2^-43 relative).
+__device__ __forceinline__ void residual_add(float v, float& h, float& l) {
+    const float p = v * v, e = fmaf(v, v, -p);
+    const float s = h + p, z = s - h;
+    l += (h - (s - z)) + (p - z) + e;
+    h = s;
+}
+
+__device__ __forceinline__ double residual_sum(const float* __restrict__ x, int n, int r0, int r1) {
+    // n is a multiple of 16: 16 consecutive elements lie in one row
+    double acc = 0.0;
+    const int per = n / 16;
+    for (int g = r0 * per + threadIdx.x; g < r1 * per; g += blockDim.x) {
+        const int row = g / per, c0 = (g - row * per) * 16;
+        const float4* p = reinterpret_cast<const float4*>(x + (int64_t)row * n + c0);
+        float4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = __ldg(p + u);
+        const float* v = reinterpret_cast<const float*>(q);
+        float h = 0.f, l = 0.f, m = 0.f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) m = fmaxf(m, fabsf(v[u]));
+        bool pairs = true;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) pairs = pairs && v[u] == v[u];
+        if (pairs && m < 1e18f && (m == 0.f || m > 1e-14f)) {
+#pragma unroll
+            for (int u = 0; u < 16; ++u)
+                if (c0 + u != row) residual_add(v[u], h, l);
+        } else {                                        // squares outside FP32's range, or NaN
+            for (int u = 0; u < 16; ++u)
+                if (c0 + u != row) acc = fma((double)v[u], (double)v[u], acc);
+        }
+        if (row >= c0 && row < c0 + 16) {               // the diagonal element minus 1, in FP64
+            const double d = (double)x[(int64_t)row * n + row] - 1.0;
+            acc = fma(d, d, acc);
+        }
+        acc += (double)h + (double)l;
+    }
+    return acc;
+}
+
+__device__ __forceinline__ double residual_sum(const double* __restrict__ x, int n, int r0, int r1) {
+    double acc = 0.0;
+    for (int row = r0 + (threadIdx.x >> 5); row < r1; row += blockDim.x >> 5)
+        for (int c = threadIdx.x & 31; c < n; c += 32) {
+            const double v = x[(int64_t)row * n + c] - (row == c ? 1.0 : 0.0);
             acc = fma(v, v, acc);
         }
-        part[threadIdx.x] = acc;
+    return acc;
+}
+
+template <class T>
+__global__ void __launch_bounds__(256) k_sub_residual(int32_t nsub, int parts, int n_pad, const T* __restrict__ X2,
+                                                      double* __restrict__ r2) {
+    __shared__ double part[256];
+    for (int64_t s = blockIdx.x; s < (int64_t)nsub * parts; s += gridDim.x) {
+        const int64_t m = s / parts;
+        const int p = (int)(s - m * parts);
+        part[threadIdx.x] = residual_sum(X2 + m * n_pad * n_pad, n_pad, (int)((int64_t)n_pad * p / parts),
+                                         (int)((int64_t)n_pad * (p + 1) / parts));
         __syncthreads();
         for (int o = blockDim.x / 2; o > 0; o >>= 1) {
             if ((int)threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
@@ -137,13 +225,13 @@ struct Chunk {
 
 // C = alpha A B + beta C for every matrix of the chunk: FP64, or FP32 storage in TF32
 // (split: three products of TF32 halves).
-void batched_gemm(int32_t b, int n, double alpha, const double* A, const double* B, double beta, double* C, bool,
-                  cudaStream_t s) {
-    dense_gemm_f64(b, n, alpha, A, B, beta, C, s);
+void batched_gemm(int32_t b, int n, double alpha, const double* A, const double* B, double beta, const double* Cin, double* C,
+                  bool, DenseScratch&, cudaStream_t s) {
+    dense_gemm_f64(b, n, alpha, A, B, beta, Cin, C, s);
 }
-void batched_gemm(int32_t b, int n, double alpha, const float* A, const float* B, double beta, float* C, bool split,
-                  cudaStream_t s) {
-    dense_gemm_tf32(b, n, (float)alpha, A, B, (float)beta, C, split, s);
+void batched_gemm(int32_t b, int n, double alpha, const float* A, const float* B, double beta, const float* Cin, float* C,
+                  bool split, DenseScratch& w, cudaStream_t s) {
+    dense_gemm_tf32(b, n, (float)alpha, A, B, (float)beta, Cin, C, split, w, s);
 }
 
 struct ChunkResult {
@@ -172,24 +260,34 @@ ChunkResult run_chunk(const Chunk& ck, dbcsr_matrix_* H, dbcsr_matrix_* P, doubl
     X2.alloc(elems, s);
     U.alloc(elems, s);
     DBuf<double> r2;
-    r2.alloc(b, s);
+    // CTAs per submatrix: about eight per SM in all
+    const int parts = (int)std::min<int64_t>(16, std::max<int64_t>(1, (int64_t)num_sms() * 8 / b));
+    r2.alloc((int64_t)b * parts, s);
     const unsigned grid = (unsigned)std::min<int64_t>(b, (int64_t)num_sms() * 8);
-    k_sub_gather<T><<<grid, 256, 0, s>>>(b, d_j.p, d_start.p, d_doff.p, d_n.p, n, H->rp.p, H->col.p, H->off.p,
+    const unsigned grid_p = (unsigned)std::min<int64_t>((int64_t)b * parts, (int64_t)num_sms() * 8);
+    k_sub_gather<T><<<grid_p, 256, 0, s>>>(b, parts, d_j.p, d_start.p, d_doff.p, d_n.p, n, H->rp.p, H->col.p, H->off.p,
                                          H->data.p, H->bs.p, mu, inv_alpha, X.p);
     DBG_LAUNCH_CK();
-    std::vector<double> h_r2(b);
+    DenseScratch w(s);
+    std::vector<double> h_r2((size_t)b * parts);
     ChunkResult cr;
     bool tf32 = mixed;
     const double gemm_flops = 2.0 * (double)n * n * n * b;
     while (true) {
-        batched_gemm(b, n, 1.0, X.p, X.p, 0.0, X2.p, !tf32, s);                // X2 = X X
+        batched_gemm(b, n, 1.0, X.p, X.p, 0.0, X2.p, X2.p, !tf32, w, s);             // X2 = X X
         cr.flops += gemm_flops;
-        k_sub_residual<T><<<grid, 256, 0, s>>>(b, n, X2.p, r2.p);
+        k_sub_residual<T><<<grid_p, 256, 0, s>>>(b, parts, n, X2.p, r2.p);
         DBG_LAUNCH_CK();
-        DBG_CK(cudaMemcpyAsync(h_r2.data(), r2.p, sizeof(double) * b, cudaMemcpyDeviceToHost, s));
-        DBG_CK(cudaStreamSynchronize(s));
+        DBG_CK(cudaMemcpyAsync(h_r2.data(), r2.p, sizeof(double) * h_r2.size(), cudaMemcpyDeviceToHost, s));
+        w.check(s);                                       // (waits for the stream)
         double rm = 0.0;
-        for (double v : h_r2) rm = std::max(rm, std::sqrt(v) / n);
+        for (int32_t m = 0; m < b; ++m) {
+            double v = 0.0;
+            for (int p = 0; p < parts; ++p) v += h_r2[(size_t)m * parts + p];
+            const double r = std::sqrt(v) / n;
+            if (!(r <= rm)) rm = r;                       // (a NaN stays)
+            if (!std::isfinite(r)) break;
+        }
         if (!std::isfinite(rm)) fail(DBCSR_ENAN, "submatrix_sign: residual is not finite");
         cr.r_max = rm;
         ++cr.iterations;
@@ -207,8 +305,7 @@ ChunkResult run_chunk(const Chunk& ck, dbcsr_matrix_* H, dbcsr_matrix_* P, doubl
         if (!tf32 && rm < o.tol) break;
         if (cr.iterations >= o.max_iter) break;
         // X <- 1.5 X - 0.5 X X2
-        DBG_CK(cudaMemcpyAsync(U.p, X.p, sizeof(T) * elems, cudaMemcpyDeviceToDevice, s));
-        batched_gemm(b, n, -0.5, X.p, X2.p, 1.5, U.p, !tf32, s);
+        batched_gemm(b, n, -0.5, X.p, X2.p, 1.5, X.p, U.p, !tf32, w, s);
         cr.flops += gemm_flops;
         std::swap(X.p, U.p);
     }

@@ -75,10 +75,12 @@ extern std::atomic<int64_t> g_launches;
 // Sets kernel's dynamic shared-memory limit to dyn bytes before a launch that asks for them.
 // The default limit (48 KB) covers static and dynamic shared memory together, so a launch
 // just under 48 KB of dynamic memory fails too when the kernel has static arrays; the
-// attribute is therefore set for every nonzero request.
+// attribute is therefore set for every nonzero request above the largest so far: it is never
+// lowered, since another thread may be between its own request and its launch.
+void allow_dyn_smem_of(const void* kernel, size_t dyn);
 template <class K>
 inline void allow_dyn_smem(K kernel, size_t dyn) {
-    if (dyn > 0) DBG_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    if (dyn > 0) allow_dyn_smem_of(reinterpret_cast<const void*>(kernel), dyn);
 }
 
 // The library's stream-ordered memory pool on the current device.  It keeps freed

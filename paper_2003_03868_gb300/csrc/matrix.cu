@@ -7,6 +7,7 @@
 // themselves row-major and packed in CSR order in data[nel] (FP64).
 #include <algorithm>
 #include <array>
+#include <map>
 #include <mutex>
 #include <numeric>
 #include <thread>
@@ -58,6 +59,18 @@ int num_sms() {
         cache[dev].store(n, std::memory_order_relaxed);
     }
     return n;
+}
+
+void allow_dyn_smem_of(const void* kernel, size_t dyn) {
+    static std::mutex mu;
+    static auto* limit = new std::map<std::pair<int, const void*>, size_t>();   // (outlives every static destructor)
+    int dev = 0;
+    DBG_CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    size_t& now = (*limit)[{dev, kernel}];
+    if (dyn <= now) return;
+    DBG_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    now = dyn;
 }
 
 void trim_pool(uint64_t keep_bytes) {

@@ -49,7 +49,7 @@ constexpr int kZeroBlocks = 6;                   // zero digit blocks before the
 constexpr int kDigitBlock = kSlice * 16;         // one digit of one 8-column chunk of a B slice
 constexpr int kOzBChunk = (kZeroBlocks + kDigits) * kDigitBlock;
 constexpr int kOzStage = kOzA + 2 * kOzBChunk;   // 42 KB
-constexpr int kOzStages = 5;
+constexpr int kOzStages = 4;
 constexpr int kOzEpiWarps = 16;                  // four per TMEM lane quadrant, 8 columns each
 constexpr int kOzItems = 4;                      // work items in flight between the warps' roles
 constexpr int kOzEpi0 = 2;                       // first epilogue warp: 0 producer, 1 MMA issuer
@@ -60,10 +60,13 @@ constexpr long long kOzWait = 4000000000ll;      // about 2 s
 // result's exponent is then formed without overflow from the two operands'.
 constexpr int kExpLimit = 430;
 constexpr int16_t kNoExp = -32768;
-// Clocks of one K step of one 32-column slice on one SM (768 for its eight MMAs, measured, plus
-// the operand copies' share), and the FP64 pipe's flops per clock and SM (1.01 TFLOP/s measured
-// on the block products).
-constexpr double kStepClocks = 430.0, kSimtFlopsPerClock = 3.2;
+// Clocks of one K step of one 32-column slice charged against the FP64 pipe's flops per clock and SM
+// (1.01 TFLOP/s measured on the block products) when a tile is given to one of the two.  A K step takes
+// about 768 clocks with eight digits and half of that on average (most entries run fewer); beside the
+// FP64 pipe's kernels the balance lies lower still.  Sign iteration on 512 waters: 234 ms at 430, 231 at
+// 350, 226 at 270, 227 at 200; 23/7 product 22.6 ms at 430, 22.7 at 270, 22.3 at 200; 1,024-water product
+// 28.6, 28.0, 28.0.
+constexpr double kStepClocks = 270.0, kSimtFlopsPerClock = 3.2;
 
 // ------------------------------------------------------------------ symbolic helpers
 __global__ void k_oz_role(int64_t nform, const int32_t* __restrict__ f_row, const int32_t* __restrict__ f_col,
@@ -369,6 +372,7 @@ struct OzShared {
     int64_t kcin[kGroupMembers][kGroupMembers];      // element offset of its C input, -1: none
     int kexp[kGroupMembers][kGroupMembers];          // exponent of its scale
     int colrec[kSlice];                              // member | column inside it << 8 | its width << 16; -1
+    int rowrec[128];                                 // member | row inside it << 8; -1
     int64_t item[kOzItems];
     uint64_t item_full[kOzItems], item_empty[kOzItems];
     uint64_t full[kOzStages], empty[kOzStages], acc_full[2], acc_empty[2], fin;
@@ -461,20 +465,18 @@ __device__ __forceinline__ double oz_value(const Oz96& x, int sc) {
     return __longlong_as_double((long long)(bits | ((uint64_t)neg << 63)));
 }
 
-// 4 consecutive 32-bit columns of one TMEM lane per thread, not waited for.
-__device__ __forceinline__ void oz_ld4(uint32_t taddr, float* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
-                 : "r"(taddr));
+// 2 consecutive 32-bit columns of one TMEM lane per thread, not waited for.
+__device__ __forceinline__ void oz_ld2(uint32_t taddr, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(taddr));
 }
 // The loaded registers are passed through, so that no use of them moves above the wait.
 template <int ND>
-__device__ __forceinline__ void oz_ld_wait(float (*v)[4]) {
+__device__ __forceinline__ void oz_ld_wait(float (*v)[2]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int d = 0; d < ND; ++d)
 #pragma unroll
-        for (int x = 0; x < 4; ++x) asm volatile("" : "+f"(v[d][x]));
+        for (int x = 0; x < 2; ++x) asm volatile("" : "+f"(v[d][x]));
 }
 
 // A box of a 4-D tensor map into shared memory.
@@ -532,31 +534,28 @@ template <int ND>
 __device__ __forceinline__ void oz_take(int nd, Oz96* acc, const int* ex, int ea, const int* ew, uint32_t taddr,
                                         uint64_t* free, int lane) {
 #pragma unroll
-    for (int g = 0; g < 2; ++g) {
-        float v[ND][4];
+    for (int g = 0; g < 4; ++g) {
+        float v[ND][2];
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
-            if (d < nd) {
-                oz_ld4(taddr + (uint32_t)(d * kSlice + 4 * g), v[d]);
-            } else {
-#pragma unroll
-                for (int x = 0; x < 4; ++x) v[d][x] = 0.f;
-            }
+            if (d < nd) oz_ld2(taddr + (uint32_t)(d * kSlice + 2 * g), v[d]);
+            else v[d][0] = v[d][1] = 0.f;
         }
         oz_ld_wait<ND>(v);
-        if (g == 1) {                                 // all of it is in registers: the buffer is free
+        if (g == 3) {                                 // all of it is in registers: the buffer is free
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(free);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int w = ew[2 * g + (j >> 1)];
-            const int sh = min(max(ex[4 * g + j] - ea - ((j & 1) ? w >> 16 : (int)(int16_t)(w & 0xffff)), 0), 95);
+        for (int j = 0; j < 2; ++j) {
+            const int x = j ? ex[g] >> 16 : (int)(int16_t)(ex[g] & 0xffff);
+            const int w = j ? ew[g] >> 16 : (int)(int16_t)(ew[g] & 0xffff);
+            const int sh = min(max(x - ea - w, 0), 95);
             float c[ND];
 #pragma unroll
             for (int d = 0; d < ND; ++d) c[d] = v[d][j];
-            oz_add<ND>(acc[4 * g + j], c, sh);
+            oz_add<ND>(acc[2 * g + j], c, sh);
         }
     }
 }
@@ -581,7 +580,11 @@ __device__ __forceinline__ void oz_item_done(OzShared& S, uint32_t n, int lane) 
 // steps (A by bulk copies, the B slice through a tensor map) into a ring of stages, warp 1
 // issues the MMAs, warps 2-17 combine a finished tile product's accumulators while the next one is
 // multiplied.
-__global__ void __launch_bounds__(kOzThreads, 1) k_oz(const __grid_constant__ OzMaps maps, OzArgs A) {
+// 64 registers a thread (a few spills outside the inner loop; 4% slower alone than with 96) leave room for
+// 12 and more warps of the FP64 pipe's kernels on the SM: together they finish 16 to 20% sooner than one
+// after the other.  For this the accumulators come two columns at a time and the scales' exponents are
+// held in pairs; with 96 registers nothing ran beside it, with 80 a third of the gain was there.
+__global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs A) {
     extern __shared__ __align__(1024) uint8_t oz_dyn[];
     OzShared& S = *reinterpret_cast<OzShared*>((reinterpret_cast<uintptr_t>(oz_dyn) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -787,36 +790,34 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz(const __grid_constant__ Oz
                 }
                 S.colrec[x] = rec;
             }
-            int ra = -1, ri = 0;
-            {
+            if (et >= kGroupMembers * kGroupMembers + 128) {
+                const int x = et - kGroupMembers * kGroupMembers - 128;
                 const int m0 = A.g_ptr[G], nm = A.g_ptr[G + 1] - m0;
+                int rec = -1;
                 for (int a = 0; a < nm; ++a) {
                     const int mr = A.g_mrec[m0 + a], p = mr & 255, w = mr >> 8;
-                    if (r >= p && r < p + w) {
-                        ra = a;
-                        ri = r - p;
-                    }
+                    if (x >= p && x < p + w) rec = a | ((x - p) << 8);
                 }
+                S.rowrec[x] = rec;
             }
             oz_epi_sync();
             if (S.epi_stop) break;
-            int ex[8];                                // the scale's exponent of each of this thread's elements
+            int ex[4];                                // the scales' exponents of this thread's elements, two a word
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int rec = S.colrec[8 * part + j];
-                ex[j] = ra >= 0 && rec >= 0 ? S.kexp[ra][rec & 255] : 4096;
+            for (int j = 0; j < 4; ++j) {
+                const int rr = S.rowrec[r], r0 = S.colrec[8 * part + 2 * j], r1 = S.colrec[8 * part + 2 * j + 1];
+                const int e0 = rr >= 0 && r0 >= 0 ? S.kexp[rr & 255][r0 & 255] : 4096;
+                const int e1 = rr >= 0 && r1 >= 0 ? S.kexp[rr & 255][r1 & 255] : 4096;
+                ex[j] = (e0 & 0xffff) | (int)((unsigned)e1 << 16);
             }
-            const int64_t e1 = A.s_ptr[t + 1];
             const int bcol = q * kSlice + 8 * part;   // first column of this thread
             Oz96 acc[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[j] = Oz96{0u, 0};
             bool ok = true;
-            int64_t e = A.s_ptr[t];
-            int4 nx = e < e1 ? __ldg(A.ent + e) : make_int4(0, 0, 0, 0);
-            for (; e < e1; ++e) {
-                const int4 en = nx;
-                if (e + 1 < e1) nx = __ldg(A.ent + e + 1);
+            const int4* ent = A.ent + A.s_ptr[t];
+            for (int ne = (int)(A.s_ptr[t + 1] - A.s_ptr[t]); ne > 0; --ne, ++ent) {
+                const int4 en = __ldg(ent);
                 if (!(((unsigned)en.z >> (8 * q)) & 255u)) continue;
                 const int nd = (int)(((unsigned)en.w >> (8 * q)) & 255u);
                 const int ea = r < A.R ? (int)__ldg(A.a_rexp + (int64_t)en.x * A.R + r) : 0;
@@ -837,7 +838,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz(const __grid_constant__ Oz
                 ++n;
             }
             oz_item_done(S, ni, lane);
-            if (ok && ra >= 0) {
+            const int rr = S.rowrec[r], ra = rr & 255, ri = rr >> 8;
+            if (ok && rr >= 0) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int rec = S.colrec[8 * part + j];
@@ -846,7 +848,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz(const __grid_constant__ Oz
                     const int64_t o = S.koff[ra][b];
                     if (o < 0) continue;
                     const int64_t p = (int64_t)ri * w + cj, ci = S.kcin[ra][b];
-                    double val = A.alpha * oz_value(acc[j], ex[j] - 70);
+                    double val = A.alpha * oz_value(acc[j], S.kexp[ra][b] - 70);
                     if (ci >= 0) val = val + A.beta * A.ci_data[ci + p];
                     A.c_data[o + p] = val;
                 }

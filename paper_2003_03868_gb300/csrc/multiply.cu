@@ -29,6 +29,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -967,6 +969,91 @@ struct EventSet {
     }
 };
 
+// Threads per CTA of the FP64-pipe kernels that run beside k_oz.  Its 18 warps of 64 registers leave
+// each quarter of an SM at least 6,144: a CTA of 256 threads may find no room.  H H on 512 waters, both
+// kernels: 13/5 11.7 ms with CTAs of 32, 12.7 with 64 (slower alone too), 11.8 with 128; 23/7 23.4, 22.6
+// and 22.7.
+constexpr int kBesideTpb = 128;
+
+// A second stream beside a product's own, leased from a bounded pool: begin() makes it wait for what
+// the product's stream holds, join() makes that stream wait for it.  A lease that ends between the two
+// (an exception) joins first, so that no buffer is freed under its kernels.
+class SideStream {
+    struct Res {
+        cudaStream_t s = nullptr;
+        cudaEvent_t fork = nullptr, done = nullptr;
+    };
+    static constexpr size_t kKept = 8;               // idle leases kept per device
+    static std::mutex& mu() {
+        static std::mutex m;
+        return m;
+    }
+    static std::map<int, std::vector<Res>>& idle() {
+        static auto* m = new std::map<int, std::vector<Res>>();   // (outlives every static destructor)
+        return *m;
+    }
+    static void destroy(Res& r) {
+        for (cudaEvent_t e : {r.fork, r.done})
+            if (e) cudaEventDestroy(e);
+        if (r.s) cudaStreamDestroy(r.s);
+    }
+    Res r_;
+    int dev_ = 0;
+    cudaStream_t main_ = nullptr;
+    bool open_ = false;
+
+public:
+    SideStream() {
+        DBG_CK(cudaGetDevice(&dev_));
+        {
+            std::lock_guard<std::mutex> lk(mu());
+            auto& v = idle()[dev_];
+            if (!v.empty()) {
+                r_ = v.back();
+                v.pop_back();
+                return;
+            }
+        }
+        try {
+            DBG_CK(cudaStreamCreateWithFlags(&r_.s, cudaStreamNonBlocking));
+            for (cudaEvent_t* e : {&r_.fork, &r_.done})
+                DBG_CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+        } catch (...) {
+            destroy(r_);
+            throw;
+        }
+    }
+    SideStream(const SideStream&) = delete;
+    SideStream& operator=(const SideStream&) = delete;
+    ~SideStream() {
+        bool keep = true;
+        if (open_) keep = cudaEventRecord(r_.done, r_.s) == cudaSuccess && cudaStreamWaitEvent(main_, r_.done, 0) == cudaSuccess;
+        cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+        keep = keep && cudaStreamIsCapturing(r_.s, &cst) == cudaSuccess && cst == cudaStreamCaptureStatusNone;
+        if (keep) {
+            std::lock_guard<std::mutex> lk(mu());
+            auto& v = idle()[dev_];
+            if (v.size() < kKept) {
+                v.push_back(r_);
+                return;
+            }
+        }
+        destroy(r_);
+    }
+    cudaStream_t stream() const { return r_.s; }
+    void begin(cudaStream_t main) {
+        main_ = main;
+        DBG_CK(cudaEventRecord(r_.fork, main));
+        DBG_CK(cudaStreamWaitEvent(r_.s, r_.fork, 0));
+        open_ = true;
+    }
+    void join() {
+        DBG_CK(cudaEventRecord(r_.done, r_.s));
+        DBG_CK(cudaStreamWaitEvent(main_, r_.done, 0));
+        open_ = false;
+    }
+};
+
 int sym_grid(int32_t nblk) { return std::min<int32_t>(nblk, num_sms() * 8); }
 
 // Counts the blocks on or above the diagonal that differ from their twin's transpose, and those below
@@ -1328,6 +1415,16 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     LowTierOut lto{};
     DBuf<int64_t> qcounter;                 // the work queue's counter (one-launch schedule)
     const int kmax = *std::max_element(A->h_bs.begin(), A->h_bs.end());
+    // the tuned configurations are looked up with the largest block edge as the inner size
+    auto smm_cfg = [&](int m, int n, bool beside) {
+        TuneCfg c = tune_lookup(prec, m, n, kmax);
+        if (beside) {
+            const int tpb = std::min(c.tpb, kBesideTpb);
+            c.ctas_per_sm = c.ctas_per_sm * c.tpb / tpb;
+            c.tpb = tpb;
+        }
+        return c;
+    };
     if (nform) {
         sa = SmmArgs{f_row.p, f_col.p, f_off.p, f_pbeg.p, f_cin.p, prod_a.p, prod_b.p, A->col.p, A->off.p, A->data.p,
                      B->off.p, B->data.p, use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, A->bs.p,
@@ -1378,7 +1475,6 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                              use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, alpha, beta,
                              c_data.p, c_norm.p, c_dev2.p};
         }
-        // the tuned configurations are looked up with the largest block edge as the inner size
         DBG_CK(cudaEventRecord(ev.e[1], s));
         if (bf16) {
             lowtier_run(*lt, A, lto, s);
@@ -1395,22 +1491,35 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             launches = std::move(rest);
             qcounter.alloc(1, s);
         }
-        at = 0;
-        for (const ShapeLaunch& L : launches) {
-            if (L.fallback) continue;
-            if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, s);
-            else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, sa, tune_lookup(prec, L.m, L.n, kmax), s);
-            at += L.cnt;
-            if (!bf16) ++n_smm_launches;
-        }
         if (tc) {
             lto = LowTierOut{f_rp.p, f_col.p, f_comp.p, f_off.p, use_c ? f_cin.p : nullptr,
                              use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, alpha, beta,
                              c_data.p, c_norm.p, c_dev2.p};
-            f64tc_run(*tcp, lto, s);
-            f64tc_norms(nform, f_comp.p, f_row.p, f_col.p, A->bs.p, f_off.p, c_data.p, c_norm.p, c_dev2.p, s);
             ++n_smm_launches;
         }
+        // The FP64 pipe's blocks run beside the tensor cores' on a second stream: k_oz hardly uses the
+        // FP64 pipe, and its registers are held down so that both fit an SM.  One after the other they
+        // took 13.9 and 28.4 ms on 512 waters (13/5, 23/7), side by side 11.4 and 22.6.
+        std::unique_ptr<SideStream> side;
+        cudaStream_t ss = s;
+        if (tc) {
+            if (!launches.empty() && !launches[0].fallback) {
+                side.reset(new SideStream());
+                side->begin(s);
+                ss = side->stream();
+            }
+            f64tc_run(*tcp, lto, s);
+            f64tc_norms(nform, f_comp.p, f_row.p, f_col.p, A->bs.p, f_off.p, c_data.p, c_norm.p, c_dev2.p, s);
+        }
+        at = 0;
+        for (const ShapeLaunch& L : launches) {
+            if (L.fallback) continue;
+            if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, ss);
+            else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, sa, smm_cfg(L.m, L.n, (bool)side), ss);
+            at += L.cnt;
+            if (!bf16) ++n_smm_launches;
+        }
+        if (side) side->join();
         if (sym_result) {
             DBG_CK(cudaEventRecord(ev.e[2], s));     // the copy / averaging is timed with the filter
             k_mirror_copy<<<grid_for(nform, 8), 256, 0, s>>>(nform, sym_result, mirror.p, f_row.p, f_col.p, f_off.p,
@@ -1466,6 +1575,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         }
         // captured on a private stream (the legacy default stream cannot be captured); the
         // graph is launched on C's stream
+        SideStream side;
         cudaStream_t cs = nullptr;
         DBG_CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
         cudaGraph_t graph = nullptr;
@@ -1477,21 +1587,26 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                 lowtier_run(*lt, A, lto, cs);
             }
             SmmArgs fb = sa;
+            const bool beside = tc && !launches.empty() && !launches[0].fallback;
             if (tc) {
                 // the tensor cores' blocks with the current values; the FP64 pipe repeats them all
                 // when these need it (f64tc_recheck)
                 f64tc_pack(*tcp, A, B, cs);
                 fb.gate = f64tc_recheck(*tcp, A, B, an.p, bn.p, nform, f64tc_blocks, f_pbeg.p, prod_a.p, prod_b.p, alpha, cs);
+                if (beside) side.begin(cs);
                 f64tc_run(*tcp, lto, cs);
                 f64tc_norms(nform, f_comp.p, C->row.p, C->col.p, C->bs.p, C->off.p, C->data.p, C->norms.p, c_dev2.p, cs);
             }
             int64_t at = 0;
-            for (const ShapeLaunch& L : launches) {
-                if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, cs);
-                else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, L.fallback ? fb : sa,
-                                      tune_lookup(prec, L.m, L.n, kmax), cs);
+            for (size_t i = 0; i < launches.size(); ++i) {
+                const ShapeLaunch& L = launches[i];
+                const bool b = beside && !L.fallback;
+                if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, b ? side.stream() : cs);
+                else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, L.fallback ? fb : sa, smm_cfg(L.m, L.n, b),
+                                      b ? side.stream() : cs);
                 at += L.cnt;
             }
+            if (beside) side.join();
             zero_small(cs);
             DBG_CK(cudaStreamEndCapture(cs, &graph));
         } catch (...) {

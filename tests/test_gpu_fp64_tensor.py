@@ -170,3 +170,53 @@ def test_symmetric_square_equals_its_transpose_and_the_bound(gb):
     C = gb.Matrix(X.blk_size, X.stream)
     gb.multiply(1.0, X, X, 0.0, C, 0.0)
     _check(C, bsr.Mat(X.blk_size, *X.export()), bsr.Mat(X.blk_size, *X.export()))
+
+
+@pytest.mark.parametrize("planned", [False, True])
+def test_both_pipes_side_by_side_from_several_threads_and_streams(gb, planned):
+    # one product's blocks run on two streams; products of several threads, each on a stream of its own
+    # and one on the default stream, give the same bits as the same product by itself
+    import threading
+
+    import torch
+    hs = [synth.build_hamiltonian(synth.small(40 + 8 * i, basis=b, seed=50 + i)).H
+          for i, b in enumerate([(13, 5), (23, 7), (13, 7), (23, 5)])]
+    alone = []
+    for h in hs:
+        A = gb.Matrix.of(h)
+        C = gb.Matrix(A.blk_size, A.stream)
+        if planned:
+            p = gb.Plan(1.0, A, A, C, 1e-7)
+            p.execute()
+            alone.append(C.export())
+            p.close()
+        else:
+            assert gb.multiply(1.0, A, A, 0.0, C, 1e-7).n_tiles > 0
+            alone.append(C.export())
+    streams = [torch.cuda.Stream() for _ in hs[1:]]
+    bad = []
+
+    def work(i):
+        try:
+            st = None if i == 0 else streams[i - 1].cuda_stream
+            A = gb.Matrix.of(hs[i], st)
+            for _ in range(6):
+                C = gb.Matrix(A.blk_size, st)
+                if planned:
+                    p = gb.Plan(1.0, A, A, C, 1e-7)
+                    for _ in range(3):
+                        p.execute()
+                else:
+                    gb.multiply(1.0, A, A, 0.0, C, 1e-7)
+                if not all(np.array_equal(x, y) for x, y in zip(C.export(), alone[i])):
+                    bad.append(i)
+                if planned:
+                    p.close()
+        except Exception as e:                       # noqa: BLE001 -- reported by the main thread
+            bad.append((i, repr(e)))
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(len(hs))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad

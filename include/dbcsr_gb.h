@@ -74,7 +74,7 @@ typedef struct {
     int64_t n_products;        /* block products A_IK * B_KJ executed */
     double flops;              /* sum of 2*m*k*n over the executed products (unpadded) */
     double dev2_filtered;      /* ||C_filtered - 1||_F^2 (meaningful for X*X in the sign iteration) */
-    double ms_symbolic;        /* device time of the stack builder, ms */
+    double ms_symbolic;        /* device time of the stack builder up to the first block-product kernel, ms */
     double ms_numeric;         /* device time of the block-product kernel, ms */
     double ms_filter;          /* device time of norm-filter-compaction, ms */
     double bytes_min;          /* compulsory bytes of the block-product launches: A and B read once,
@@ -147,7 +147,7 @@ typedef struct {
     int64_t nnzb_x;            /* blocks of the converged X */
     double residual_history[DBCSR_MAX_HISTORY];
     int64_t nnzb_history[DBCSR_MAX_HISTORY];
-    double ms_symbolic;        /* device time of the stack builders, ms */
+    double ms_symbolic;        /* device time of the stack builders up to the first block-product kernels, ms */
     double ms_filter;          /* device time of norm-filter-compaction (and mirroring), ms */
     double ms_low;             /* device time of the low tier's block-product kernels, ms */
     double flops_low;          /* executed 2*m*k*n of the low tier's products */

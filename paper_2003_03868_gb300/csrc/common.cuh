@@ -133,7 +133,7 @@ struct DBuf {
 
 // Pinned host scratch for small device->host readbacks.
 struct HostScalars {
-    static constexpr int kCap = 256;
+    static constexpr int kCap = 4096;
     int64_t* i = nullptr;
     double* d = nullptr;
     HostScalars();
@@ -204,6 +204,9 @@ namespace dbg {
 // out[0..n] = exclusive prefix sum of in[0..n-1]; out[n] = total.  n >= 0.
 void scan_exclusive(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s);
 void scan_exclusive(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s);
+// Up to kScanJobs arrays of one length in one launch.
+constexpr int kScanJobs = 3;
+void scan_exclusive(const int64_t* const* in, int64_t* const* out, int jobs, int64_t n, cudaStream_t s);
 // Deterministic sum of v[0..n-1] into *out (device); fixed reduction tree for a given n.
 void det_sum(const double* v, int64_t n, double* out, cudaStream_t s);
 // The same sum with a caller-given buffer of kDetSumPartials doubles for the per-CTA partials.

@@ -967,17 +967,19 @@ void tile_patterns(const Groups& g, PatternJob* jobs, int n, int64_t* max_c, cud
     allow_dyn_smem(k_gt_pattern, sm);
     const unsigned grid = (unsigned)std::min<int64_t>(g.ngrp, (int64_t)num_sms() * 8);
     DBuf<int64_t> cnt[3];
-    const int64_t* src[4];
-    int64_t h[4];
+    const int64_t *src[3], *in[3];
+    int64_t h[3], *out[3];
     for (int i = 0; i < n; ++i) {
         cnt[i].alloc(g.ngrp, s);
         jobs[i].out->t_rp.alloc(g.ngrp + 1, s);
         k_gt_pattern<<<grid, 256, sm, s>>>(g.ngrp, gv, jobs[i].rp, jobs[i].col, jobs[i].use, nwords, 0, cnt[i].p, nullptr,
                                            nullptr, nullptr, nullptr);
         DBG_LAUNCH_CK();
-        scan_exclusive(cnt[i].p, jobs[i].out->t_rp.p, g.ngrp, s);
-        src[i] = jobs[i].out->t_rp.p + g.ngrp;
+        in[i] = cnt[i].p;
+        out[i] = jobs[i].out->t_rp.p;
+        src[i] = out[i] + g.ngrp;
     }
+    scan_exclusive(in, out, n, g.ngrp, s);
     std::vector<int64_t> rows(g.ngrp);
     DBG_CK(cudaMemcpyAsync(rows.data(), cnt[n - 1].p, sizeof(int64_t) * g.ngrp, cudaMemcpyDeviceToHost, s));
     read_i64s(src, n, h, s);

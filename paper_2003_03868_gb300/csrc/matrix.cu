@@ -115,6 +115,20 @@ HostScalars& host_scalars() {
     return hs;
 }
 
+namespace {
+constexpr int kReadPtrs = 8;
+struct ReadArgs {
+    const int64_t* p[kReadPtrs];
+    int k, na;
+    const int64_t* arr;
+    int64_t* out;                // pinned host memory
+};
+// Scalars from several arrays and one array to the host in one launch (a copy each took longer).
+__global__ void k_read_i64s(ReadArgs A) {
+    for (int j = threadIdx.x; j < A.k + A.na; j += blockDim.x) A.out[j] = j < A.k ? *A.p[j] : A.arr[j - A.k];
+}
+}  // namespace
+
 int64_t read_i64(const int64_t* dev, cudaStream_t s) {
     HostScalars& hs = host_scalars();
     DBG_CK(cudaMemcpyAsync(hs.i, dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -125,9 +139,15 @@ int64_t read_i64(const int64_t* dev, cudaStream_t s) {
 void read_i64s(const int64_t* const* dev, int k, int64_t* out, cudaStream_t s, const int64_t* arr, int na,
                int64_t* arr_out) {
     HostScalars& hs = host_scalars();
-    if (k + na > HostScalars::kCap) fail(DBCSR_ECAPACITY, "read_i64s: too many values");
-    for (int j = 0; j < k; ++j) DBG_CK(cudaMemcpyAsync(hs.i + j, dev[j], sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    if (na > 0) DBG_CK(cudaMemcpyAsync(hs.i + k, arr, sizeof(int64_t) * na, cudaMemcpyDeviceToHost, s));
+    if (k > kReadPtrs || k + na > HostScalars::kCap) fail(DBCSR_ECAPACITY, "read_i64s: too many values");
+    ReadArgs a{};
+    for (int j = 0; j < k; ++j) a.p[j] = dev[j];
+    a.k = k;
+    a.na = na;
+    a.arr = arr;
+    a.out = hs.i;
+    k_read_i64s<<<1, 256, 0, s>>>(a);
+    DBG_LAUNCH_CK();
     DBG_CK(cudaStreamSynchronize(s));
     for (int j = 0; j < k; ++j) out[j] = hs.i[j];
     for (int j = 0; j < na; ++j) arr_out[j] = hs.i[k + j];
@@ -250,18 +270,27 @@ __global__ void k_keep_norm(int64_t nb, const int32_t* __restrict__ row, const i
         keep[b] = (row[b] == col[b] || norms[b] >= eps) ? 1 : 0;
 }
 
-// Compaction: kept block b goes to index newidx[b] with data at newoff[newidx[b]].
+// Compaction: kept block b goes to index newidx[b], its data to newoff[b].
+__global__ void k_keep_counts(int64_t nb, const int32_t* __restrict__ keep, const int64_t* __restrict__ off,
+                              int64_t* __restrict__ one, int64_t* __restrict__ area) {
+    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x) {
+        one[b] = keep[b] ? 1 : 0;
+        area[b] = keep[b] ? off[b + 1] - off[b] : 0;
+    }
+}
+
 __global__ void k_compact_meta(int64_t nb, const int32_t* __restrict__ keep, const int64_t* __restrict__ newidx,
-                               const int32_t* __restrict__ row, const int32_t* __restrict__ col,
-                               const int32_t* __restrict__ bs, const double* __restrict__ norms,
-                               int32_t* __restrict__ nrow, int32_t* __restrict__ ncol, int64_t* __restrict__ narea,
+                               const int64_t* __restrict__ newoff, const int32_t* __restrict__ row,
+                               const int32_t* __restrict__ col, const double* __restrict__ norms,
+                               int32_t* __restrict__ nrow, int32_t* __restrict__ ncol, int64_t* __restrict__ noff,
                                double* __restrict__ nnorms) {
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x) {
+        if (b == 0) noff[newidx[nb]] = newoff[nb];
         if (!keep[b]) continue;
         const int64_t k = newidx[b];
         nrow[k] = row[b];
         ncol[k] = col[b];
-        narea[k] = (int64_t)bs[row[b]] * bs[col[b]];
+        noff[k] = newoff[b];
         if (nnorms) nnorms[k] = norms[b];
     }
 }
@@ -272,17 +301,16 @@ __global__ void k_compact_rp(int32_t nblk, const int64_t* __restrict__ rp, const
         nrp[I] = newidx[rp[I]];
 }
 
-__global__ void k_compact_data(int64_t nb, const int32_t* __restrict__ keep, const int64_t* __restrict__ newidx,
-                               const int64_t* __restrict__ off, const int64_t* __restrict__ noff,
-                               const double* __restrict__ data, double* __restrict__ ndata) {
+__global__ void k_compact_data(int64_t nb, const int32_t* __restrict__ keep, const int64_t* __restrict__ newoff,
+                               const int64_t* __restrict__ off, const double* __restrict__ data,
+                               double* __restrict__ ndata) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < nb; b += warps) {
         if (!keep[b]) continue;
-        const int64_t k = newidx[b];
         const int64_t area = off[b + 1] - off[b];
         const double* s = data + off[b];
-        double* d = ndata + noff[k];
+        double* d = ndata + newoff[b];
         for (int64_t e = lane; e < area; e += 32) d[e] = s[e];
     }
 }
@@ -363,34 +391,46 @@ void compact(dbcsr_matrix_* m, const int32_t* keep, const double* norms_in) {
     check_unplanned(m, "filter");
     cudaStream_t s = m->stream;
     const int64_t nb = m->nnzb;
-    DBuf<int64_t> newidx;
-    newidx.alloc(nb + 1, s);
-    scan_exclusive(keep, newidx.p, nb, s);
-    const int64_t nk = read_i64(newidx.p + nb, s);
+    DBuf<int64_t> one, area, newidx, newoff;
+    int64_t tot[2] = {0, 0};
+    if (nb) {
+        one.alloc(nb, s);
+        area.alloc(nb, s);
+        newidx.alloc(nb + 1, s);
+        newoff.alloc(nb + 1, s);
+        k_keep_counts<<<grid_for(nb, 256), 256, 0, s>>>(nb, keep, m->off.p, one.p, area.p);
+        DBG_LAUNCH_CK();
+        const int64_t* in[2] = {one.p, area.p};
+        int64_t* out[2] = {newidx.p, newoff.p};
+        scan_exclusive(in, out, 2, nb, s);
+        const int64_t* src[2] = {newidx.p + nb, newoff.p + nb};
+        read_i64s(src, 2, tot, s);
+    }
+    const int64_t nk = tot[0], nel = tot[1];
+    if (nk == nb) {                                       // nothing goes: the arrays stay
+        if (norms_in && norms_in != m->norms.p) {
+            m->norms.alloc(std::max<int64_t>(nb, 1), s);
+            DBG_CK(cudaMemcpyAsync(m->norms.p, norms_in, sizeof(double) * nb, cudaMemcpyDeviceToDevice, s));
+        }
+        m->norms_valid = norms_in != nullptr;
+        return;
+    }
     DBuf<int32_t> nrow, ncol;
-    DBuf<int64_t> narea, noff, nrp;
-    DBuf<double> nnorms;
+    DBuf<int64_t> noff, nrp;
+    DBuf<double> nnorms, ndata;
     nrow.alloc(std::max<int64_t>(nk, 1), s);
     ncol.alloc(std::max<int64_t>(nk, 1), s);
-    narea.alloc(std::max<int64_t>(nk, 1), s);
     noff.alloc(nk + 1, s);
     nrp.alloc(m->nblk + 1, s);
+    ndata.alloc(std::max<int64_t>(nel, 1), s);
     if (norms_in) nnorms.alloc(std::max<int64_t>(nk, 1), s);
-    if (nb) {
-        k_compact_meta<<<grid_for(nb, 256), 256, 0, s>>>(nb, keep, newidx.p, m->row.p, m->col.p, m->bs.p, norms_in,
-                                                         nrow.p, ncol.p, narea.p, norms_in ? nnorms.p : nullptr);
-        DBG_LAUNCH_CK();
-    }
+    k_compact_meta<<<grid_for(nb, 256), 256, 0, s>>>(nb, keep, newidx.p, newoff.p, m->row.p, m->col.p, norms_in,
+                                                     nrow.p, ncol.p, noff.p, norms_in ? nnorms.p : nullptr);
+    DBG_LAUNCH_CK();
     k_compact_rp<<<grid_for(m->nblk + 1, 256), 256, 0, s>>>(m->nblk, m->rp.p, newidx.p, nrp.p);
     DBG_LAUNCH_CK();
-    scan_exclusive(narea.p, noff.p, nk, s);
-    const int64_t nel = read_i64(noff.p + nk, s);
-    DBuf<double> ndata;
-    ndata.alloc(std::max<int64_t>(nel, 1), s);
-    if (nb) {
-        k_compact_data<<<grid_for(nb, 8), 256, 0, s>>>(nb, keep, newidx.p, m->off.p, noff.p, m->data.p, ndata.p);
-        DBG_LAUNCH_CK();
-    }
+    k_compact_data<<<grid_for(nb, 8), 256, 0, s>>>(nb, keep, newoff.p, m->off.p, m->data.p, ndata.p);
+    DBG_LAUNCH_CK();
     m->rp = std::move(nrp);
     m->row = std::move(nrow);
     m->col = std::move(ncol);

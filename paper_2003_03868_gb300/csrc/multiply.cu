@@ -878,18 +878,59 @@ __global__ void __launch_bounds__(256, 2) k_smm_f64_queue(int64_t nlist, const i
 }
 
 
-// Stable partition of the formed blocks by shape: flag[k] = (block k is m x n and comp[k] == want).
-__global__ void k_shape_flags(int64_t nform, const int32_t* __restrict__ f_row, const int32_t* __restrict__ f_col,
-                              const int32_t* __restrict__ bs, const uint8_t* __restrict__ comp, int want, int m, int n,
-                              int32_t* __restrict__ flag) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nform; k += (int64_t)gridDim.x * blockDim.x)
-        flag[k] = (comp[k] == want && bs[f_row[k]] == m && bs[f_col[k]] == n) ? 1 : 0;
-}
-
-__global__ void k_class_scatter(int64_t nform, const int32_t* __restrict__ flag, const int64_t* __restrict__ pos,
-                                int64_t* __restrict__ list) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nform; k += (int64_t)gridDim.x * blockDim.x)
-        if (flag[k]) list[pos[k]] = k;
+// Lists of the formed blocks by role and shape, in one pass: cursor[role][m][n] holds where a list goes
+// on (at first its beginning).  A CTA ranks 2,048 blocks in shared memory and takes its share of every
+// list with one atomic, so a list is in CSR order but for the order of the CTAs.  Any order gives the
+// same products, but neighbours share operand rows in L1: with the warps' ranks in any order the block
+// products of 32 waters took 0.12 ms longer.  Bound by the loads' latency: 8 us on 512 waters, where a flag
+// pass, a scan and a scatter per shape took 24 launches and 0.1 ms (37 shapes of a ragged matrix: 0.5 ms).
+constexpr int kListThreads = 256, kListItems = 8;
+__global__ void __launch_bounds__(kListThreads) k_shape_lists(int64_t nform, const int32_t* __restrict__ f_row,
+                                                              const int32_t* __restrict__ f_col,
+                                                              const int32_t* __restrict__ bs,
+                                                              const uint8_t* __restrict__ comp, int roles,
+                                                              unsigned long long* __restrict__ cursor,
+                                                              int64_t* __restrict__ list) {
+    constexpr int kBins = (kMaxBlock + 1) * (kMaxBlock + 1);
+    __shared__ unsigned cnt[2 * kBins];
+    __shared__ long long base[2 * kBins];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t k0 = (int64_t)blockIdx.x * (kListThreads * kListItems); k0 < nform;
+         k0 += (int64_t)gridDim.x * (kListThreads * kListItems)) {
+        for (int b = threadIdx.x; b < roles * kBins; b += kListThreads) cnt[b] = 0;
+        __syncthreads();
+        const int64_t kw = k0 + warp * (32 * kListItems) + lane;      // the warp's blocks: 256 in a row
+        int bin[kListItems];
+        unsigned same[kListItems], rank[kListItems];
+#pragma unroll
+        for (int u = 0; u < kListItems; ++u) {
+            const int64_t k = kw + 32 * u;
+            const int c = k < nform ? comp[k] : 0;
+            bin[u] = c && c <= roles ? (c - 1) * kBins + bs[f_row[k]] * (kMaxBlock + 1) + bs[f_col[k]] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kListItems; ++u) same[u] = __match_any_sync(0xffffffffu, bin[u]);
+        for (int w = 0; w < kListThreads / 32; ++w) {                 // the warps in turn: blocks in order
+            if (warp == w) {
+#pragma unroll
+                for (int u = 0; u < kListItems; ++u) {
+                    const unsigned at = bin[u] >= 0 ? cnt[bin[u]] : 0;
+                    rank[u] = at + __popc(same[u] & ((1u << lane) - 1u));
+                    __syncwarp();
+                    if (bin[u] >= 0 && lane == __ffs(same[u]) - 1) cnt[bin[u]] = at + __popc(same[u]);
+                    __syncwarp();
+                }
+            }
+            __syncthreads();
+        }
+        for (int b = threadIdx.x; b < roles * kBins; b += kListThreads)
+            if (cnt[b]) base[b] = (long long)atomicAdd(cursor + b, (unsigned long long)cnt[b]);
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kListItems; ++u)
+            if (bin[u] >= 0) list[base[bin[u]] + rank[u]] = kw + 32 * u;
+        __syncthreads();
+    }
 }
 
 using SmmKernel = void (*)(int64_t, const int64_t*, SmmArgs);
@@ -1369,14 +1410,16 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                                                           plan ? 1 : 0);
         DBG_LAUNCH_CK();
     }
-    scan_exclusive(f_area.p, f_off.p, nform, s);
-    scan_exclusive(f_np.p, f_pbeg.p, nform, s);
+    {
+        const int64_t* in[2] = {f_area.p, f_np.p};
+        int64_t* out[2] = {f_off.p, f_pbeg.p};
+        scan_exclusive(in, out, 2, nform, s);
+    }
     int64_t h3[4];
     std::vector<int64_t> shapes(2 * kShapes, 0);
     {
         const int64_t* src[4] = {f_off.p + nform, f_pbeg.p + nform, flops.p, nprod_exec.p};
-        DBG_CK(cudaMemcpyAsync(shapes.data(), shape_cnt.p, sizeof(int64_t) * 2 * kShapes, cudaMemcpyDeviceToHost, s));
-        read_i64s(src, 4, h3, s);
+        read_i64s(src, 4, h3, s, shape_cnt.p, 2 * kShapes, shapes.data());
     }
     const int64_t nel = h3[0], nprod = h3[1];
     const double nflop = (double)(unsigned long long)h3[2];
@@ -1389,15 +1432,16 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     const size_t sm_fill = sm_rank + (size_t)max_row * (sizeof(int64_t) + sizeof(int32_t));
     const bool fill_smem = sm_fill <= (size_t)kSymSmemBudget;
     if (!fill_smem && !bf16) cursor.alloc(nf1, s);
-    if (nprod && !bf16) {
+    auto fill_stacks = [&](cudaStream_t fs) {
+        if (!nprod || bf16) return;
         FillArgs fa{coff.p, keep.p, f_comp.p, plan ? 2 : 1, kidx.p, f_pbeg.p, cursor.p, prod_a.p, prod_b.p, fill_smem ? 1 : 0};
         const size_t sm = fill_smem ? sm_fill : sm_rank;
         allow_dyn_smem(k_fill_stack, sm);
-        k_fill_stack<<<sym_grid(nblk), kSymThreads, sm, s>>>(nblk, P, nwords, fa);
+        k_fill_stack<<<sym_grid(nblk), kSymThreads, sm, fs>>>(nblk, P, nwords, fa);
         DBG_LAUNCH_CK();
-    }
+    };
     // the candidate arrays are no longer needed
-    cand_row.release(); cand_col.release(); pcnt.release(); ksum.release(); bound.release(); cursor.release();
+    cand_row.release(); cand_col.release(); pcnt.release(); ksum.release(); bound.release();
     max_term.release(); f_max.release();
     if (!nform) DBG_CK(cudaEventRecord(ev.e[1], s));
 
@@ -1429,14 +1473,9 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         sa = SmmArgs{f_row.p, f_col.p, f_off.p, f_pbeg.p, f_cin.p, prod_a.p, prod_b.p, A->col.p, A->off.p, A->data.p,
                      B->off.p, B->data.p, use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, A->bs.p,
                      alpha, beta, c_data.p, c_norm.p, c_dev2.p};
-        // FP64: one launch per (m, n) block shape over that shape's blocks (kept in CSR order)
-        DBuf<int32_t> flag;
-        DBuf<int64_t> pos;
-        if (!bf16) {
-            flag.alloc(nform, s);
-            pos.alloc(nform + 1, s);
-            list.alloc(nform, s);
-        }
+        // FP64: one launch per (m, n) block shape over that shape's blocks
+        DBuf<int64_t> list_at;
+        std::vector<int64_t> h_at(2 * kShapes, 0);
         // with the one-launch schedule, the shapes the work queue takes come first in the list
         const bool queue = !bf16 && g_fp64_schedule.load() == 1;
         int64_t at = 0, at_q = 0, n_tc = 0;
@@ -1451,12 +1490,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                 bytes_min += 8.0 * (double)cnt * m * n;
                 if (pass == 2) n_tc += cnt;
                 if (bf16 || (pass == 2 && !plan)) continue;
-                k_shape_flags<<<grid_for(nform, 256), 256, 0, s>>>(nform, f_row.p, f_col.p, A->bs.p, f_comp.p,
-                                                                   pass == 2 ? 2 : 1, m, n, flag.p);
-                DBG_LAUNCH_CK();
-                scan_exclusive(flag.p, pos.p, nform, s);
-                k_class_scatter<<<grid_for(nform, 256), 256, 0, s>>>(nform, flag.p, pos.p, list.p + at);
-                DBG_LAUNCH_CK();
+                h_at[(pass == 2 ? kShapes : 0) + m * (kMaxBlock + 1) + n] = at;
                 if (pass == 0) at_q += cnt;
                 launches.push_back({m, n, cnt, pass == 2});
                 at += cnt;
@@ -1475,6 +1509,20 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                              use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, alpha, beta,
                              c_data.p, c_norm.p, c_dev2.p};
         }
+        if (at) {
+            list.alloc(at, s);
+            list_at.alloc(2 * kShapes, s);
+        }
+        // the stacks and lists of the FP64 pipe's blocks
+        auto fp64_lists = [&](cudaStream_t ls) {
+            if (!at) return;
+            fill_stacks(ls);
+            DBG_CK(cudaMemcpyAsync(list_at.p, h_at.data(), sizeof(int64_t) * 2 * kShapes, cudaMemcpyHostToDevice, ls));
+            k_shape_lists<<<grid_for(nform, kListThreads * kListItems), kListThreads, 0, ls>>>(
+                nform, f_row.p, f_col.p, A->bs.p, f_comp.p, plan && tc ? 2 : 1, (unsigned long long*)list_at.p, list.p);
+            DBG_LAUNCH_CK();
+        };
+        fp64_lists(s);
         DBG_CK(cudaEventRecord(ev.e[1], s));
         if (bf16) {
             lowtier_run(*lt, A, lto, s);

@@ -1016,13 +1016,21 @@ struct EventSet {
 // and 22.7.
 constexpr int kBesideTpb = 128;
 
-// A second stream beside a product's own, leased from a bounded pool: begin() makes it wait for what
-// the product's stream holds, join() makes that stream wait for it.  A lease that ends between the two
+// Streams beside a product's own, leased from a bounded pool: begin() makes them wait for what the
+// product's stream holds, join() makes that stream wait for them.  A lease that ends between the two
 // (an exception) joins first, so that no buffer is freed under its kernels.
-class SideStream {
+// Four of them: the launches of a product's shapes do not depend on one another, and a shape with few
+// blocks leaves most of the chip idle (a ragged matrix has one to thirty launches of a few blocks each).
+// With two streams, four and eight: 32 waters 1.07, 0.89 and 0.88 ms, a batch of twelve systems 65.9, 60.1
+// and 61.9, the ragged update 2.25, 2.22 and 2.40.
+class SideStreams {
+public:
+    static constexpr int kStreams = 4;
+
+private:
     struct Res {
-        cudaStream_t s = nullptr;
-        cudaEvent_t fork = nullptr, done = nullptr;
+        cudaStream_t s[kStreams] = {};
+        cudaEvent_t fork = nullptr, done[kStreams] = {};
     };
     static constexpr size_t kKept = 8;               // idle leases kept per device
     static std::mutex& mu() {
@@ -1034,17 +1042,18 @@ class SideStream {
         return *m;
     }
     static void destroy(Res& r) {
-        for (cudaEvent_t e : {r.fork, r.done})
+        if (r.fork) cudaEventDestroy(r.fork);
+        for (cudaEvent_t e : r.done)
             if (e) cudaEventDestroy(e);
-        if (r.s) cudaStreamDestroy(r.s);
+        for (cudaStream_t x : r.s)
+            if (x) cudaStreamDestroy(x);
     }
     Res r_;
-    int dev_ = 0;
+    int dev_ = 0, open_ = 0, next_ = 0;              // open_: streams between begin() and join()
     cudaStream_t main_ = nullptr;
-    bool open_ = false;
 
 public:
-    SideStream() {
+    SideStreams() {
         DBG_CK(cudaGetDevice(&dev_));
         {
             std::lock_guard<std::mutex> lk(mu());
@@ -1056,21 +1065,25 @@ public:
             }
         }
         try {
-            DBG_CK(cudaStreamCreateWithFlags(&r_.s, cudaStreamNonBlocking));
-            for (cudaEvent_t* e : {&r_.fork, &r_.done})
-                DBG_CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+            for (cudaStream_t& x : r_.s) DBG_CK(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
+            DBG_CK(cudaEventCreateWithFlags(&r_.fork, cudaEventDisableTiming));
+            for (cudaEvent_t& e : r_.done) DBG_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         } catch (...) {
             destroy(r_);
             throw;
         }
     }
-    SideStream(const SideStream&) = delete;
-    SideStream& operator=(const SideStream&) = delete;
-    ~SideStream() {
+    SideStreams(const SideStreams&) = delete;
+    SideStreams& operator=(const SideStreams&) = delete;
+    ~SideStreams() {
         bool keep = true;
-        if (open_) keep = cudaEventRecord(r_.done, r_.s) == cudaSuccess && cudaStreamWaitEvent(main_, r_.done, 0) == cudaSuccess;
-        cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
-        keep = keep && cudaStreamIsCapturing(r_.s, &cst) == cudaSuccess && cst == cudaStreamCaptureStatusNone;
+        for (int i = 0; i < open_; ++i)
+            keep = cudaEventRecord(r_.done[i], r_.s[i]) == cudaSuccess &&
+                   cudaStreamWaitEvent(main_, r_.done[i], 0) == cudaSuccess && keep;
+        for (cudaStream_t x : r_.s) {
+            cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+            keep = cudaStreamIsCapturing(x, &cst) == cudaSuccess && cst == cudaStreamCaptureStatusNone && keep;
+        }
         if (keep) {
             std::lock_guard<std::mutex> lk(mu());
             auto& v = idle()[dev_];
@@ -1081,17 +1094,22 @@ public:
         }
         destroy(r_);
     }
-    cudaStream_t stream() const { return r_.s; }
-    void begin(cudaStream_t main) {
+    // The streams in turn.
+    cudaStream_t stream() { return r_.s[next_++ % open_]; }
+    void begin(cudaStream_t main, size_t launches) {
         main_ = main;
         DBG_CK(cudaEventRecord(r_.fork, main));
-        DBG_CK(cudaStreamWaitEvent(r_.s, r_.fork, 0));
-        open_ = true;
+        while (open_ < kStreams && open_ < (int)launches) {
+            DBG_CK(cudaStreamWaitEvent(r_.s[open_], r_.fork, 0));
+            ++open_;
+        }
     }
     void join() {
-        DBG_CK(cudaEventRecord(r_.done, r_.s));
-        DBG_CK(cudaStreamWaitEvent(main_, r_.done, 0));
-        open_ = false;
+        while (open_ > 0) {
+            DBG_CK(cudaEventRecord(r_.done[open_ - 1], r_.s[open_ - 1]));
+            DBG_CK(cudaStreamWaitEvent(main_, r_.done[open_ - 1], 0));
+            --open_;
+        }
     }
 };
 
@@ -1455,6 +1473,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     SmmArgs sa{};
     struct ShapeLaunch { int m, n; int64_t cnt; bool fallback; };
     std::vector<ShapeLaunch> launches;
+    int n_simt = 0;                         // launches on the FP64 pipe that are not a plan's fallback
     std::unique_ptr<LowTierPlan, void (*)(LowTierPlan*)> lt(nullptr, lowtier_plan_delete);
     LowTierOut lto{};
     DBuf<int64_t> qcounter;                 // the work queue's counter (one-launch schedule)
@@ -1539,31 +1558,33 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             launches = std::move(rest);
             qcounter.alloc(1, s);
         }
+        for (const ShapeLaunch& L : launches) n_simt += L.fallback ? 0 : 1;
         if (tc) {
             lto = LowTierOut{f_rp.p, f_col.p, f_comp.p, f_off.p, use_c ? f_cin.p : nullptr,
                              use_c ? C->off.p : nullptr, use_c ? C->data.p : nullptr, alpha, beta,
                              c_data.p, c_norm.p, c_dev2.p};
             ++n_smm_launches;
         }
-        // The FP64 pipe's blocks run beside the tensor cores' on a second stream: k_oz hardly uses the
-        // FP64 pipe, and its registers are held down so that both fit an SM.  One after the other they
-        // took 13.9 and 28.4 ms on 512 waters (13/5, 23/7), side by side 11.4 and 22.6.
-        std::unique_ptr<SideStream> side;
-        cudaStream_t ss = s;
+        // The FP64 pipe's blocks run beside the tensor cores', on other streams: k_oz hardly uses the FP64
+        // pipe, and its registers are held down so that both fit an SM.  One after the other the two took
+        // 13.9 and 28.4 ms on 512 waters (13/5, 23/7), side by side 11.4 and 22.6.  With the shapes'
+        // launches side by side too (four streams): 10.9 and 22.1, and 0.78 -> 0.26 ms on 32 waters,
+        // where a shape alone does not fill the chip.
+        std::unique_ptr<SideStreams> side;
+        if (n_simt >= (tc ? 1 : 2)) {
+            side.reset(new SideStreams());
+            side->begin(s, n_simt);
+        }
         if (tc) {
-            if (!launches.empty() && !launches[0].fallback) {
-                side.reset(new SideStream());
-                side->begin(s);
-                ss = side->stream();
-            }
             f64tc_run(*tcp, lto, s);
             f64tc_norms(nform, f_comp.p, f_row.p, f_col.p, A->bs.p, f_off.p, c_data.p, c_norm.p, c_dev2.p, s);
         }
         at = 0;
         for (const ShapeLaunch& L : launches) {
             if (L.fallback) continue;
-            if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, ss);
-            else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, sa, smm_cfg(L.m, L.n, (bool)side), ss);
+            const cudaStream_t ls = side ? side->stream() : s;
+            if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, ls);
+            else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, sa, smm_cfg(L.m, L.n, tc), ls);
             at += L.cnt;
             if (!bf16) ++n_smm_launches;
         }
@@ -1623,7 +1644,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         }
         // captured on a private stream (the legacy default stream cannot be captured); the
         // graph is launched on C's stream
-        SideStream side;
+        SideStreams side;
         cudaStream_t cs = nullptr;
         DBG_CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
         cudaGraph_t graph = nullptr;
@@ -1635,13 +1656,14 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                 lowtier_run(*lt, A, lto, cs);
             }
             SmmArgs fb = sa;
-            const bool beside = tc && !launches.empty() && !launches[0].fallback;
+            const bool beside = n_simt >= (tc ? 1 : 2);
+            if (beside && !tc) side.begin(cs, n_simt);
             if (tc) {
                 // the tensor cores' blocks with the current values; the FP64 pipe repeats them all
                 // when these need it (f64tc_recheck)
                 f64tc_pack(*tcp, A, B, cs);
                 fb.gate = f64tc_recheck(*tcp, A, B, an.p, bn.p, nform, f64tc_blocks, f_pbeg.p, prod_a.p, prod_b.p, alpha, cs);
-                if (beside) side.begin(cs);
+                if (beside) side.begin(cs, n_simt);
                 f64tc_run(*tcp, lto, cs);
                 f64tc_norms(nform, f_comp.p, C->row.p, C->col.p, C->bs.p, C->off.p, C->data.p, C->norms.p, c_dev2.p, cs);
             }
@@ -1649,9 +1671,9 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             for (size_t i = 0; i < launches.size(); ++i) {
                 const ShapeLaunch& L = launches[i];
                 const bool b = beside && !L.fallback;
-                if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, b ? side.stream() : cs);
-                else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, L.fallback ? fb : sa, smm_cfg(L.m, L.n, b),
-                                      b ? side.stream() : cs);
+                const cudaStream_t ls = b ? side.stream() : cs;
+                if (L.m == 0) launch_smm_queue(L.cnt, list.p, sa, (unsigned long long*)qcounter.p, ls);
+                else launch_smm_shape(L.m, L.n, L.cnt, list.p + at, L.fallback ? fb : sa, smm_cfg(L.m, L.n, tc && b), ls);
                 at += L.cnt;
             }
             if (beside) side.join();

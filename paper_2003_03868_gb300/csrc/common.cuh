@@ -131,6 +131,16 @@ struct DBuf {
     }
 };
 
+// Arrays (multiples of 4 bytes) between the device and the host, on s: through a kernel where the host
+// side is pinned, else by a copy each.
+constexpr int kHostCopies = 3;
+struct HostCopy {
+    const void* src;
+    void* dst;
+    int64_t bytes;
+};
+void copy_with_host(const HostCopy* c, int n, bool to_host, cudaStream_t s);
+
 // Pinned host scratch for small device->host readbacks.
 struct HostScalars {
     static constexpr int kCap = 4096;

@@ -16,6 +16,9 @@
 #include <cstdio>
 #include <cstring>
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include "common.cuh"
 #include "dbcsr_gb_bench.h"
 
@@ -71,6 +74,88 @@ void allow_dyn_smem_of(const void* kernel, size_t dyn) {
     if (dyn <= now) return;
     DBG_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     now = dyn;
+}
+
+namespace {
+
+constexpr int kHostCopyThreads = 512;
+constexpr int64_t kHostCopyPiece = 1 << 16;          // bytes a CTA copies at a time
+
+struct HostCopyArgs {
+    HostCopy c[kHostCopies];
+    int n;
+};
+
+// Arrays to or from pinned host memory.  Both ends run at the link's rate (193 GB/s to the host), but the
+// first access to a host page after other work waits for its translation, and the copy engine takes
+// these waits one after another: 1.1 GB of a density matrix took 28 to 52 ms after a sign iteration
+// (5.6 when repeated), this kernel, with the accesses of 152 CTAs in flight, 5.6 to 8.5 ms.
+__global__ void __launch_bounds__(kHostCopyThreads) k_host_copy(HostCopyArgs A) {
+    for (int i = 0; i < A.n; ++i) {
+        const char* src = static_cast<const char*>(A.c[i].src);
+        char* dst = static_cast<char*>(A.c[i].dst);
+        const int64_t bytes = A.c[i].bytes;                           // a multiple of 4
+        const bool wide = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
+        for (int64_t p = (int64_t)blockIdx.x * kHostCopyPiece; p < bytes; p += (int64_t)gridDim.x * kHostCopyPiece) {
+            const int64_t e = min(p + kHostCopyPiece, bytes), ew = wide ? e & ~(int64_t)15 : p;
+            for (int64_t x = p + 16 * threadIdx.x; x < ew; x += 16 * kHostCopyThreads)
+                *reinterpret_cast<int4*>(dst + x) = *reinterpret_cast<const int4*>(src + x);
+            for (int64_t x = ew + 4 * threadIdx.x; x < e; x += 4 * kHostCopyThreads)
+                *reinterpret_cast<int*>(dst + x) = *reinterpret_cast<const int*>(src + x);
+        }
+    }
+}
+
+// The device's address of pinned host memory [p, p + bytes), or null: pageable, managed or device memory,
+// a range that leaves its allocation, or memory to be written that is not known to be writable.
+void* pinned_address(const void* p, int64_t bytes, bool write) {
+    static const PFN_cuPointerGetAttributes_v7000 get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        DBG_CK(cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &q));
+        return q == cudaDriverEntryPointSuccess ? reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(f) : nullptr;
+    }();
+    if (!get || bytes <= 0 || (reinterpret_cast<uintptr_t>(p) & 3)) return nullptr;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute at[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[] = {&type, &managed, &dev, &start, &size};
+    if (get(5, at, out, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || managed || !dev || !start || dev < start) return nullptr;
+    if (dev - start + (size_t)bytes > size) return nullptr;
+    unsigned flags = 0;
+    if (write && (cudaHostGetFlags(&flags, reinterpret_cast<void*>((uintptr_t)start)) != cudaSuccess ||
+                  (flags & cudaHostRegisterReadOnly))) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return reinterpret_cast<void*>((uintptr_t)dev);
+}
+
+}  // namespace
+
+void copy_with_host(const HostCopy* c, int n, bool to_host, cudaStream_t s) {
+    HostCopyArgs a{};
+    int64_t most = 0;
+    for (int i = 0; i < n; ++i) {
+        if (c[i].bytes <= 0) continue;
+        HostCopy k = c[i];
+        void* h = pinned_address(to_host ? k.dst : k.src, k.bytes, to_host);
+        if (!h || a.n == kHostCopies) {
+            DBG_CK(cudaMemcpyAsync(k.dst, k.src, (size_t)k.bytes, to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, s));
+            continue;
+        }
+        if (to_host) k.dst = h;
+        else k.src = h;
+        a.c[a.n++] = k;
+        most = std::max(most, k.bytes);
+    }
+    if (!a.n) return;
+    k_host_copy<<<grid_for(most, (int)kHostCopyPiece, num_sms()), kHostCopyThreads, 0, s>>>(a);
+    DBG_LAUNCH_CK();
 }
 
 void trim_pool(uint64_t keep_bytes) {
@@ -656,9 +741,10 @@ dbcsr_status dbcsr_put_values(dbcsr_matrix m, const double* data, int on_device)
     return guarded([&] {
         dbg::check_finalized(m);
         if (!data && m->nel) dbg::fail(DBCSR_EINVAL, "put_values: null data");
-        if (m->nel)
-            DBG_CK(cudaMemcpyAsync(m->data.p, data, sizeof(double) * m->nel,
-                                   on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, m->stream));
+        if (m->nel && on_device)
+            DBG_CK(cudaMemcpyAsync(m->data.p, data, sizeof(double) * m->nel, cudaMemcpyDeviceToDevice, m->stream));
+        const dbg::HostCopy c{data, m->data.p, (int64_t)sizeof(double) * m->nel};
+        if (!on_device) dbg::copy_with_host(&c, 1, false, m->stream);
         if (!on_device) DBG_CK(cudaStreamSynchronize(m->stream));
         m->exact_sym = false;
         m->norms_valid = false;
@@ -891,9 +977,12 @@ dbcsr_status dbcsr_export(dbcsr_matrix m, int64_t* row_ptr, int32_t* col, double
     return guarded([&] {
         dbg::check_finalized(m);
         cudaStream_t s = m->stream;
-        if (row_ptr) DBG_CK(cudaMemcpyAsync(row_ptr, m->rp.p, sizeof(int64_t) * (m->nblk + 1), cudaMemcpyDeviceToHost, s));
-        if (col && m->nnzb) DBG_CK(cudaMemcpyAsync(col, m->col.p, sizeof(int32_t) * m->nnzb, cudaMemcpyDeviceToHost, s));
-        if (data && m->nel) DBG_CK(cudaMemcpyAsync(data, m->data.p, sizeof(double) * m->nel, cudaMemcpyDeviceToHost, s));
+        dbg::HostCopy c[3];
+        int n = 0;
+        if (row_ptr) c[n++] = {m->rp.p, row_ptr, (int64_t)sizeof(int64_t) * (m->nblk + 1)};
+        if (col) c[n++] = {m->col.p, col, (int64_t)sizeof(int32_t) * m->nnzb};
+        if (data) c[n++] = {m->data.p, data, (int64_t)sizeof(double) * m->nel};
+        dbg::copy_with_host(c, n, true, s);
         DBG_CK(cudaStreamSynchronize(s));
     });
 }

@@ -43,34 +43,6 @@ __global__ void k_shift_i64(int64_t n, const int64_t* __restrict__ in, int64_t a
         out[i] = in[i] + add;
 }
 
-// Per-system Gershgorin bound: one thread per matrix row, max over the system's rows.
-__global__ void k_gershgorin_sys(int32_t nblk, const int32_t* __restrict__ bs, const int64_t* __restrict__ rp,
-                                 const int32_t* __restrict__ col, const int64_t* __restrict__ off,
-                                 const double* __restrict__ data, const int32_t* __restrict__ row_sys,
-                                 const double* __restrict__ mu, unsigned long long* __restrict__ maxbits) {
-    const int32_t I = blockIdx.x;
-    const int m = bs[I];
-    const int i = threadIdx.x;
-    if (i >= m) return;
-    const int32_t sys = row_sys[I];
-    const double shift = mu[sys];
-    double s = 0.0;
-    bool has_diag = false;
-    for (int64_t q = rp[I]; q < rp[I + 1]; ++q) {
-        const int32_t J = col[q];
-        const int n = bs[J];
-        const double* x = data + off[q] + (int64_t)i * n;
-        for (int j = 0; j < n; ++j) {
-            double v = x[j];
-            if (J == I && j == i) v -= shift;
-            s += fabs(v);
-        }
-        has_diag |= (J == I);
-    }
-    if (!has_diag) s += fabs(shift);
-    atomicMax(maxbits + sys, (unsigned long long)__double_as_longlong(s));
-}
-
 // X = (H - mu_s 1) / alpha_s, one warp per block.
 __global__ void k_scale_shift_sys(int64_t nb, const int32_t* __restrict__ row, const int32_t* __restrict__ col,
                                   const int32_t* __restrict__ bs, const int64_t* __restrict__ off,
@@ -225,9 +197,7 @@ dbcsr_status sign_iterate_batched(int32_t nsys, dbcsr_matrix_* const* H, const d
 
     // ---- per-system scale and X_0
     d_alpha.zero();
-    k_gershgorin_sys<<<nblk, kMaxBlock, 0, st>>>(nblk, HB->bs.p, HB->rp.p, HB->col.p, HB->off.p, HB->data.p, d_row_sys.p,
-                                                 d_mu.p, (unsigned long long*)d_alpha.p);
-    DBG_LAUNCH_CK();
+    gershgorin_sys(HB.get(), d_row_sys.p, d_mu.p, d_alpha.p, st);
     std::vector<double> alpha(nsys), scale(nsys), shift(nsys);
     DBG_CK(cudaMemcpyAsync(alpha.data(), d_alpha.p, sizeof(double) * nsys, cudaMemcpyDeviceToHost, st));
     DBG_CK(cudaStreamSynchronize(st));

@@ -247,6 +247,8 @@ void add(dbcsr_matrix_* A, double alpha, const dbcsr_matrix_* B, double beta);
 double trace(dbcsr_matrix_* m);
 double trace_product(dbcsr_matrix_* a, dbcsr_matrix_* b);
 double gershgorin(dbcsr_matrix_* m, double mu);
+// The bound of every system of a batch, added into bound[system] (zeroed by the caller) as a maximum.
+void gershgorin_sys(const dbcsr_matrix_* m, const int32_t* row_sys, const double* mu, double* bound, cudaStream_t s);
 // part[b] = <A_b, B_JI^T> for every block b = (I, J) of A (the first stage of trace_product).
 void trace_product_parts_into(dbcsr_matrix_* a, dbcsr_matrix_* b, double* part, cudaStream_t s);
 

@@ -389,7 +389,7 @@ dbcsr_status dbcsr_sign_iterate(dbcsr_matrix H, double mu, const dbcsr_sign_opts
  * P_out and rep as dbcsr_sign_iterate would (rep continues prev's histories and totals).
  * An FP64 iteration, and a mixed one resumed after its switch to FP64, take exactly the
  * products of the uninterrupted run: the resumed P equals its P bit for bit.  Resumed inside
- * a split-BF16 tier, the tensor-core tier regroups the blocks of X, so the products agree to
+ * a split-BF16 tier, whose groups of blocks are then made again from H, the products agree to
  * rounding.  X is not modified.  Errors: EINVAL (null arguments, block sizes of X or P_out
  * not those of H, a report with a negative or too long history); as dbcsr_sign_iterate.
  */
@@ -478,9 +478,9 @@ dbcsr_status dbcsr_sign_iterate_nonorth(dbcsr_matrix K, dbcsr_matrix S, double m
  *   multiple of 16 with an identity block; all submatrices of one padded size run as one
  *   batch of dense Newton-Schulz steps X <- 1.5 X - 0.5 X X^2 until every
  *   ||X^2 - 1||_F / n_pad < tol; P = (1 - X) / 2 on the taken blocks.
- * The dense products are strided-batched cuBLAS GEMMs.  opts: tol, max_iter, verbose;
- * prec DBCSR_FP64 (DGEMM) or DBCSR_MIXED (FP32: TF32 tensor-core GEMMs while the largest
- * residual is >= switch_tol, default 1e-3, then plain FP32 GEMMs; tol must then stay
+ * The dense products are the library's own (dbcsr_dense_multiply).  opts: tol, max_iter, verbose;
+ * prec DBCSR_FP64 or DBCSR_MIXED (FP32 storage: TF32 products while the largest
+ * residual is >= switch_tol, default 1e-3, then split TF32; tol must then stay
  * above the FP32 rounding floor, about 1e-6).  eps_filter is not used.  rep: iterations
  * (the most of any batch), residual (the largest), fp64_from = the first step after the
  * TF32 phase, n_products = submatrices, flops = dense GEMM flops, trace_p, e_band.

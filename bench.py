@@ -36,13 +36,12 @@ NOMINAL_BF16 = 2250.0
 NOMINAL_FP64 = 1.25
 FALLBACK_BF16_BURST, FALLBACK_BF16_SUSTAINED = 1900.0, 1700.0
 
-# DRAM bytes per flop of the FP64 block-product kernels: dram__bytes_read.sum +
-# dram__bytes_write.sum over three captured launches (7x7, 23x7 and 7x23 classes of one product
-# of the 512-water 23/7 case) divided by their executed DFMA flops (2 x
-# sm__sass_thread_inst_executed_op_dfma_pred_on.sum): 2.680 GB / 21.63 GFLOP.  A full launch's
-# traffic is this ratio times its flops (the larger systems are assumed to re-read operands at the
-# same rate per flop).  Reset to None whenever the kernel changes.
-SMM_F64_BYTES_PER_FLOP = 0.1239
+# DRAM bytes per flop of the FP64 block-product kernels from a capture; None: not captured since the
+# products moved to the tensor cores.
+SMM_F64_BYTES_PER_FLOP = None
+# BF16 digit products per FP64 product on the tensor cores (eight digits, the pairs of weight 0 to 7)
+DIGIT_PRODUCTS = 36
+F64_KERNELS = "k_oz beside k_smm_f64"
 
 
 def bf16_peak():
@@ -60,6 +59,14 @@ def hbm_peak():
         return float(json.load(open(PEAKS_FILE))["hbm_gbs"]), "measured copy"
     except Exception:
         return 6800.0, "fallback copy"
+
+
+def fp64_digit_roofline(achieved):
+    """The FP64 products against the tensor cores' rate for them: most run there as digit products, so
+    the fraction of the FP64 pipe's rate is above one."""
+    pk, src = bf16_peak()
+    return {"digit_peak": pk / DIGIT_PRODUCTS, "digit_frac": achieved * DIGIT_PRODUCTS / pk,
+            "digit_peak_source": f"{src} / {DIGIT_PRODUCTS} digit products"}
 
 
 def fp64_derived_peak():
@@ -850,16 +857,17 @@ def sign_leg(gb, torch, barrier, H, h, w, steps, warmup, prec, **kw):
 
 
 def fp64_roofline(acc, ms, steps, peak, peak_info):
-    """k_smm_f64 in a step: executed FP64 flops over the FP64 block-product kernels' own time
-    (CUDA events the library records around them on the launching stream)."""
+    """The FP64 block products in a step: their flops over their kernels' own time (CUDA events the
+    library records around them on the launching stream)."""
     f = acc["flops"] - acc["flops_low"]
     t = acc["ms_multiply"] - acc["ms_low"]
     nl = acc["launches_fp64"]
     achieved = f / (t * 1e-3) / 1e12 if t > 0 else 0.0
-    return {"bound": "fp64", "kernel": "k_smm_f64", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": achieved / peak,
+    return {"bound": "fp64", "kernel": F64_KERNELS, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak, **fp64_digit_roofline(achieved),
             "traffic": SMM_F64_BYTES_PER_FLOP * f / nl if SMM_F64_BYTES_PER_FLOP and nl else None,
-            "traffic_note": "DRAM bytes per launch: bytes per flop of a small-case capture x flops per launch",
+            "traffic_note": "DRAM bytes per launch: bytes per flop of a small-case capture x flops per launch, "
+                            "null where there is no capture",
             "kernel_share_of_step": t / ms if ms > 0 else None, "launches_per_step": nl / steps,
             "compulsory_bytes_per_launch": acc["bytes_min_fp64"] / nl if nl else None,
             "ms_per_step": t / steps, **peak_info}
@@ -1303,7 +1311,7 @@ def main():
     peak, peak_info = fp64_peak(gb, torch)
     achieved = flops / (ms_mult * 1e-3) / 1e12 if ms_mult > 0 else 0.0
     roofline = {"bound": "fp64", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "kernel": "k_smm_f64",
+                "frac": achieved / peak, "kernel": F64_KERNELS, **fp64_digit_roofline(achieved),
                 "traffic": (SMM_F64_BYTES_PER_FLOP * flops / smm_launches
                             if SMM_F64_BYTES_PER_FLOP and smm_launches else None),
                 "kernel_share_of_step": ms_mult / ms if ms > 0 else None,

@@ -751,9 +751,8 @@ dbcsr_status dbcsr_put_values(dbcsr_matrix m, const double* data, int on_device)
     });
 }
 
-// Every staged block is copied at once into a device staging pool (host sources
-// through one cudaMemcpyAsync, so pinned host buffers move by DMA); the host-side records of
-// the blocks are written while that copy runs.
+// Every staged block is copied at once into a device staging pool (pinned host sources by a
+// kernel, see k_host_copy); the host-side records of the blocks are written while that copy runs.
 static void stage(dbcsr_matrix m, int64_t n, const int32_t* rows, const int32_t* cols, const double* packed,
                   int on_device) {
     if (!m) fail(DBCSR_EINVAL, "null matrix handle");
@@ -790,9 +789,12 @@ static void stage(dbcsr_matrix m, int64_t n, const int32_t* rows, const int32_t*
                                    m->stream));
         m->st_dev = std::move(nb);
     }
-    if (total)
-        DBG_CK(cudaMemcpyAsync(m->st_dev.p + m->st_dev_used, packed, sizeof(double) * total,
-                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, m->stream));
+    double* const staged = m->st_dev.p + m->st_dev_used;
+    const int64_t bytes = (int64_t)sizeof(double) * total;
+    if (total && on_device)
+        DBG_CK(cudaMemcpyAsync(staged, packed, (size_t)bytes, cudaMemcpyDeviceToDevice, m->stream));
+    const dbg::HostCopy upload{packed, staged, bytes};
+    if (!on_device) dbg::copy_with_host(&upload, 1, false, m->stream);
     const size_t base = m->st_row.size();
     m->st_row.resize(base + n);
     m->st_col.resize(base + n);

@@ -57,6 +57,8 @@ def test_export_and_put_values(gb, kind, nblk):
         values.mul_(-3.0).add_(1.0)
         M.put_values(values.numpy())
         assert np.array_equal(M.export()[2], values.numpy())
+        new = gb.Matrix.from_blocks(M.blk_size, rp, col, values.numpy())     # staged from that buffer
+        assert np.array_equal(new.export()[2], values.numpy())
     finally:
         for _, _, keep in bufs:
             if keep:

@@ -345,11 +345,12 @@ struct F64TcBlocks {
 };
 void f64tc_delete(F64TcPlan* p);
 // Tile patterns, stacks and digit tiles of C = alpha A B and the blocks the tensor cores take;
-// null when the product does not fit them (then comp is not complete).
+// null when the product does not fit them (then comp is not complete).  planned: the tiles serve later
+// values of A and B too, so nothing is taken from the values these have now.
 std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A, dbcsr_matrix_* B,
                                                                std::shared_ptr<Groups> groups, int64_t nform,
                                                                const int64_t* f_rp, const F64TcBlocks& f, double alpha,
-                                                               cudaStream_t s);
+                                                               bool planned, cudaStream_t s);
 // The current values into the digit tiles (f64tc_prepare has done it for its values).
 void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s);
 // After f64tc_pack of a planned product's new values: the flag returned (device) becomes nonzero when

@@ -1042,7 +1042,7 @@ void oz_depth(F64TcPlan& L, cudaStream_t s) {
 std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A, dbcsr_matrix_* B,
                                                                std::shared_ptr<Groups> groups, int64_t nform,
                                                                const int64_t* f_rp, const F64TcBlocks& f, double alpha,
-                                                               cudaStream_t s) {
+                                                               bool planned, cudaStream_t s) {
     std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> P(nullptr, f64tc_delete);
     if (groups->ngrp > kMaxBlockRowsLt || !nform) return P;
     std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> up(new F64TcPlan(), f64tc_delete);
@@ -1053,8 +1053,9 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     L.R = (wmax + 7) & ~7;
     L.KS = (wmax + 15) / 16;
     L.nsl = (int)ceil_div(wmax, kSlice);
-    // B's K-major tiles are the tiles of its transpose: with B exactly symmetric those of B itself
-    L.b_sym = B->exact_sym;
+    // B's K-major tiles are the tiles of its transpose: with B exactly symmetric those of B itself (not in
+    // a planned product, whose later values need not be symmetric)
+    L.b_sym = B->exact_sym && !planned;
     L.b_is_a = A == B && L.b_sym;
     k_oz_role<<<grid_for(nform, 256), 256, 0, s>>>(nform, f.row, f.col, f.mirror, f.sym, g.g_of.p, f.by_group, f.comp);
     DBG_LAUNCH_CK();

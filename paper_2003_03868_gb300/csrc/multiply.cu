@@ -1417,7 +1417,8 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         if (tc) {
             // group tile patterns, digit tiles and the blocks the tensor cores take (f_comp = 2)
             tcp = f64tc_prepare(A, B, groups, nform, f_rp.p,
-                                F64TcBlocks{f_row.p, f_col.p, mirror.p, f_ksum.p, f_max.p, f_comp.p, sym_result, by_group}, alpha, s);
+                                F64TcBlocks{f_row.p, f_col.p, mirror.p, f_ksum.p, f_max.p, f_comp.p, sym_result, by_group}, alpha,
+                                plan != nullptr, s);
             tc = tcp != nullptr;
         }
         k_form_stats<<<grid_for(nform, 256, (int64_t)num_sms() * 8), 256, 0, s>>>(nform, f_row.p, f_col.p, f_np.p, f_ksum.p, mirror.p,

@@ -1,0 +1,74 @@
+"""FP64 products with operands that the library knows, or once knew, to be exactly symmetric: the tensor cores
+read such an operand's tiles as those of its transpose, so the knowledge must not outlive the values.
+
+Every block is compared with a plain FP64 product within twice what any sum of n rounded terms keeps (both
+sides are rounded): ||error|| <= 2 (n + 4) 2^-53 sum_K ||A_IK|| ||B_KJ||.  A transposed operand is wrong in
+the first digits."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+WATERS = 40
+
+
+@pytest.fixture(scope="module")
+def gb():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2003_03868_gb300 as m
+    m.lib()
+    return m
+
+
+@pytest.fixture(scope="module")
+def hamiltonian():
+    return synth.build_hamiltonian(synth.small(WATERS, seed=2100)).H
+
+
+def _dense(M):
+    rp, col, data = M.export()
+    bs = np.asarray(M.blk_size)
+    off = np.concatenate([[0], np.cumsum(bs)])
+    D, at = np.zeros((off[-1], off[-1])), 0
+    for i in range(len(bs)):
+        for j in col[rp[i]:rp[i + 1]]:
+            n = bs[i] * bs[j]
+            D[off[i]:off[i + 1], off[j]:off[j + 1]] = data[at:at + n].reshape(bs[i], bs[j])
+            at += n
+    return D
+
+
+def _check(M, A, B):
+    start = np.concatenate([[0], np.cumsum(M.blk_size)])[:-1]
+    a, b = _dense(A), _dense(B)
+    norms = lambda D: np.sqrt(np.add.reduceat(np.add.reduceat(D * D, start, 0), start, 1))  # noqa: E731
+    bound = 2 * (a.shape[0] + 4) * 2.0 ** -53 * (norms(a) @ norms(b))
+    assert np.all(norms(_dense(M) - a @ b) <= bound)
+
+
+def _flagged(gb, h):
+    """An exactly symmetric result of the library, and a copy of it."""
+    X = gb.sign_iterate(gb.Matrix.of(h), 0.0, 1e-7, 1e-9, max_iter=2, return_x=True).P
+    D = _dense(X)
+    assert np.array_equal(D, D.T)
+    return X
+
+
+@pytest.mark.parametrize("which", ["b", "both", "copy"])
+def test_plan_on_a_symmetric_result_takes_asymmetric_values(gb, hamiltonian, which):
+    X = _flagged(gb, hamiltonian)
+    B = X.copy() if which == "copy" else X
+    A = X if which == "both" else gb.Matrix.of(hamiltonian)
+    Cm = gb.Matrix(X.blk_size, X.stream)
+    plan = gb.Plan(1.0, A, B, Cm, 0.0)
+    assert plan.stats.n_tiles > 0
+    _check(Cm, A, B)
+    rng = np.random.default_rng(21)
+    for _ in range(2):
+        B.put_values(rng.uniform(-1.0, 1.0, len(B.export()[2])))
+        plan.execute()
+        _check(Cm, A, B)
+    plan.close()

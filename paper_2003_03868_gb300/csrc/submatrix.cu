@@ -396,7 +396,9 @@ dbcsr_status submatrix_sign(dbcsr_matrix_* H, double mu, const dbcsr_sign_opts* 
             nsub += (int64_t)ck.sub_j.size();
         }
     }
+    // (P's flags were H's; its columns come from different submatrices: nothing makes it exactly symmetric)
     P->norms_valid = false;
+    P->exact_sym = false;
     r.trace_p = trace(P);
     r.e_band = trace_product(P, H);
     DBG_CK(cudaStreamSynchronize(s));

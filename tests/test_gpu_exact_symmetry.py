@@ -72,3 +72,15 @@ def test_plan_on_a_symmetric_result_takes_asymmetric_values(gb, hamiltonian, whi
         plan.execute()
         _check(Cm, A, B)
     plan.close()
+
+
+def test_submatrix_result_of_a_symmetric_matrix(gb, hamiltonian):
+    # P takes its pattern from a matrix that is exactly symmetric, but is not symmetric itself
+    X = _flagged(gb, hamiltonian)
+    P = gb.submatrix_sign(X, 0.0, 1e-6, max_iter=40).P
+    D = _dense(P)
+    assert np.abs(D - D.T).max() > 1e-9
+    K = gb.Matrix.of(hamiltonian)
+    Cm = gb.Matrix(X.blk_size, X.stream)
+    assert gb.multiply(1.0, K, P, 0.0, Cm, 0.0).n_tiles > 0
+    _check(Cm, K, P)

@@ -311,6 +311,7 @@ dbcsr_status sign_iterate_batched(int32_t nsys, dbcsr_matrix_* const* H, const d
             pm->nnzb = nbk;
             pm->nel = nel_s;
             pm->norms_valid = false;
+            pm->exact_sym = X->exact_sym;        // (not that of what P held before)
             pm->finalized = true;
             // X of a mixed run with a plain BF16 tier is symmetric only to that tier's accuracy: keep
             // its symmetric part (mirrored products keep X exactly symmetric)

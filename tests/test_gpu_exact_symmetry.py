@@ -4,6 +4,8 @@ read such an operand's tiles as those of its transpose, so the knowledge must no
 Every block is compared with a plain FP64 product within twice what any sum of n rounded terms keeps (both
 sides are rounded): ||error|| <= 2 (n + 4) 2^-53 sum_K ||A_IK|| ||B_KJ||.  A transposed operand is wrong in
 the first digits."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -84,3 +86,19 @@ def test_submatrix_result_of_a_symmetric_matrix(gb, hamiltonian):
     Cm = gb.Matrix(X.blk_size, X.stream)
     assert gb.multiply(1.0, K, P, 0.0, Cm, 0.0).n_tiles > 0
     _check(Cm, K, P)
+
+
+def test_batch_into_handles_that_held_symmetric_results(gb, hamiltonian):
+    # full products keep both triangles as computed: the filtered X is symmetric only up to its last bits
+    H = gb.Matrix.of(hamiltonian)
+    P = _flagged(gb, hamiltonian)
+    mu = np.zeros(1)
+    o = gb.SignOpts(1e-4, 1e-9, 3, gb.DBCSR_FP64, 1e-4, 0.5, 0, gb._ffi.DBCSR_SIGN_FULL_PRODUCTS, 2, 0)
+    st = gb.lib().dbcsr_sign_iterate_batched(1, (C.c_void_p * 1)(H.handle.value), C.c_void_p(mu.ctypes.data), C.byref(o),
+                                             (C.c_void_p * 1)(P.handle.value), (gb.SignReport * 1)())
+    assert st in (gb._ffi.DBCSR_OK, gb._ffi.DBCSR_ENOTCONV)
+    D = _dense(P)
+    assert np.abs(D - D.T).max() > 1e-9
+    Cm = gb.Matrix(P.blk_size, P.stream)
+    assert gb.multiply(1.0, H, P, 0.0, Cm, 0.0).n_tiles > 0
+    _check(Cm, H, P)

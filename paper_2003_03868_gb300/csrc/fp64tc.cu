@@ -270,8 +270,11 @@ __global__ void k_oz_guard(OzGuardArgs A) {
         for (int64_t e = e0; e < e1; ++e)
             E = max(E, (int)A.a_mexp[(int64_t)A.st_a[e] * kGroupMembers + a] +
                            (int)A.b_mexp[(int64_t)A.st_b[e] * kGroupMembers + b]);
-        // (a norm product past FP32's range says nothing: FP64 pipe)
-        if (E > kNoExp / 2 && !(ldexpf(A.abs_alpha, E - 8) < A.f_max[k] && A.f_max[k] <= 3e38f)) continue;
+        // (a norm product near the ends of FP32's range, or past them, says nothing: FP64 pipe; below, it is
+        // rounded up to a denormal while the scales' product underflows to 0)
+        if (E > kNoExp / 2 &&
+            !(ldexpf(A.abs_alpha, E - 8) < A.f_max[k] && A.f_max[k] >= 1e-30f && A.f_max[k] <= 3e38f))
+            continue;
         A.comp[k] = 2;
         A.c_tbl[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int32_t)k;
         A.c_exp[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int16_t)max(E, -4096);

@@ -220,3 +220,18 @@ def test_both_pipes_side_by_side_from_several_threads_and_streams(gb, planned):
     for t in ts:
         t.join()
     assert not bad
+
+
+@pytest.mark.parametrize("power", [-110, -75, 60, 80])
+def test_badly_scaled_blocks_of_tiny_and_huge_operands(gb, power):
+    # the norm products lie near the ends of FP32's range and past them, where the choice of the blocks
+    # for the tensor cores is made
+    bs = [13, 5, 5] * 20
+    a = _scaled(synth.random_block_matrix(bs, 0.9, 1520), 8.0, 5)
+    b = _scaled(synth.random_block_matrix(bs, 0.9, 1521), 8.0, 6)
+    a.data *= 2.0 ** power
+    b.data *= 2.0 ** power
+    A, B = gb.Matrix.of(a), gb.Matrix.of(b)
+    C = gb.Matrix(A.blk_size, A.stream)
+    gb.multiply(1.0, A, B, 0.0, C, 0.0)
+    _check(C, bsr.Mat.of(a), bsr.Mat.of(b))

@@ -165,15 +165,21 @@ __global__ void __launch_bounds__(256) k_oz_pack(OzPackArgs P) {
             if (a == 255) continue;
             unsigned m = 0;
 #pragma unroll
-            for (int x = 0; x < 8; ++x) m = max(m, (unsigned)(load(r, a, 8 * c + x) >> 52) & 0x7ffu);
+            for (int x = 0; x < 8; ++x) {
+                const uint64_t b = load(r, a, 8 * c + x);
+                m = max(m, 2u * ((unsigned)(b >> 52) & 0x7ffu) + ((b << 1) != 0u ? 1u : 0u));
+            }
             if (m) atomicMax(&rmax[r], (int)m);
         }
         __syncthreads();
         if (tid < P.R) {
-            const int m = rmax[tid];
-            if (m && (m > 1023 + kExpLimit || m < 1023 - kExpLimit)) atomicExch(P.bad, 1);
+            // (a row of subnormals alone, m = 0 with a nonzero element, is outside the range as well)
+            const int any = rmax[tid] & 1, m = rmax[tid] >> 1;
+            if (any && (m > 1023 + kExpLimit || m < 1023 - kExpLimit)) atomicExch(P.bad, 1);
+            rmax[tid] = m;
             P.rexp[t * P.R + tid] = (int16_t)(m ? m - 1022 : 0);
         }
+        __syncthreads();
         if (tid < kGroupMembers) {
             int m = 0;
             if (tid < nm)

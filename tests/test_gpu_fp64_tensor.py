@@ -235,3 +235,17 @@ def test_badly_scaled_blocks_of_tiny_and_huge_operands(gb, power):
     C = gb.Matrix(A.blk_size, A.stream)
     gb.multiply(1.0, A, B, 0.0, C, 0.0)
     _check(C, bsr.Mat.of(a), bsr.Mat.of(b))
+
+
+def test_rows_of_subnormals(gb):
+    # a block row that holds nothing but subnormals, times large elements: no element of the product is small
+    bs = [23, 7, 7] * 10
+    a = synth.random_block_matrix(bs, 0.9, 1620)
+    b = synth.random_block_matrix(bs, 0.9, 1621)
+    n = a.blk_off()[a.row_ptr[1]]
+    a.data[:n] = np.ldexp(np.rint(a.data[:n] * 2.0 ** 20), -1070)
+    b.data *= 2.0 ** 398
+    A, B = gb.Matrix.of(a), gb.Matrix.of(b)
+    C = gb.Matrix(A.blk_size, A.stream)
+    gb.multiply(1.0, A, B, 0.0, C, 0.0)
+    _check(C, bsr.Mat.of(a), bsr.Mat.of(b))

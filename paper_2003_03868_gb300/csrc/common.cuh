@@ -340,6 +340,7 @@ double lowtier_copy_bytes(const LowTierPlan& L);
 struct F64TcBlocks {
     const int32_t* row; const int32_t* col; const int64_t* mirror; const int32_t* ksum;
     const float* max_term;               // largest |alpha| ||A_IK|| ||B_KJ|| of every block
+    const int32_t* max_at;               // and which block of A's row I it is
     uint8_t* comp;                       // out: 0 copied or dropped, 1 FP64 pipe, 2 tensor cores
     int sym, by_group;                   // as block_role's
 };

@@ -18,14 +18,20 @@
 //     sum per element, all in integers.  The sum is rounded to FP64 once, at the end: no FP64
 //     operation per term is left.
 //
-// Accuracy: against an FP64 chain the error of a product is smaller (relative Frobenius error of
-// H H on water with 13/5 blocks 2.2e-16 against 2.3e-15, of X X in the middle of the sign
-// iteration 1.6e-16 against 1.3e-15).  Only where a C block's terms are all far below the product
-// of the tile rows' maxima (A strong in one atom of the tile, B in another) would the common
-// scale cost bits: k_oz_guard finds those blocks (largest scale product at least 2^8 times the
-// largest norm product, from which on the two errors were equal or the tile's larger) and leaves
-// them to the FP64 pipe, as it does with the blocks of tiles too empty to pay, and with every
-// block when an operand holds a value that is not finite or too large or small for the scales.
+// Accuracy: over whole products the error is smaller than an FP64 chain's (relative Frobenius error of
+// H H on water with 13/5 blocks 2.2e-16 against 2.3e-15, of X X in the middle of the sign iteration
+// 1.6e-16 against 1.3e-15).  Element by element it is about 2^-61 of the largest scale product 2^E of the
+// C block's tile rows, whatever the element's own terms are (nearly all of it the pairs s + t = 8 that are left
+// out), while the chain's goes with sum_k |a_ik| |b_kj|.  A block whose terms are far below 2^E (A strong in one
+// atom of the tile, B in another), or weak in one of its elements (a row graded against its neighbours, an element
+// beside a larger one that meets a zero), would lose bits.  k_oz_guard and k_oz_weak leave such blocks to
+// the FP64 pipe: a block runs here only if its largest norm product is above 2^(E - 7) and if the block
+// product that gives it, taken of the absolute values, is at least 2^(E - 13) in every element.  Digits
+// against chain (emulated; root mean square over elements, in units of 2^-53 sum_k |a_ik| |b_kj|), blocks whose
+// weakest element lies at 2^-12 to 2^-13: H H with 13/5 blocks 1.7 against 1.9, with 23/7 2.8 against 2.6, X X
+// 0.8 against 1.4 and 1.4 against 1.8; at 2^-13 to 2^-14 up to 5 against 3.  All blocks: 0.3 to 0.9 against
+// 1.4 to 2.6.  The FP64 pipe also takes the blocks of tiles too empty to pay, and every block when an operand
+// holds a value that is not finite or too large or small for the scales.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -245,33 +251,43 @@ struct OzGuardArgs {
     const int64_t* s_ptr; const int32_t* st_a; const int32_t* st_b;
     const int16_t* a_mexp; const int16_t* b_mexp;
     const float* f_max;                              // largest |alpha| ||A_IK|| ||B_KJ|| of every block
+    const int32_t* f_at;                             // and which block of A's row I that is
     const unsigned long long* tile_flops;
     float abs_alpha;
     const int* bad;
+    int16_t* f_exp;                                  // k_oz_guard to k_oz_weak: exponent of the block's scale
     uint8_t* comp;
     int32_t* c_tbl; int16_t* c_exp; unsigned* c_slices;
     const int32_t* g_pos; const int32_t* bs;
+    const int64_t* a_rp; const int32_t* a_col; const int64_t* a_off; const double* a_data;
+    const int64_t* b_rp; const int32_t* b_col; const int64_t* b_off; const double* b_data;
 };
 
 // A computed block runs on the tensor cores (comp = 2) unless
 //   * its tile's tensor-core time (every stack entry at full width; a rule on the tile alone, so
 //     a block takes the same path in any batch) is above the FP64 pipe's time for its blocks;
-//   * the largest product of its tile rows' scales, max 2^(e_a + e_b), is at least 2^8 times its
-//     largest norm product: below that ratio the tile's error is smaller than the FP64 chain's
-//     (ratio 2^4: 0.2 of it, 2^7: 0.7, 2^8: 1.4, medians over water products), above it larger;
+//   * the largest product of its tile rows' scales, max 2^(e_a + e_b), is at least 2^7 times its
+//     largest norm product (Frobenius error of a block in units of the FP64 chain's, root mean square over
+//     water products, emulated: 0.1 below 2^4, 0.4 to 0.9 at 2^6 to 2^7, 0.7 to 1.5 above, 1.7 at 2^8);
+//   * its weakest element is too far below those scales (k_oz_weak);
 //   * an operand holds a value outside the scales' range.
+// The blocks that both rules send back cost the FP64 pipe's rate: the sign iteration on 512 waters takes
+// 245 ms with them, 204 with 2^8 and no rule on elements, 222 with 2^8 and 2^-14, 239 with 2^8 and 2^-13.
+constexpr float kNormRatio = 0.0078125f;             // 2^-7
+constexpr int kWeakBits = 13;
+constexpr int kNoTerm = -4096;                       // exponent of a block all of whose products are zero
 __global__ void k_oz_guard(OzGuardArgs A) {
-    if (*A.bad) return;
+    const bool bad = *A.bad != 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < A.nform; k += (int64_t)gridDim.x * blockDim.x) {
+        A.f_exp[k] = kNoExp;                          // FP64 pipe
         const int32_t t = A.blk_tile[k];
-        if (t < 0) continue;
+        if (bad || t < 0) continue;
         const int64_t e0 = A.s_ptr[t], e1 = A.s_ptr[t + 1];
         const int wc = A.g_w[A.c_tcol[t]];
         const int slices = (wc + kSlice - 1) / kSlice;
         const double clocks = (double)(e1 - e0) * (kGroupWidth / 16) * slices * kStepClocks;
         if (clocks * kSimtFlopsPerClock > (double)A.tile_flops[t]) continue;
-        const int32_t I = A.f_row[k], J = A.f_col[k];
-        const int a = A.g_midx[I], b = A.g_midx[J];
+        const int a = A.g_midx[A.f_row[k]], b = A.g_midx[A.f_col[k]];
         int E = 2 * kNoExp;
         for (int64_t e = e0; e < e1; ++e)
             E = max(E, (int)A.a_mexp[(int64_t)A.st_a[e] * kGroupMembers + a] +
@@ -279,14 +295,81 @@ __global__ void k_oz_guard(OzGuardArgs A) {
         // (a norm product near the ends of FP32's range, or past them, says nothing: FP64 pipe; below, it is
         // rounded up to a denormal while the scales' product underflows to 0)
         if (E > kNoExp / 2 &&
-            !(ldexpf(A.abs_alpha, E - 8) < A.f_max[k] && A.f_max[k] >= 1e-30f && A.f_max[k] <= 3e38f))
+            !(ldexpf(A.abs_alpha, E) * kNormRatio < A.f_max[k] && A.f_max[k] >= 1e-30f && A.f_max[k] <= 3e38f))
             continue;
-        A.comp[k] = 2;
-        A.c_tbl[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int32_t)k;
-        A.c_exp[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int16_t)max(E, -4096);
-        unsigned m = 0;
-        for (int q = A.g_pos[J] / kSlice; q <= (A.g_pos[J] + A.bs[J] - 1) / kSlice; ++q) m |= 1u << q;
-        atomicOr(A.c_slices + t, m);
+        A.f_exp[k] = (int16_t)max(E, kNoTerm);
+    }
+}
+
+// n elements of a block as floats |x| 2^-e, e the exponent above the largest (returned), cut to 21 bits: by
+// the high words, since the FP64 pipe converts a few values per clock and SM.
+__device__ __forceinline__ int oz_abs(const double* __restrict__ x, int n, int lane, float* out) {
+    unsigned mx = 0;
+    for (int e = lane; e < n; e += 32) {
+        const unsigned hi = __ldg(reinterpret_cast<const unsigned*>(x + e) + 1) & 0x7fffffffu;
+        out[e] = __uint_as_float(hi);
+        mx = max(mx, hi >> 20);
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    for (int e = lane; e < n; e += 32) {              // (each lane its own elements)
+        const int v = (int)__float_as_uint(out[e]) - (((int)mx - 126) << 20);
+        out[e] = v >= (1 << 20) ? __int_as_float(v << 3) : 0.f;
+    }
+    return (int)mx - 1022;
+}
+
+// Whether every element of |A_IK| |B_KJ| is at least 2^(E - bits) (one warp; sh: two blocks).
+__device__ __forceinline__ bool oz_no_weak(const double* a, const double* b, int m, int kk, int n, int E, int bits,
+                                           int lane, float (*sh)[kMaxBlock * kMaxBlock]) {
+    __syncwarp();                                     // the last block's elements are read
+    const int ea = oz_abs(a, m * kk, lane, sh[0]), eb = oz_abs(b, kk * n, lane, sh[1]);
+    __syncwarp();
+    float low = 3e38f;
+    for (int e = lane; e < m * n; e += 32) {
+        const int i = e / n, j = e - i * n;
+        float s = 0.f;
+        for (int t = 0; t < kk; ++t) s = fmaf(sh[0][i * kk + t], sh[1][t * n + j], s);
+        low = fminf(low, s);
+    }
+    low = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(low)));
+    const int x = E - bits - ea - eb;                 // at least -bits: 2^E is a scale product of the same rows
+    return x < 100 && low >= ldexpf(1.f, x);
+}
+
+// The blocks that k_oz_guard lets through, one warp each: their strongest block product without signs is a
+// lower bound of sum_k |a_ik| |b_kj| for every element, 8 times below it on water in the median.  Bound by the
+// loads of the two operand blocks and 2 m n k / 32 shared-memory reads a block.
+constexpr int kWeakWarps = 4;
+__global__ void __launch_bounds__(32 * kWeakWarps) k_oz_weak(OzGuardArgs A) {
+    __shared__ float sh[kWeakWarps][2][kMaxBlock * kMaxBlock];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t k = (int64_t)blockIdx.x * kWeakWarps + warp; k < A.nform; k += (int64_t)gridDim.x * kWeakWarps) {
+        const int E = A.f_exp[k];
+        if (E == kNoExp) continue;
+        const int32_t t = A.blk_tile[k], I = A.f_row[k], J = A.f_col[k];
+        if (E > kNoTerm) {
+            const int64_t p = A.a_rp[I] + A.f_at[k];
+            const int32_t K = A.a_col[p];
+            int64_t lo = A.b_rp[K], hi = A.b_rp[K + 1];
+            const int64_t end = hi;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (A.b_col[mid] < J) lo = mid + 1; else hi = mid;
+            }
+            if (!(lo < end && A.b_col[lo] == J)) continue;
+            if (!oz_no_weak(A.a_data + A.a_off[p], A.b_data + A.b_off[lo], A.bs[I], A.bs[K], A.bs[J], E, kWeakBits, lane,
+                            sh[warp]))
+                continue;
+        }
+        if (lane == 0) {
+            const int64_t at = (int64_t)t * (kGroupMembers * kGroupMembers) + A.g_midx[I] * kGroupMembers + A.g_midx[J];
+            A.comp[k] = 2;
+            A.c_tbl[at] = (int32_t)k;
+            A.c_exp[at] = (int16_t)E;
+            unsigned m = 0;
+            for (int q = A.g_pos[J] / kSlice; q <= (A.g_pos[J] + A.bs[J] - 1) / kSlice; ++q) m |= 1u << q;
+            atomicOr(A.c_slices + t, m);
+        }
     }
 }
 
@@ -1142,10 +1225,15 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     k_oz_tile_flops<<<grid_for(nform, 256), 256, 0, s>>>(nform, L.cp.blk_tile.p, f.row, f.col, f.ksum, A->bs.p,
                                                          L.tile_flops.p);
     DBG_LAUNCH_CK();
+    DBuf<int16_t> f_exp;
+    f_exp.alloc(nform, s);
     OzGuardArgs ga{nform, L.cp.blk_tile.p, f.row, f.col, g.g_midx.p, g.g_w.p, L.cp.t_col.p, L.s_ptr.p, L.st_a.p, L.st_b.p,
-                   L.a.mexp.p, b.mexp.p, f.max_term, L.tile_flops.p, (float)std::fabs(alpha), L.flags.p + 1, f.comp,
-                   L.c_tbl.p, L.c_exp.p, L.c_slices.p, g.g_pos.p, A->bs.p};
+                   L.a.mexp.p, b.mexp.p, f.max_term, f.max_at, L.tile_flops.p, (float)std::fabs(alpha), L.flags.p + 1,
+                   f_exp.p, f.comp, L.c_tbl.p, L.c_exp.p, L.c_slices.p, g.g_pos.p, A->bs.p,
+                   A->rp.p, A->col.p, A->off.p, A->data.p, B->rp.p, B->col.p, B->off.p, B->data.p};
     k_oz_guard<<<grid_for(nform, 256), 256, 0, s>>>(ga);
+    DBG_LAUNCH_CK();
+    k_oz_weak<<<grid_for(nform, kWeakWarps, (int64_t)num_sms() * 64), 32 * kWeakWarps, 0, s>>>(ga);
     DBG_LAUNCH_CK();
     oz_depth(L, s);
     return up;
@@ -1159,31 +1247,54 @@ void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cu
 
 namespace {
 
-// A planned product's new values: one warp per tensor-core block, its largest norm product over
-// its stack against its tile rows' scales, as in k_oz_guard with one more bit of room.
-__global__ void k_oz_recheck(OzGuardArgs A, const int64_t* __restrict__ pbeg, const int32_t* __restrict__ prod_a,
-                             const int32_t* __restrict__ prod_b, const double* __restrict__ an,
-                             const double* __restrict__ bn, int* __restrict__ bad) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < A.nform; k += warps) {
+// A planned product's new values: one warp per tensor-core block, the tests of k_oz_guard and k_oz_weak on
+// its stack, with one more bit of room.
+__global__ void __launch_bounds__(32 * kWeakWarps) k_oz_recheck(OzGuardArgs A, const int64_t* __restrict__ pbeg,
+                                                                const int32_t* __restrict__ prod_a,
+                                                                const int32_t* __restrict__ prod_b,
+                                                                const double* __restrict__ an,
+                                                                const double* __restrict__ bn, int* __restrict__ bad) {
+    __shared__ float sh[kWeakWarps][2][kMaxBlock * kMaxBlock];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t k = (int64_t)blockIdx.x * kWeakWarps + warp; k < A.nform; k += (int64_t)gridDim.x * kWeakWarps) {
         if (A.comp[k] != 2) continue;
-        const int32_t t = A.blk_tile[k];
-        const int a = A.g_midx[A.f_row[k]], b = A.g_midx[A.f_col[k]];
+        const int32_t t = A.blk_tile[k], I = A.f_row[k], J = A.f_col[k];
+        const int a = A.g_midx[I], b = A.g_midx[J];
         int E = 2 * kNoExp;
         for (int64_t e = A.s_ptr[t] + lane; e < A.s_ptr[t + 1]; e += 32)
             E = max(E, (int)A.a_mexp[(int64_t)A.st_a[e] * kGroupMembers + a] +
                            (int)A.b_mexp[(int64_t)A.st_b[e] * kGroupMembers + b]);
+        E = __reduce_max_sync(0xffffffffu, E);
         double mx = 0.0;
-        for (int64_t p = pbeg[k] + lane; p < pbeg[k + 1]; p += 32) mx = fmax(mx, an[prod_a[p]] * bn[prod_b[p]]);
+        int64_t at = -1;                              // the strongest block product (of equal ones any)
+        for (int64_t p = pbeg[k] + lane; p < pbeg[k + 1]; p += 32) {
+            const double v = an[prod_a[p]] * bn[prod_b[p]];
+            if (v > mx) {
+                mx = v;
+                at = p;
+            }
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const double omx = __shfl_xor_sync(0xffffffffu, mx, o);
+            const int64_t oat = __shfl_xor_sync(0xffffffffu, at, o);
+            if (omx > mx || (omx == mx && oat > at)) {
+                mx = omx;
+                at = oat;
+            }
+        }
+        bool ok = true;
+        if (E > kNoExp / 2) {
+            ok = at >= 0 && ldexp((double)kNormRatio, E - 1) < mx && mx <= 1e300;
+            if (ok) {
+                const int32_t p = prod_a[at], q = prod_b[at];
+                ok = oz_no_weak(A.a_data + A.a_off[p], A.b_data + A.b_off[q], A.bs[I], A.bs[A.a_col[p]], A.bs[J], E,
+                                kWeakBits + 1, lane, sh[warp]);
+            }
         }
         if (lane == 0) {
-            A.c_exp[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int16_t)max(E, -4096);
-            if (E > kNoExp / 2 && !(ldexp(1.0, E - 9) < mx && mx <= 1e300)) atomicExch(bad, 1);
+            A.c_exp[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int16_t)max(E, kNoTerm);
+            if (!ok) atomicExch(bad, 1);
         }
     }
 }
@@ -1202,9 +1313,10 @@ const int* f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matri
         bnp = bn;
     }
     OzGuardArgs ga{nform, L.cp.blk_tile.p, f.row, f.col, g.g_midx.p, g.g_w.p, L.cp.t_col.p, L.s_ptr.p, L.st_a.p, L.st_b.p,
-                   L.a.mexp.p, b.mexp.p, nullptr, L.tile_flops.p, (float)std::fabs(alpha), nullptr, f.comp,
-                   L.c_tbl.p, L.c_exp.p, nullptr, g.g_pos.p, A->bs.p};
-    k_oz_recheck<<<grid_for(nform, 8), 256, 0, s>>>(ga, f_pbeg, prod_a, prod_b, an, bnp, L.flags.p + 1);
+                   L.a.mexp.p, b.mexp.p, nullptr, nullptr, L.tile_flops.p, (float)std::fabs(alpha), nullptr, nullptr, f.comp,
+                   L.c_tbl.p, L.c_exp.p, nullptr, g.g_pos.p, A->bs.p,
+                   A->rp.p, A->col.p, A->off.p, A->data.p, B->rp.p, B->col.p, B->off.p, B->data.p};
+    k_oz_recheck<<<grid_for(nform, kWeakWarps, (int64_t)num_sms() * 64), 32 * kWeakWarps, 0, s>>>(ga, f_pbeg, prod_a, prod_b, an, bnp, L.flags.p + 1);
     DBG_LAUNCH_CK();
     oz_depth(L, s);
     return L.flags.p + 1;

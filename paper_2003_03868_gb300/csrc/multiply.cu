@@ -148,6 +148,7 @@ struct BoundArgs {
     int use_fast;            // FP32 upper bound with atomics (needs use_smem and < 4096 terms per candidate)
     const float* b_norm_ru;  // use_fast: B's norms rounded up to FP32, once per block
     float* max_term;         // per candidate (nullable): its largest |alpha| ||A_IK|| ||B_KJ||
+    int32_t* max_at;         // with max_term: which block of A's row I that is
     unsigned long long* flops;   // sum of 2 m n k over the kept candidates
 };
 
@@ -176,8 +177,8 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
         const int nc = build_row(P, I, bm, wpre, nwords, sh_scan);
         const int64_t cb = B.coff[I];
         // per candidate in shared memory: use_fast the FP32 bound, the packed counters (terms,
-        // below 4096, in the low 12 bits, the sum of k above) and the largest term, 12 bytes;
-        // otherwise the FP64 bound, the two counters and the largest term
+        // below 4096, in the low 12 bits, the sum of k above) and the largest term (its place in the
+        // low 12 bits), 12 bytes; otherwise the FP64 bound, the two counters, the largest term and its place
         double* bnd = B.use_smem ? sh_bound : B.bound + cb;
         int32_t* pc = B.use_smem ? (int32_t*)(sh_bound + nc) : B.pcnt + cb;
         int32_t* ks = B.use_smem ? pc + nc : B.ksum + cb;
@@ -185,6 +186,7 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
         unsigned* pk = (unsigned*)(fb + nc);
         float* mx = B.use_fast ? (float*)(pk + nc) : B.use_smem ? (float*)(ks + nc) : B.max_term + cb;
         const bool want_max = B.max_term != nullptr;
+        int32_t* at = B.use_fast ? nullptr : B.use_smem ? (int32_t*)(mx + nc) : B.max_at + cb;
         // candidates in ascending J
         for (int w = threadIdx.x; w < nwords; w += blockDim.x) {
             uint32_t bits = bm[w];
@@ -202,7 +204,10 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
                     pc[r] = 0;
                     ks[r] = 0;
                 }
-                if (want_max) mx[r] = 0.f;
+                if (want_max) {
+                    mx[r] = 0.f;
+                    if (at) at[r] = 0;
+                }
                 if (B.cin) B.cin[cb + r] = -1;
                 ++r;
             }
@@ -224,7 +229,8 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
                     const float term = na == 0.f || nb == 0.f ? 0.f : __fmul_ru(na, nb);
                     atomicAdd(&fb[r], term);
                     atomicAdd(&pk[r], kk);
-                    if (want_max) atomicMax((int*)&mx[r], __float_as_int(term));
+                    if (want_max)
+                        atomicMax((int*)&mx[r], (__float_as_int(term) & ~4095) | (int)(p - P.a_rp[I]));
                 }
             }
         } else {
@@ -240,7 +246,10 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
                     bnd[r] = bnd[r] + term;
                     pc[r] += 1;
                     ks[r] += kk;
-                    if (want_max) mx[r] = fmaxf(mx[r], (float)term);
+                    if (want_max && (float)term > mx[r]) {
+                        mx[r] = (float)term;
+                        at[r] = (int32_t)(p - P.a_rp[I]);
+                    }
                 }
                 __syncthreads();
             }
@@ -259,7 +268,11 @@ __global__ void k_cand_bound(int32_t nblk, RowPattern P, int nwords, BoundArgs B
             if (B.use_smem) {
                 B.pcnt[cb + r] = B.use_fast ? (int)(pk[r] & 4095u) : pc[r];
                 B.ksum[cb + r] = k;
-                if (want_max) B.max_term[cb + r] = mx[r];
+                if (want_max) {
+                    const int v = __float_as_int(mx[r]);
+                    B.max_term[cb + r] = B.use_fast ? __int_as_float(v & ~4095) : mx[r];
+                    B.max_at[cb + r] = B.use_fast ? v & 4095 : at[r];
+                }
             }
             if (keep) fl += 2ull * (unsigned long long)(mI * B.bs[J]) * (unsigned long long)k;
         }
@@ -283,7 +296,8 @@ __global__ void k_form_meta(int64_t ncand, const int32_t* __restrict__ keep, con
                             const int64_t* __restrict__ cin, const int32_t* __restrict__ bs,
                             int32_t* __restrict__ f_row, int32_t* __restrict__ f_col, int64_t* __restrict__ f_area,
                             int64_t* __restrict__ f_np, int64_t* __restrict__ f_cin, int32_t* __restrict__ f_ksum,
-                            const float* __restrict__ max_term, float* __restrict__ f_max) {
+                            const float* __restrict__ max_term, const int32_t* __restrict__ max_at,
+                            float* __restrict__ f_max, int32_t* __restrict__ f_at) {
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncand; c += (int64_t)gridDim.x * blockDim.x) {
         if (!keep[c]) continue;
         const int64_t k = kidx[c];
@@ -294,7 +308,10 @@ __global__ void k_form_meta(int64_t ncand, const int32_t* __restrict__ keep, con
         f_np[k] = pcnt[c];
         f_cin[k] = cin ? cin[c] : -1;
         f_ksum[k] = ksum[c];
-        if (f_max) f_max[k] = max_term[c];
+        if (f_max) {
+            f_max[k] = max_term[c];
+            f_at[k] = max_at[c];
+        }
     }
 }
 
@@ -1331,11 +1348,15 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     // a candidate's bound has at most (largest A row) terms: the FP32 margin covers 4095
     const bool few_terms = max_arow < 4096;
     const size_t sm_acc = sm_rank + (size_t)max_row * (few_terms ? 2 * sizeof(float) + sizeof(unsigned)
-                                                                 : sizeof(double) + 2 * sizeof(int32_t) + sizeof(float));
+                                                                 : sizeof(double) + 3 * sizeof(int32_t) + sizeof(float));
     const bool acc_smem = sm_acc <= (size_t)kSymSmemBudget;
     const bool fast_bound = acc_smem && few_terms;
     DBuf<float> max_term;                 // FP64 products: for the choice between the FP64 pipe and the tensor cores
-    if (!bf16) max_term.alloc(nc1, s);
+    DBuf<int32_t> max_at;
+    if (!bf16) {
+        max_term.alloc(nc1, s);
+        max_at.alloc(nc1, s);
+    }
     if (!acc_smem) bound.alloc(nc1, s);
     if (ncand) {
         DBuf<float> b_norm_ru;
@@ -1347,7 +1368,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         BoundArgs ba{std::fabs(alpha), std::fabs(beta), eps * (1.0 - 1e-12), A->norms.p, B->norms.p,
                      use_c ? C->norms.p : nullptr, A->bs.p, coff.p, cand_row.p, cand_col.p,
                      bound.p, pcnt.p, ksum.p, use_c ? cin.p : nullptr, keep.p, acc_smem ? 1 : 0,
-                     fast_bound ? 1 : 0, b_norm_ru.p, max_term.p, (unsigned long long*)maxrow.p + 2};
+                     fast_bound ? 1 : 0, b_norm_ru.p, max_term.p, max_at.p, (unsigned long long*)maxrow.p + 2};
         const size_t sm = acc_smem ? sm_acc : sm_rank;
         allow_dyn_smem(k_cand_bound, sm);
         k_cand_bound<<<sym_grid(nblk), kSymThreads, sm, s>>>(nblk, P, nwords, ba);
@@ -1379,7 +1400,11 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     DBuf<uint8_t> f_comp;                 // 1: the block is computed (0: copied from its twin or dropped)
     DBuf<int64_t> f_area, f_np, f_cin, f_off, f_pbeg, f_rp, flops, nprod_exec, shape_cnt, mirror;
     DBuf<float> f_max;
-    if (tc) f_max.alloc(nf1, s);
+    DBuf<int32_t> f_at;
+    if (tc) {
+        f_max.alloc(nf1, s);
+        f_at.alloc(nf1, s);
+    }
     f_ksum.alloc(nf1, s);
     f_comp.alloc(nf1, s);
     mirror.alloc(nf1, s);
@@ -1401,7 +1426,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     if (ncand) {
         k_form_meta<<<grid_for(ncand, 256), 256, 0, s>>>(ncand, keep.p, kidx.p, cand_row.p, cand_col.p, pcnt.p, ksum.p,
                                                          use_c ? cin.p : nullptr, A->bs.p, f_row.p, f_col.p, f_area.p,
-                                                         f_np.p, f_cin.p, f_ksum.p, max_term.p, f_max.p);
+                                                         f_np.p, f_cin.p, f_ksum.p, max_term.p, max_at.p, f_max.p, f_at.p);
         DBG_LAUNCH_CK();
     }
     std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> tcp(nullptr, f64tc_delete);
@@ -1417,7 +1442,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         if (tc) {
             // group tile patterns, digit tiles and the blocks the tensor cores take (f_comp = 2)
             tcp = f64tc_prepare(A, B, groups, nform, f_rp.p,
-                                F64TcBlocks{f_row.p, f_col.p, mirror.p, f_ksum.p, f_max.p, f_comp.p, sym_result, by_group}, alpha,
+                                F64TcBlocks{f_row.p, f_col.p, mirror.p, f_ksum.p, f_max.p, f_at.p, f_comp.p, sym_result, by_group}, alpha,
                                 plan != nullptr, s);
             tc = tcp != nullptr;
         }
@@ -1461,7 +1486,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     };
     // the candidate arrays are no longer needed
     cand_row.release(); cand_col.release(); pcnt.release(); ksum.release(); bound.release();
-    max_term.release(); f_max.release();
+    max_term.release(); max_at.release(); f_max.release(); f_at.release();
     if (!nform) DBG_CK(cudaEventRecord(ev.e[1], s));
 
     // 5. numeric
@@ -1638,7 +1663,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         };
         zero_small(s);
         DBuf<double> an, bn;                       // the operands' block norms at an execution
-        const F64TcBlocks f64tc_blocks{C->row.p, C->col.p, mirror.p, f_ksum.p, nullptr, f_comp.p, sym_result, by_group};
+        const F64TcBlocks f64tc_blocks{C->row.p, C->col.p, mirror.p, f_ksum.p, nullptr, nullptr, f_comp.p, sym_result, by_group};
         if (tc) {
             an.alloc(std::max<int64_t>(A->nnzb, 1), s);
             bn.alloc(std::max<int64_t>(B->nnzb, 1), s);

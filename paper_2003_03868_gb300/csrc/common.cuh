@@ -354,11 +354,15 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
                                                                bool planned, cudaStream_t s);
 // The current values into the digit tiles (f64tc_prepare has done it for its values).
 void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s);
-// After f64tc_pack of a planned product's new values: the flag returned (device) becomes nonzero when
-// a tensor-core block needs the FP64 pipe with them.  an, bn: room for the operands' block norms.
-const int* f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, double* an, double* bn,
-                         int64_t nform, const F64TcBlocks& f, const int64_t* f_pbeg, const int32_t* prod_a,
-                         const int32_t* prod_b, double alpha, cudaStream_t s);
+// After f64tc_pack of a planned product's new values: the tensor-core blocks that need the FP64 pipe with
+// them (device: a mark per block, and whether there is one).  an, bn: room for the operands' block norms.
+struct F64TcRedo {
+    const int* any;
+    const uint8_t* block;
+};
+F64TcRedo f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, double* an, double* bn,
+                        int64_t nform, const F64TcBlocks& f, const int64_t* f_pbeg, const int32_t* prod_a,
+                        const int32_t* prod_b, double alpha, cudaStream_t s);
 void f64tc_run(F64TcPlan& L, const LowTierOut& o, cudaStream_t s);
 void f64tc_norms(int64_t nform, const uint8_t* comp, const int32_t* row, const int32_t* col, const int32_t* bs,
                  const int64_t* off, const double* data, double* norms, double* dev2, cudaStream_t s);

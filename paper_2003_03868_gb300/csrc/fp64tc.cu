@@ -66,6 +66,9 @@ constexpr long long kOzWait = 4000000000ll;      // about 2 s
 // result's exponent is then formed without overflow from the two operands'.
 constexpr int kExpLimit = 430;
 constexpr int16_t kNoExp = -32768;
+// A product's flags on the device.  0: a wait ran out (1) or the pattern is asymmetric (2); 1: a value outside
+// the scales' range; 2: a planned product's execution has blocks to repeat on the FP64 pipe.
+constexpr int kFlagFailed = 0, kFlagRange = 1, kFlagRedo = 2, kFlags = 3;
 // Clocks of one K step of one 32-column slice charged against the FP64 pipe's flops per clock and SM
 // (1.01 TFLOP/s measured on the block products) when a tile is given to one of the two.  A K step takes
 // about 768 clocks with eight digits and half of that on average (most entries run fewer); beside the
@@ -454,7 +457,7 @@ struct OzArgs {
     const int64_t* ci_off; const double* ci_data;
     double alpha, beta;
     double* c_data;
-    int* err;
+    int* flags;
     unsigned long long* next;                        // the work items' counter
 };
 
@@ -476,7 +479,7 @@ __device__ __forceinline__ void oz_epi_sync() { asm volatile("bar.sync 1, %0;" :
 
 __device__ __forceinline__ void oz_fail(const OzArgs& A, OzShared& S) {
     *(volatile int*)&S.abort = 1;
-    atomicExch(A.err, 1);
+    atomicExch(A.flags + kFlagFailed, 1);
 }
 __device__ __forceinline__ int oz_aborted(const OzShared& S) { return *(volatile const int*)&S.abort; }
 
@@ -679,6 +682,7 @@ __device__ __forceinline__ void oz_item_done(OzShared& S, uint32_t n, int lane) 
 __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs A) {
     extern __shared__ __align__(1024) uint8_t oz_dyn[];
     OzShared& S = *reinterpret_cast<OzShared*>((reinterpret_cast<uintptr_t>(oz_dyn) + 1023) & ~(uintptr_t)1023);
+    if (A.flags[kFlagRange]) return;                  // (a planned product: the FP64 pipe forms every block)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < kOzStages * 2 * kZeroBlocks * (kDigitBlock / 16); i += kOzThreads) {
         const int per = kZeroBlocks * (kDigitBlock / 16);
@@ -1040,7 +1044,8 @@ struct F64TcPlan {
     DBuf<unsigned> c_slices;
     DBuf<int4> ent;
     DBuf<unsigned long long> tile_flops;
-    DBuf<int> flags;                     // 0: a wait ran out / asymmetric pattern, 1: a value outside the scales' range
+    DBuf<int> flags;                     // see kFlag*
+    DBuf<uint8_t> redo;                  // planned products: blocks the FP64 pipe repeats
     int64_t nentries = 0;
 };
 
@@ -1114,7 +1119,7 @@ void oz_pack(F64TcPlan& L, OzOperand& o, const dbcsr_matrix_* M, cudaStream_t s)
     const Groups& g = *L.groups;
     OzPackArgs p{o.pat.nt, o.transpose ? o.pat.t_col.p : o.pat.t_row.p, o.transpose ? o.pat.t_row.p : o.pat.t_col.p,
                  o.tab.p, o.smask.p, g.g_ptr.p, g.g_mrec.p, g.g_w.p, M->off.p, M->data.p, o.transpose, L.R, L.KS,
-                 o.pack.p, o.rexp.p, o.mexp.p, L.flags.p + 1};
+                 o.pack.p, o.rexp.p, o.mexp.p, L.flags.p + kFlagRange};
     k_oz_pack<<<(unsigned)std::min<int64_t>(o.pat.nt, (int64_t)num_sms() * 64), 256, 0, s>>>(p);
     DBG_LAUNCH_CK();
 }
@@ -1170,7 +1175,7 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
         if ((L.a.pat.nt + L.b.pat.nt) * oz_tile_bytes(L) > tot / 4) return P;
     }
     if (!L.cp.nt || (int64_t)(L.a.pat.nt + L.b.pat.nt) * L.KS > 0x7fffffff) return P;
-    L.flags.alloc(2, s);
+    L.flags.alloc(kFlags, s);
     oz_tables(L, L.a, A, s);
     if (!L.b_is_a) {
         L.b.transpose = L.b_sym ? 0 : 1;
@@ -1181,7 +1186,7 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     if (L.b_sym && b.pat.nt) {
         L.b_map.alloc(b.pat.nt, s);
         k_gt_transpose<<<grid_for(b.pat.nt, 256), 256, 0, s>>>(b.pat.nt, b.pat.t_row.p, b.pat.t_col.p, b.pat.t_rp.p,
-                                                               L.b_map.p, L.flags.p);
+                                                               L.b_map.p, L.flags.p + kFlagFailed);
         DBG_LAUNCH_CK();
     }
     // stacks of tile products per C tile
@@ -1221,6 +1226,7 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     L.c_tbl.alloc(L.cp.nt * kGroupMembers * kGroupMembers, s);
     L.c_exp.alloc(L.cp.nt * kGroupMembers * kGroupMembers, s);
     L.next.alloc(1, s);
+    if (planned) L.redo.alloc(nform, s);
     DBG_CK(cudaMemsetAsync(L.c_tbl.p, 0xff, sizeof(int32_t) * L.cp.nt * kGroupMembers * kGroupMembers, s));
     k_oz_tile_flops<<<grid_for(nform, 256), 256, 0, s>>>(nform, L.cp.blk_tile.p, f.row, f.col, f.ksum, A->bs.p,
                                                          L.tile_flops.p);
@@ -1228,7 +1234,7 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     DBuf<int16_t> f_exp;
     f_exp.alloc(nform, s);
     OzGuardArgs ga{nform, L.cp.blk_tile.p, f.row, f.col, g.g_midx.p, g.g_w.p, L.cp.t_col.p, L.s_ptr.p, L.st_a.p, L.st_b.p,
-                   L.a.mexp.p, b.mexp.p, f.max_term, f.max_at, L.tile_flops.p, (float)std::fabs(alpha), L.flags.p + 1,
+                   L.a.mexp.p, b.mexp.p, f.max_term, f.max_at, L.tile_flops.p, (float)std::fabs(alpha), L.flags.p + kFlagRange,
                    f_exp.p, f.comp, L.c_tbl.p, L.c_exp.p, L.c_slices.p, g.g_pos.p, A->bs.p,
                    A->rp.p, A->col.p, A->off.p, A->data.p, B->rp.p, B->col.p, B->off.p, B->data.p};
     k_oz_guard<<<grid_for(nform, 256), 256, 0, s>>>(ga);
@@ -1240,7 +1246,7 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
 }
 
 void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s) {
-    DBG_CK(cudaMemsetAsync(L.flags.p, 0, sizeof(int) * 2, s));
+    DBG_CK(cudaMemsetAsync(L.flags.p, 0, sizeof(int) * kFlags, s));
     oz_pack(L, L.a, A, s);
     if (!L.b_is_a) oz_pack(L, L.b, B, s);
 }
@@ -1253,7 +1259,8 @@ __global__ void __launch_bounds__(32 * kWeakWarps) k_oz_recheck(OzGuardArgs A, c
                                                                 const int32_t* __restrict__ prod_a,
                                                                 const int32_t* __restrict__ prod_b,
                                                                 const double* __restrict__ an,
-                                                                const double* __restrict__ bn, int* __restrict__ bad) {
+                                                                const double* __restrict__ bn,
+                                                                uint8_t* __restrict__ redo, int* __restrict__ any) {
     __shared__ float sh[kWeakWarps][2][kMaxBlock * kMaxBlock];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t k = (int64_t)blockIdx.x * kWeakWarps + warp; k < A.nform; k += (int64_t)gridDim.x * kWeakWarps) {
@@ -1283,8 +1290,8 @@ __global__ void __launch_bounds__(32 * kWeakWarps) k_oz_recheck(OzGuardArgs A, c
                 at = oat;
             }
         }
-        bool ok = true;
-        if (E > kNoExp / 2) {
+        bool ok = *A.bad == 0;                        // (an operand outside the scales: all of them)
+        if (ok && E > kNoExp / 2) {
             ok = at >= 0 && ldexp((double)kNormRatio, E - 1) < mx && mx <= 1e300;
             if (ok) {
                 const int32_t p = prod_a[at], q = prod_b[at];
@@ -1294,16 +1301,17 @@ __global__ void __launch_bounds__(32 * kWeakWarps) k_oz_recheck(OzGuardArgs A, c
         }
         if (lane == 0) {
             A.c_exp[(int64_t)t * (kGroupMembers * kGroupMembers) + a * kGroupMembers + b] = (int16_t)max(E, kNoTerm);
-            if (!ok) atomicExch(bad, 1);
+            redo[k] = ok ? 0 : 1;
+            if (!ok) atomicExch(any, 1);
         }
     }
 }
 
 }  // namespace
 
-const int* f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, double* an, double* bn,
-                         int64_t nform, const F64TcBlocks& f, const int64_t* f_pbeg, const int32_t* prod_a,
-                         const int32_t* prod_b, double alpha, cudaStream_t s) {
+F64TcRedo f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, double* an, double* bn,
+                        int64_t nform, const F64TcBlocks& f, const int64_t* f_pbeg, const int32_t* prod_a,
+                        const int32_t* prod_b, double alpha, cudaStream_t s) {
     const Groups& g = *L.groups;
     const OzOperand& b = L.b_is_a ? L.a : L.b;
     block_norms(A, an, s);
@@ -1313,13 +1321,15 @@ const int* f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matri
         bnp = bn;
     }
     OzGuardArgs ga{nform, L.cp.blk_tile.p, f.row, f.col, g.g_midx.p, g.g_w.p, L.cp.t_col.p, L.s_ptr.p, L.st_a.p, L.st_b.p,
-                   L.a.mexp.p, b.mexp.p, nullptr, nullptr, L.tile_flops.p, (float)std::fabs(alpha), nullptr, nullptr, f.comp,
+                   L.a.mexp.p, b.mexp.p, nullptr, nullptr, L.tile_flops.p, (float)std::fabs(alpha), L.flags.p + kFlagRange,
+                   nullptr, f.comp,
                    L.c_tbl.p, L.c_exp.p, nullptr, g.g_pos.p, A->bs.p,
                    A->rp.p, A->col.p, A->off.p, A->data.p, B->rp.p, B->col.p, B->off.p, B->data.p};
-    k_oz_recheck<<<grid_for(nform, kWeakWarps, (int64_t)num_sms() * 64), 32 * kWeakWarps, 0, s>>>(ga, f_pbeg, prod_a, prod_b, an, bnp, L.flags.p + 1);
+    k_oz_recheck<<<grid_for(nform, kWeakWarps, (int64_t)num_sms() * 64), 32 * kWeakWarps, 0, s>>>(
+        ga, f_pbeg, prod_a, prod_b, an, bnp, L.redo.p, L.flags.p + kFlagRedo);
     DBG_LAUNCH_CK();
     oz_depth(L, s);
-    return L.flags.p + 1;
+    return F64TcRedo{L.flags.p + kFlagRedo, L.redo.p};
 }
 
 void f64tc_run(F64TcPlan& L, const LowTierOut& o, cudaStream_t s) {
@@ -1350,7 +1360,7 @@ void f64tc_run(F64TcPlan& L, const LowTierOut& o, cudaStream_t s) {
     a.alpha = o.alpha;
     a.beta = o.beta;
     a.c_data = o.c_data;
-    a.err = L.flags.p;
+    a.flags = L.flags.p;
     OzMaps mb;
     for (int d = 0; d < kDigits; ++d) mb.m[d] = oz_map(b.pack.p, L.R, b.pat.nt * L.KS, d + 1);
     const size_t sm = sizeof(OzShared) + 1024;
@@ -1370,7 +1380,7 @@ int64_t f64tc_tiles(const F64TcPlan& L) { return L.cp.nt; }
 
 void f64tc_check(F64TcPlan& L, cudaStream_t s) {
     int e = 0;
-    DBG_CK(cudaMemcpyAsync(&e, L.flags.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    DBG_CK(cudaMemcpyAsync(&e, L.flags.p + kFlagFailed, sizeof(int), cudaMemcpyDeviceToHost, s));
     DBG_CK(cudaStreamSynchronize(s));
     if (e == 1) fail(DBCSR_ETIMEOUT, "multiply: a wait of the tensor-core kernel ran out");
     if (e == 2) fail(DBCSR_EINVAL, "multiply: an operand marked symmetric has an asymmetric pattern");

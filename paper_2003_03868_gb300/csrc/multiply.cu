@@ -734,8 +734,12 @@ __global__ void __launch_bounds__(256) k_smm_f64(int64_t nlist, const int64_t* _
     const int per_cta = PAIR ? (blockDim.x >> 6) : (blockDim.x >> 5);
     const int64_t stride = (int64_t)gridDim.x * per_cta;
     int parity = 0;
-    for (int64_t w = (int64_t)blockIdx.x * per_cta + pair; w < nlist; w += stride, parity ^= 1)
-        smm_block<E, PAIR>(list[w], S, lane, part, pair, parity, sh_part);
+    for (int64_t w = (int64_t)blockIdx.x * per_cta + pair; w < nlist; w += stride) {
+        const int64_t k = list[w];
+        if (S.redo && !S.redo[k]) continue;              // (the same for both warps of a pair)
+        smm_block<E, PAIR>(k, S, lane, part, pair, parity, sh_part);
+        parity ^= 1;
+    }
 }
 
 
@@ -836,8 +840,10 @@ __global__ void __launch_bounds__(256) k_smm_f64_ks(int64_t nlist, const int64_t
     if (S.gate && *S.gate == 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps)
-        smm_block_ks<EF, R>(list[w], S, lane);
+    for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps) {
+        const int64_t k = list[w];
+        if (!S.redo || S.redo[k]) smm_block_ks<EF, R>(k, S, lane);
+    }
 }
 
 // The five-slot class (23 x 7 and 7 x 23: m n = 32 x 5 + 1) with registers capped for three
@@ -847,8 +853,10 @@ __global__ void __launch_bounds__(256, 3) k_smm_f64_ks5(int64_t nlist, const int
     if (S.gate && *S.gate == 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps)
-        smm_block_ks<5, 1>(list[w], S, lane);
+    for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps) {
+        const int64_t k = list[w];
+        if (!S.redo || S.redo[k]) smm_block_ks<5, 1>(k, S, lane);
+    }
 }
 
 // One launch for every block shape of a product: the warps take C blocks from one work queue
@@ -1685,10 +1693,13 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             const bool beside = n_simt >= (tc ? 1 : 2);
             if (beside && !tc) side.begin(cs, n_simt);
             if (tc) {
-                // the tensor cores' blocks with the current values; the FP64 pipe repeats them all
-                // when these need it (f64tc_recheck)
+                // the tensor cores' blocks with the current values; the FP64 pipe repeats those that
+                // need it with these (f64tc_recheck)
                 f64tc_pack(*tcp, A, B, cs);
-                fb.gate = f64tc_recheck(*tcp, A, B, an.p, bn.p, nform, f64tc_blocks, f_pbeg.p, prod_a.p, prod_b.p, alpha, cs);
+                const F64TcRedo redo = f64tc_recheck(*tcp, A, B, an.p, bn.p, nform, f64tc_blocks, f_pbeg.p, prod_a.p,
+                                                     prod_b.p, alpha, cs);
+                fb.gate = redo.any;
+                fb.redo = redo.block;
                 if (beside) side.begin(cs, n_simt);
                 f64tc_run(*tcp, lto, cs);
                 f64tc_norms(nform, f_comp.p, C->row.p, C->col.p, C->bs.p, C->off.p, C->data.p, C->norms.p, c_dev2.p, cs);

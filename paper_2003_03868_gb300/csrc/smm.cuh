@@ -25,6 +25,7 @@ struct SmmArgs {
     int colmajor;    // lane -> element order: 0 row-major (i = idx / n), 1 column-major (i = idx % m)
     int prefetch2;   // 1: fetch the next 32 products' metadata before using the current ones
     const int* gate;     // nullable: the launch does nothing when this device flag is 0
+    const uint8_t* redo; // with gate: only the blocks marked here are formed
 };
 
 // Launch configuration of one (m, n) shape.  tpb, ctas_per_sm, colmajor and prefetch2 leave

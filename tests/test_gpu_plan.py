@@ -97,3 +97,30 @@ def test_plan_pins_its_matrices(gb):
     plan.close()
     gb.multiply(1.0, A, A, 0.0, C_, 0.0)         # free again once the plan is gone
     A.close()
+
+
+def test_new_values_send_only_the_blocks_that_need_it_to_the_fp64_units(gb):
+    # one block row of A graded by 2^-40 inside its blocks: the blocks of C in other groups' rows stay the
+    # same bits, the graded row's keep an FP64 product's accuracy in every element
+    bs = [28] * 16
+    n, nb = sum(bs), len(bs)
+    a, b = (synth.random_block_matrix(bs, 1.0, 2200 + i) for i in range(2))
+    A, B = gb.Matrix.of(a), gb.Matrix.of(b)
+    g_of, _, _ = A.groups()
+    C = gb.Matrix(A.blk_size, A.stream)
+    plan = gb.Plan(1.0, A, B, C, 0.0)
+    assert plan.stats.n_tiles > 0
+    dense = lambda d: np.asarray(d).reshape(nb, nb, 28, 28).transpose(0, 2, 1, 3).reshape(n, n)  # noqa: E731
+    plan.execute()
+    before = dense(C.export()[2])
+    v = a.data.copy()
+    rows = v[5 * nb * 784:6 * nb * 784].reshape(nb, 28, 28)
+    rows *= 2.0 ** -np.linspace(0, 40, 28).round()[None, :, None]
+    A.put_values(v)
+    plan.execute()
+    after = dense(C.export()[2])
+    other = np.repeat(g_of != g_of[5], 28)
+    assert other.any() and np.array_equal(before[other], after[other])
+    x, y = dense(v)[140:168], dense(b.data)
+    assert np.all(np.abs(after[140:168] - x @ y) <= 2 * (n + 4) * 2.0 ** -53 * (np.abs(x) @ np.abs(y)))
+    plan.close()

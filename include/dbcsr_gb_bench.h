@@ -51,6 +51,14 @@ int32_t dbcsr_pool_usage(int64_t* used_now, int64_t* used_high, int32_t reset_hi
 int32_t dbcsr_wait_selftest(int64_t limit_cycles, int32_t arrive, int64_t* waited);
 
 /*
+ * Self-test of a planned FP64 product's recovery: with fail != 0 the tensor-core kernel of the plan's
+ * later executions stops before its first block, as after a bounded wait that ran out, and the
+ * executions form those blocks on the FP64 pipe instead; fail == 0 ends that.  Errors: EINVAL (null
+ * plan, or one without tensor-core blocks); ECUDA.
+ */
+int32_t dbcsr_plan_wait_selftest(dbcsr_plan plan, int32_t fail);
+
+/*
  * The block groups of the tensor-core tier, built now from m's block norms (a BF16 product with
  * m as A builds the same groups when m carries none): the block rows are merged along their
  * strongest couplings -- every row's 12 largest off-diagonal block norms, ties to the lower

@@ -355,9 +355,9 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
 // The current values into the digit tiles (f64tc_prepare has done it for its values).
 void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s);
 // After f64tc_pack of a planned product's new values: the tensor-core blocks that need the FP64 pipe with
-// them (device: a mark per block, and whether there is one).  an, bn: room for the operands' block norms.
+// them (device: a mark per block, and SmmArgs' gate).  an, bn: room for the operands' block norms.
 struct F64TcRedo {
-    const int* any;
+    const int* gate;
     const uint8_t* block;
 };
 F64TcRedo f64tc_recheck(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, double* an, double* bn,
@@ -369,6 +369,8 @@ void f64tc_norms(int64_t nform, const uint8_t* comp, const int32_t* row, const i
 int64_t f64tc_tiles(const F64TcPlan& L);
 // Fails with DBCSR_ETIMEOUT when a bounded wait of the kernel ran out (synchronises s).
 void f64tc_check(F64TcPlan& L, cudaStream_t s);
+// Whether later runs of a planned product stop at once, as after a wait that ran out (synchronises s).
+void f64tc_selftest(F64TcPlan& L, bool fail_waits, cudaStream_t s);
 
 // ---- dense.cu
 // C[b] = alpha A[b] B[b] + beta Cin[b] (Cin may be C) for nb row-major n x n matrices (b < 65536): FP64 on the

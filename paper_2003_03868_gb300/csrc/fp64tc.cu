@@ -66,9 +66,10 @@ constexpr long long kOzWait = 4000000000ll;      // about 2 s
 // result's exponent is then formed without overflow from the two operands'.
 constexpr int kExpLimit = 430;
 constexpr int16_t kNoExp = -32768;
-// A product's flags on the device.  0: a wait ran out (1) or the pattern is asymmetric (2); 1: a value outside
-// the scales' range; 2: a planned product's execution has blocks to repeat on the FP64 pipe.
-constexpr int kFlagFailed = 0, kFlagRange = 1, kFlagRedo = 2, kFlags = 3;
+// A product's flags on the device.  0: a value outside the scales' range; 1: a planned product's execution has
+// blocks to repeat on the FP64 pipe; 2: a wait ran out (1; a planned product's execution then repeats every
+// block) or the pattern is asymmetric (2).
+constexpr int kFlagRange = 0, kFlagRedo = 1, kFlagFailed = 2, kFlags = 3;
 // Clocks of one K step of one 32-column slice charged against the FP64 pipe's flops per clock and SM
 // (1.01 TFLOP/s measured on the block products) when a tile is given to one of the two.  A K step takes
 // about 768 clocks with eight digits and half of that on average (most entries run fewer); beside the
@@ -682,7 +683,8 @@ __device__ __forceinline__ void oz_item_done(OzShared& S, uint32_t n, int lane) 
 __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs A) {
     extern __shared__ __align__(1024) uint8_t oz_dyn[];
     OzShared& S = *reinterpret_cast<OzShared*>((reinterpret_cast<uintptr_t>(oz_dyn) + 1023) & ~(uintptr_t)1023);
-    if (A.flags[kFlagRange]) return;                  // (a planned product: the FP64 pipe forms every block)
+    // (a planned product whose blocks the FP64 pipe forms: all of them for these values, or the self-test's)
+    if (A.flags[kFlagRange] || A.flags[kFlagFailed] == 1) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < kOzStages * 2 * kZeroBlocks * (kDigitBlock / 16); i += kOzThreads) {
         const int per = kZeroBlocks * (kDigitBlock / 16);
@@ -1044,7 +1046,7 @@ struct F64TcPlan {
     DBuf<unsigned> c_slices;
     DBuf<int4> ent;
     DBuf<unsigned long long> tile_flops;
-    DBuf<int> flags;                     // see kFlag*
+    DBuf<int> flags, flags0;             // see kFlag*; what they start with (0 but for the self-test)
     DBuf<uint8_t> redo;                  // planned products: blocks the FP64 pipe repeats
     int64_t nentries = 0;
 };
@@ -1176,6 +1178,8 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     }
     if (!L.cp.nt || (int64_t)(L.a.pat.nt + L.b.pat.nt) * L.KS > 0x7fffffff) return P;
     L.flags.alloc(kFlags, s);
+    L.flags0.alloc(kFlags, s);
+    L.flags0.zero();
     oz_tables(L, L.a, A, s);
     if (!L.b_is_a) {
         L.b.transpose = L.b_sym ? 0 : 1;
@@ -1246,7 +1250,7 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
 }
 
 void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s) {
-    DBG_CK(cudaMemsetAsync(L.flags.p, 0, sizeof(int) * kFlags, s));
+    DBG_CK(cudaMemcpyAsync(L.flags.p, L.flags0.p, sizeof(int) * kFlags, cudaMemcpyDeviceToDevice, s));
     oz_pack(L, L.a, A, s);
     if (!L.b_is_a) oz_pack(L, L.b, B, s);
 }
@@ -1377,6 +1381,12 @@ void f64tc_norms(int64_t nform, const uint8_t* comp, const int32_t* row, const i
 }
 
 int64_t f64tc_tiles(const F64TcPlan& L) { return L.cp.nt; }
+
+void f64tc_selftest(F64TcPlan& L, bool fail_waits, cudaStream_t s) {
+    const int v = fail_waits ? 1 : 0;
+    DBG_CK(cudaMemcpyAsync(L.flags0.p + kFlagFailed, &v, sizeof v, cudaMemcpyHostToDevice, s));
+    DBG_CK(cudaStreamSynchronize(s));
+}
 
 void f64tc_check(F64TcPlan& L, cudaStream_t s) {
     int e = 0;

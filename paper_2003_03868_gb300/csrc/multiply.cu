@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "dbcsr_gb_bench.h"
 #include "grouptiles.cuh"
 #include "smm.cuh"
 
@@ -728,7 +729,7 @@ __global__ void __launch_bounds__(256) k_smm_f64(int64_t nlist, const int64_t* _
     // element slots, so a large block needs half the registers per thread; the halves'
     // norm sums meet in shared memory behind a 64-thread named barrier of the pair.
     __shared__ double sh_part[PAIR ? 4 : 1][2][2];
-    if (S.gate && *S.gate == 0) return;
+    if (S.gate && !S.gate[0] && !S.gate[1]) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = PAIR ? (warp & 1) : 0, pair = PAIR ? (warp >> 1) : warp;
     const int per_cta = PAIR ? (blockDim.x >> 6) : (blockDim.x >> 5);
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(256) k_smm_f64(int64_t nlist, const int64_t* _
     int parity = 0;
     for (int64_t w = (int64_t)blockIdx.x * per_cta + pair; w < nlist; w += stride) {
         const int64_t k = list[w];
-        if (S.redo && !S.redo[k]) continue;              // (the same for both warps of a pair)
+        if (S.gate && !S.gate[1] && !S.redo[k]) continue;   // (the same for both warps of a pair)
         smm_block<E, PAIR>(k, S, lane, part, pair, parity, sh_part);
         parity ^= 1;
     }
@@ -837,12 +838,12 @@ __device__ __forceinline__ void smm_block_ks(int64_t k, const SmmArgs& S, int la
 
 template <int EF, int R>
 __global__ void __launch_bounds__(256) k_smm_f64_ks(int64_t nlist, const int64_t* __restrict__ list, SmmArgs S) {
-    if (S.gate && *S.gate == 0) return;
+    if (S.gate && !S.gate[0] && !S.gate[1]) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps) {
         const int64_t k = list[w];
-        if (!S.redo || S.redo[k]) smm_block_ks<EF, R>(k, S, lane);
+        if (!S.gate || S.gate[1] || S.redo[k]) smm_block_ks<EF, R>(k, S, lane);
     }
 }
 
@@ -850,12 +851,12 @@ __global__ void __launch_bounds__(256) k_smm_f64_ks(int64_t nlist, const int64_t
 // CTAs of 256 threads per SM (80 registers, no spills): at the uncapped 98 registers only two
 // fit, and the operand loads' latency showed (FP64 pipe 72% busy).
 __global__ void __launch_bounds__(256, 3) k_smm_f64_ks5(int64_t nlist, const int64_t* __restrict__ list, SmmArgs S) {
-    if (S.gate && *S.gate == 0) return;
+    if (S.gate && !S.gate[0] && !S.gate[1]) return;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nlist; w += warps) {
         const int64_t k = list[w];
-        if (!S.redo || S.redo[k]) smm_block_ks<5, 1>(k, S, lane);
+        if (!S.gate || S.gate[1] || S.redo[k]) smm_block_ks<5, 1>(k, S, lane);
     }
 }
 
@@ -1670,6 +1671,8 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
             DBG_LAUNCH_CK();
         };
         zero_small(s);
+        if (lt) lowtier_check(*lt, s);
+        if (tcp) f64tc_check(*tcp, s);
         DBuf<double> an, bn;                       // the operands' block norms at an execution
         const F64TcBlocks f64tc_blocks{C->row.p, C->col.p, mirror.p, f_ksum.p, nullptr, nullptr, f_comp.p, sym_result, by_group};
         if (tc) {
@@ -1698,7 +1701,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
                 f64tc_pack(*tcp, A, B, cs);
                 const F64TcRedo redo = f64tc_recheck(*tcp, A, B, an.p, bn.p, nform, f64tc_blocks, f_pbeg.p, prod_a.p,
                                                      prod_b.p, alpha, cs);
-                fb.gate = redo.any;
+                fb.gate = redo.gate;
                 fb.redo = redo.block;
                 if (beside) side.begin(cs, n_simt);
                 f64tc_run(*tcp, lto, cs);
@@ -1889,6 +1892,18 @@ dbcsr_status dbcsr_multiply_execute(dbcsr_plan plan) {
     } catch (const std::exception& e) {
         dbg::set_last_error(e.what());
         return DBCSR_ECUDA;
+    }
+}
+
+int32_t dbcsr_plan_wait_selftest(dbcsr_plan plan, int32_t fail) {
+    try {
+        if (!plan || !plan->plan.tc) dbg::fail(DBCSR_EINVAL, "plan_wait_selftest: no FP64 plan with tensor-core blocks");
+        dbg::f64tc_selftest(*plan->plan.tc, fail != 0, plan->plan.stream);
+        dbg::set_last_error("");
+        return DBCSR_OK;
+    } catch (const dbg::Error& e) {
+        dbg::set_last_error(e.what());
+        return e.code;
     }
 }
 

@@ -24,8 +24,10 @@ struct SmmArgs {
     double* c_data; double* c_norm; double* c_dev2;
     int colmajor;    // lane -> element order: 0 row-major (i = idx / n), 1 column-major (i = idx % m)
     int prefetch2;   // 1: fetch the next 32 products' metadata before using the current ones
-    const int* gate;     // nullable: the launch does nothing when this device flag is 0
-    const uint8_t* redo; // with gate: only the blocks marked here are formed
+    // a planned product's repetition of tensor-core blocks (nullable): gate[1] nonzero: every block, else
+    // gate[0] nonzero: those marked in redo, else none
+    const int* gate;
+    const uint8_t* redo;
 };
 
 // Launch configuration of one (m, n) shape.  tpb, ctas_per_sm, colmajor and prefetch2 leave

@@ -124,3 +124,25 @@ def test_new_values_send_only_the_blocks_that_need_it_to_the_fp64_units(gb):
     x, y = dense(v)[140:168], dense(b.data)
     assert np.all(np.abs(after[140:168] - x @ y) <= 2 * (n + 4) * 2.0 ** -53 * (np.abs(x) @ np.abs(y)))
     plan.close()
+
+
+def test_execution_whose_tensor_core_waits_run_out(gb):
+    # the kernel stops before its first block, as after a wait that ran out: the execution's result is still
+    # that of the current values (C held another one), and so is the next one
+    a, b = (synth.random_block_matrix([28] * 16, 1.0, 2300 + i) for i in range(2))
+    A, B = gb.Matrix.of(a), gb.Matrix.of(b)
+    C = gb.Matrix(A.blk_size, A.stream)
+    plan = gb.Plan(1.0, A, B, C, 0.0)
+    assert plan.stats.n_tiles > 0
+    test = gb.lib().dbcsr_plan_wait_selftest
+    x, y = bsr.to_dense(bsr.Mat.of(a)), bsr.to_dense(bsr.Mat.of(b))
+    n = x.shape[0]
+    for scale, fail in ((2.0, 1), (-0.5, 1), (4.0, 0)):
+        assert test(plan.handle, fail) == gb._ffi.DBCSR_OK
+        A.put_values(scale * a.data)
+        plan.execute()
+        got = bsr.to_dense(bsr.Mat(C.blk_size, *C.export()))
+        bound = 2 * (n + 4) * 2.0 ** -53 * (np.abs(scale * x) @ np.abs(y))
+        assert np.all(np.abs(got - scale * (x @ y)) <= bound), (scale, fail)
+    plan.close()
+    assert test(None, 1) == gb._ffi.DBCSR_EINVAL

@@ -95,3 +95,23 @@ def test_elements_of_graded_blocks(gb, kind, bits, planned):
         err, mag, tiles = _error(gb, bs, a, b, planned)
         assert tiles > 0 if bits == 0 and kind != "zeros" else True
         assert np.all(np.abs(err) <= (n + 4) * U * mag), (bs[:3], float(np.max(np.abs(err) / (U * np.maximum(mag, 1e-300)))))
+
+
+def test_digits_left_out(gb):
+    # four groups of 112 rows (A's couplings are twice as strong inside them).  In the first one the products
+    # cancel to 2^-20, in the others B is 2^-19 smaller, where the last two of eight digits may go.  What is
+    # left out of 36 digit products sums up to 2^-59.9 (root mean square: 112 terms of six digit pairs of
+    # 2^12.4, 2^-78 each, at the scale 2 of the group's own rows; the others' part is below 2^-62);
+    # an FP64 chain, seven digits for eight, or one digit less in the far groups leave 2^-55 and more
+    n, g = 448, 112
+    r = np.random.default_rng(3100)
+    a, b = r.uniform(-1.0, 1.0, (n, n)), r.uniform(-1.0, 1.0, (n, n)) * 2.0 ** -19
+    a[:, g // 2:g] = a[:, :g // 2]
+    for x in range(0, n, g):
+        a[x:x + g, x:x + g] *= 2.0
+    b[:g // 2] = r.uniform(-1.0, 1.0, (g // 2, n))
+    b[g // 2:g] = -(b[:g // 2] + 2.0 ** -20 * r.uniform(-1.0, 1.0, (g // 2, n)))
+    for planned in (False, True):
+        err, _, tiles = _error(gb, [28] * 16, a, b, planned)
+        assert planned or tiles == 16             # (a plan's groups come from the values it was made with)
+        assert np.sqrt(np.mean(err ** 2)) <= 2.0 ** -57

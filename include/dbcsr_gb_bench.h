@@ -42,6 +42,13 @@ int64_t dbcsr_launch_count(void);
 int32_t dbcsr_pool_usage(int64_t* used_now, int64_t* used_high, int32_t reset_high);
 
 /*
+ * For tests of what a call does when the device's memory runs out: allocations that would take the
+ * library's pool past `bytes` in use fail as the device's own would (DBCSR_ENOMEM), on every device; 0: no
+ * limit.  Errors: EINVAL (negative).
+ */
+int32_t dbcsr_pool_limit(int64_t bytes);
+
+/*
  * Self-test of the bounded device-side waits every persistent kernel of the library uses:
  * one CTA waits on an mbarrier for at most limit_cycles SM clock cycles (limit_cycles >= 0).
  * arrive != 0: a thread of the CTA arrives first, so the wait completes (DBCSR_OK);

@@ -91,7 +91,8 @@ cudaMemPool_t library_pool();
 void trim_pool(uint64_t keep_bytes);
 // Stream-ordered allocation from library_pool().  When the device is out of memory the
 // cached free memory is returned to the driver (after the device is idle) and the
-// allocation is tried once more; a second failure throws DBCSR_ENOMEM.
+// allocation is tried once more; a second failure throws DBCSR_ENOMEM.  So does, for tests, an
+// allocation past the limit set by dbcsr_pool_limit.
 void pool_alloc(void** p, size_t bytes, cudaStream_t s);
 
 // Device array allocated and freed in stream order from library_pool().
@@ -367,6 +368,8 @@ void f64tc_run(F64TcPlan& L, const LowTierOut& o, cudaStream_t s);
 void f64tc_norms(int64_t nform, const uint8_t* comp, const int32_t* row, const int32_t* col, const int32_t* bs,
                  const int64_t* off, const double* data, double* norms, double* dev2, cudaStream_t s);
 int64_t f64tc_tiles(const F64TcPlan& L);
+// Frees the tiles and tables (f64tc_tiles and f64tc_check may still follow).
+void f64tc_release(F64TcPlan& L);
 // Fails with DBCSR_ETIMEOUT when a bounded wait of the kernel ran out (synchronises s).
 void f64tc_check(F64TcPlan& L, cudaStream_t s);
 // Whether later runs of a planned product stop at once, as after a wait that ran out (synchronises s).

@@ -34,6 +34,8 @@
 // holds a value that is not finite or too large or small for the scales.
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <mutex>
 #include <vector>
 
 #include <cuda.h>
@@ -267,6 +269,20 @@ struct OzGuardArgs {
     const int64_t* b_rp; const int32_t* b_col; const int64_t* b_off; const double* b_data;
 };
 
+__device__ __forceinline__ bool oz_pays(int64_t entries, int width, unsigned long long flops) {
+    const int slices = (width + kSlice - 1) / kSlice;
+    return (double)entries * (kGroupWidth / 16) * slices * kStepClocks * kSimtFlopsPerClock <= (double)flops;
+}
+// Tiles for which the tensor cores pay: without one nothing is packed.
+__global__ void k_oz_pays(int64_t nt, const int64_t* __restrict__ s_ptr, const int32_t* __restrict__ c_tcol,
+                          const int32_t* __restrict__ g_w, const unsigned long long* __restrict__ flops,
+                          unsigned long long* __restrict__ count) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool pays = t < nt && oz_pays(s_ptr[t + 1] - s_ptr[t], g_w[c_tcol[t]], flops[t]);
+    const int n = __syncthreads_count(pays);
+    if (threadIdx.x == 0 && n) atomicAdd(count, (unsigned long long)n);
+}
+
 // A computed block runs on the tensor cores (comp = 2) unless
 //   * its tile's tensor-core time (every stack entry at full width; a rule on the tile alone, so
 //     a block takes the same path in any batch) is above the FP64 pipe's time for its blocks;
@@ -287,10 +303,7 @@ __global__ void k_oz_guard(OzGuardArgs A) {
         const int32_t t = A.blk_tile[k];
         if (bad || t < 0) continue;
         const int64_t e0 = A.s_ptr[t], e1 = A.s_ptr[t + 1];
-        const int wc = A.g_w[A.c_tcol[t]];
-        const int slices = (wc + kSlice - 1) / kSlice;
-        const double clocks = (double)(e1 - e0) * (kGroupWidth / 16) * slices * kStepClocks;
-        if (clocks * kSimtFlopsPerClock > (double)A.tile_flops[t]) continue;
+        if (!oz_pays(e1 - e0, A.g_w[A.c_tcol[t]], A.tile_flops[t])) continue;
         const int a = A.g_midx[A.f_row[k]], b = A.g_midx[A.f_col[k]];
         int E = 2 * kNoExp;
         for (int64_t e = e0; e < e1; ++e)
@@ -1096,6 +1109,21 @@ void tile_patterns(const Groups& g, PatternJob* jobs, int n, int64_t* max_c, cud
     }
 }
 
+int64_t device_memory() {
+    static std::mutex mu;
+    static auto* bytes = new std::map<int, int64_t>();   // (outlives every static destructor)
+    int dev = 0;
+    DBG_CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    int64_t& n = (*bytes)[dev];
+    if (!n) {
+        size_t fr = 0, all = 0;
+        DBG_CK(cudaMemGetInfo(&fr, &all));
+        n = (int64_t)all;
+    }
+    return n;
+}
+
 int64_t oz_tile_bytes(const F64TcPlan& L) { return (int64_t)L.KS * 2 * kDigits * 16 * L.R; }
 
 void oz_tables(F64TcPlan& L, OzOperand& o, const dbcsr_matrix_* M, cudaStream_t s) {
@@ -1165,27 +1193,14 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     jobs[nj++] = {f_rp, f.col, f.comp, nform, &L.cp};
     int64_t max_row = 0;
     tile_patterns(g, jobs, nj, &max_row, s);
-    // the packed operands stay within a quarter of the device's memory
-    {
-        static std::atomic<int64_t> total{0};
-        int64_t tot = total.load();
-        if (!tot) {
-            size_t fr = 0, t = 0;
-            DBG_CK(cudaMemGetInfo(&fr, &t));
-            total.store(tot = (int64_t)t);
-        }
-        if ((L.a.pat.nt + L.b.pat.nt) * oz_tile_bytes(L) > tot / 4) return P;
-    }
+    // the packed operands stay within a quarter of the device's memory (and where what is free does not hold
+    // them, the product runs again without them: multiply)
+    if ((L.a.pat.nt + L.b.pat.nt) * oz_tile_bytes(L) > device_memory() / 4) return P;
     if (!L.cp.nt || (int64_t)(L.a.pat.nt + L.b.pat.nt) * L.KS > 0x7fffffff) return P;
     L.flags.alloc(kFlags, s);
     L.flags0.alloc(kFlags, s);
+    L.flags.zero();
     L.flags0.zero();
-    oz_tables(L, L.a, A, s);
-    if (!L.b_is_a) {
-        L.b.transpose = L.b_sym ? 0 : 1;
-        oz_tables(L, L.b, B, s);
-    }
-    f64tc_pack(L, A, B, s);
     OzOperand& b = L.b_is_a ? L.a : L.b;
     if (L.b_sym && b.pat.nt) {
         L.b_map.alloc(b.pat.nt, s);
@@ -1211,7 +1226,30 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     k_gt_stack<<<grid, 256, sm, s>>>(g.ngrp, sa, nwords);
     DBG_LAUNCH_CK();
     scan_exclusive(cnt.p, L.s_ptr.p, L.cp.nt, s);
-    L.nentries = read_i64(L.s_ptr.p + L.cp.nt, s);
+    L.tile_flops.alloc(L.cp.nt, s);
+    L.tile_flops.zero();
+    k_oz_tile_flops<<<grid_for(nform, 256), 256, 0, s>>>(nform, L.cp.blk_tile.p, f.row, f.col, f.ksum, A->bs.p,
+                                                         L.tile_flops.p);
+    DBG_LAUNCH_CK();
+    L.next.alloc(1, s);
+    L.next.zero();
+    k_oz_pays<<<(unsigned)ceil_div(L.cp.nt, 256), 256, 0, s>>>(L.cp.nt, L.s_ptr.p, L.cp.t_col.p, g.g_w.p, L.tile_flops.p,
+                                                               L.next.p);
+    DBG_LAUNCH_CK();
+    {
+        const int64_t* src[2] = {L.s_ptr.p + L.cp.nt, (const int64_t*)L.next.p};
+        int64_t h[2];
+        read_i64s(src, 2, h, s);
+        L.nentries = h[0];
+        if (!h[1]) return P;
+    }
+    oz_tables(L, L.a, A, s);
+    oz_pack(L, L.a, A, s);
+    if (!L.b_is_a) {
+        L.b.transpose = L.b_sym ? 0 : 1;
+        oz_tables(L, L.b, B, s);
+        oz_pack(L, L.b, B, s);
+    }
     const int64_t ne = std::max<int64_t>(L.nentries, 1);
     L.st_a.alloc(ne, s);
     L.st_b.alloc(ne, s);
@@ -1223,18 +1261,12 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     k_gt_stack<<<grid, 256, sm, s>>>(g.ngrp, sa, nwords);
     DBG_LAUNCH_CK();
     // which blocks the tensor cores take
-    L.tile_flops.alloc(L.cp.nt, s);
-    L.tile_flops.zero();
     L.c_slices.alloc(L.cp.nt, s);
     L.c_slices.zero();
     L.c_tbl.alloc(L.cp.nt * kGroupMembers * kGroupMembers, s);
     L.c_exp.alloc(L.cp.nt * kGroupMembers * kGroupMembers, s);
-    L.next.alloc(1, s);
     if (planned) L.redo.alloc(nform, s);
     DBG_CK(cudaMemsetAsync(L.c_tbl.p, 0xff, sizeof(int32_t) * L.cp.nt * kGroupMembers * kGroupMembers, s));
-    k_oz_tile_flops<<<grid_for(nform, 256), 256, 0, s>>>(nform, L.cp.blk_tile.p, f.row, f.col, f.ksum, A->bs.p,
-                                                         L.tile_flops.p);
-    DBG_LAUNCH_CK();
     DBuf<int16_t> f_exp;
     f_exp.alloc(nform, s);
     OzGuardArgs ga{nform, L.cp.blk_tile.p, f.row, f.col, g.g_midx.p, g.g_w.p, L.cp.t_col.p, L.s_ptr.p, L.st_a.p, L.st_b.p,
@@ -1381,6 +1413,19 @@ void f64tc_norms(int64_t nform, const uint8_t* comp, const int32_t* row, const i
 }
 
 int64_t f64tc_tiles(const F64TcPlan& L) { return L.cp.nt; }
+
+void f64tc_release(F64TcPlan& L) {
+    for (OzOperand* o : {&L.a, &L.b}) {
+        o->pack.release();
+        o->tab.release();
+        o->rexp.release();
+    }
+    L.st_a.release();
+    L.st_b.release();
+    L.ent.release();
+    L.c_tbl.release();
+    L.c_exp.release();
+}
 
 void f64tc_selftest(F64TcPlan& L, bool fail_waits, cudaStream_t s) {
     const int v = fail_waits ? 1 : 0;

@@ -171,8 +171,16 @@ void trim_pool(uint64_t keep_bytes) {
     DBG_CK(cudaMemPoolTrimTo(pool, (size_t)keep_bytes));
 }
 
+static std::atomic<int64_t> g_pool_limit{0};
+
 void pool_alloc(void** p, size_t bytes, cudaStream_t s) {
     cudaMemPool_t pool = library_pool();
+    if (const int64_t limit = g_pool_limit.load(std::memory_order_relaxed)) {
+        uint64_t used = 0;
+        DBG_CK(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+        if ((int64_t)(used + bytes) > limit)
+            fail(DBCSR_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes: past the pool's limit");
+    }
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         (void)cudaGetLastError();
@@ -713,6 +721,13 @@ dbcsr_status dbcsr_create(dbcsr_matrix* out, int32_t nblk, const int32_t* blk_si
             throw;
         }
         *out = m;
+    });
+}
+
+int32_t dbcsr_pool_limit(int64_t bytes) {
+    return guarded([&] {
+        if (bytes < 0) fail(DBCSR_EINVAL, "pool_limit: negative limit");
+        dbg::g_pool_limit.store(bytes);
     });
 }
 

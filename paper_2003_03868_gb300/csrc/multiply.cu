@@ -1274,8 +1274,16 @@ void symmetrize(dbcsr_matrix_* m) {
     m->exact_sym = true;
 }
 
-void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbcsr_matrix_* C, double eps, int prec,
-              dbcsr_mult_stats* stats, bool want_dev2, int sym_result, MultPlan* plan, double tc_min_flops) {
+namespace {
+
+// How far a product got: whether it uses the FP64 tensor-core tiles, and whether C has the new arrays.
+struct MultProgress {
+    bool tc = false, installed = false;
+};
+
+void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbcsr_matrix_* C, double eps, int prec,
+                   dbcsr_mult_stats* stats, bool want_dev2, int sym_result, MultPlan* plan, double tc_min_flops,
+                   MultProgress& progress) {
     check_finalized(A);
     check_finalized(B);
     if (!C) fail(DBCSR_EINVAL, "multiply: null C");
@@ -1392,6 +1400,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     const int64_t nform = hk[0];
     // FP64 products of at least tc_min_flops may use the tensor cores (fp64tc.cu decides per block)
     bool tc = !bf16 && nform && (double)(unsigned long long)hk[1] >= tc_min_flops;
+    progress.tc = tc;
     if (tc && !groups) {
         groups = build_groups(A);
         A->groups = groups;
@@ -1503,6 +1512,11 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     c_data.alloc(std::max<int64_t>(nel, 1), s);
     c_norm.alloc(nf1, s);
     c_dev2.alloc(nf1, s);
+    DBuf<double> an, bn;                    // a plan's operands' block norms at an execution
+    if (plan && tc) {
+        an.alloc(std::max<int64_t>(A->nnzb, 1), s);
+        bn.alloc(std::max<int64_t>(B->nnzb, 1), s);
+    }
     // kept by a plan: the shape lists, the tensor-core tier's patterns and the launch sequence
     DBuf<int64_t> list;
     SmmArgs sa{};
@@ -1644,8 +1658,10 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
     if (!plan) {
         prod_a.release();
         prod_b.release();
+        if (tcp) f64tc_release(*tcp);                // room for the filter's compaction
     }
 
+    progress.installed = true;
     // install the formed blocks as C (A or B may alias C: every read above is queued before)
     C->rp = std::move(f_rp);
     C->row = std::move(f_row);
@@ -1673,12 +1689,7 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         zero_small(s);
         if (lt) lowtier_check(*lt, s);
         if (tcp) f64tc_check(*tcp, s);
-        DBuf<double> an, bn;                       // the operands' block norms at an execution
         const F64TcBlocks f64tc_blocks{C->row.p, C->col.p, mirror.p, f_ksum.p, nullptr, nullptr, f_comp.p, sym_result, by_group};
-        if (tc) {
-            an.alloc(std::max<int64_t>(A->nnzb, 1), s);
-            bn.alloc(std::max<int64_t>(B->nnzb, 1), s);
-        }
         // captured on a private stream (the legacy default stream cannot be captured); the
         // graph is launched on C's stream
         SideStreams side;
@@ -1810,6 +1821,21 @@ void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbc
         stats->bytes_tensor = lt ? lowtier_copy_bytes(*lt) : 0.0;
         stats->n_tiles = lt ? lowtier_tiles(*lt) : tcp ? f64tc_tiles(*tcp) : 0;
     }
+}
+
+}  // namespace
+
+void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbcsr_matrix_* C, double eps, int prec,
+              dbcsr_mult_stats* stats, bool want_dev2, int sym_result, MultPlan* plan, double tc_min_flops) {
+    MultProgress progress;
+    try {
+        multiply_once(alpha, A, B, beta, C, eps, prec, stats, want_dev2, sym_result, plan, tc_min_flops, progress);
+        return;
+    } catch (const Error& e) {
+        if (e.code != DBCSR_ENOMEM || !progress.tc || progress.installed) throw;
+    }
+    // no room for the digit tiles beside the rest: every block on the FP64 pipe, which needs none
+    multiply_once(alpha, A, B, beta, C, eps, prec, stats, want_dev2, sym_result, plan, HUGE_VAL, progress);
 }
 
 void execute_plan(MultPlan* plan) {

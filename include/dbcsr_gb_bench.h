@@ -53,7 +53,9 @@ int32_t dbcsr_pool_limit(int64_t bytes);
  * one CTA waits on an mbarrier for at most limit_cycles SM clock cycles (limit_cycles >= 0).
  * arrive != 0: a thread of the CTA arrives first, so the wait completes (DBCSR_OK);
  * arrive == 0: nothing ever arrives, the wait runs out and the call returns DBCSR_ETIMEOUT,
- * the context staying usable.  *waited (nullable) receives the cycles the wait took.
+ * the context staying usable; arrive == 2: the wait of the warp's first lane runs out (the other lanes
+ * may wait 64 times as long, and another warp arrives after four times), and so does the warp's as a
+ * whole (DBCSR_ETIMEOUT; DBCSR_ECUDA if the lanes disagreed; limit_cycles at most 2^32).  *waited (nullable) receives the cycles the wait took.
  */
 int32_t dbcsr_wait_selftest(int64_t limit_cycles, int32_t arrive, int64_t* waited);
 

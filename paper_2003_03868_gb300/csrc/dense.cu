@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(32 * (2 + (SPLIT ? kTConvWarps : 0) + kDEpiWar
         for (int64_t tile = blockIdx.x; tile < D.ntiles && ok; tile += gridDim.x, ++k) {
             const uint32_t buf = k & 1u;
             const uint32_t d = tc::uniform(tmem + buf * kDNMax);
-            ok = tc::mbar_wait(&S.acc_empty[buf], ((k >> 1) & 1u) ^ 1u, kDWaitLimit);
+            ok = tc::mbar_wait_warp(&S.acc_empty[buf], ((k >> 1) & 1u) ^ 1u, kDWaitLimit);
             uint32_t acc = 0;
             for (int s = 0; s < nstage && ok; ++s) {
                 ok = tc::mbar_wait(SPLIT ? &S.conv[slot] : &S.full[slot], phase, kDWaitLimit) && !aborted();

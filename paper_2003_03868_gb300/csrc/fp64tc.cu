@@ -825,7 +825,7 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                 const int nd = (int)tc::uniform(((unsigned)en.w >> qs) & 255u);
                 const uint32_t buf = n & 1u;
                 const uint32_t d = tc::uniform(tmem + buf * 256u);
-                ok = tc::mbar_wait(&S.acc_empty[buf], ((n >> 1) & 1u) ^ 1u, kOzWait);
+                bool mine = tc::mbar_wait(&S.acc_empty[buf], ((n >> 1) & 1u) ^ 1u, kOzWait);
                 // two K steps at a time where there are two: an MMA's issue waits until the tensor cores
                 // are nearly through with the ones before it, so what lies between two batches of
                 // MMAs leaves them idle
@@ -834,15 +834,14 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                     const int st0 = stage, st1 = stage + 1 == kOzStages ? 0 : stage + 1;
                     mask &= mask - 1;
                     const bool two = mask != 0;
-                    ok = tc::mbar_wait(&S.full[st0], phase, kOzWait);
-                    if (two && ok) ok = tc::mbar_wait(&S.full[st1], phase ^ (st1 == 0 ? 1u : 0u), kOzWait);
-                    if (!ok) break;
-                    mask &= mask - 1;
-                    tc::fence_after_sync();
                     const uint32_t sa0 = tc::uniform(s0 + (uint32_t)st0 * (kOzStage / 16));
                     const uint32_t sa1 = tc::uniform(s0 + (uint32_t)st1 * (kOzStage / 16));
+                    mine = mine && tc::mbar_wait(&S.full[st0], phase, kOzWait);
+                    if (two) mine = mine && tc::mbar_wait(&S.full[st1], phase ^ (st1 == 0 ? 1u : 0u), kOzWait);
+                    mask &= mask - 1;
+                    tc::fence_after_sync();
                     constexpr uint32_t b_off = kOzA / 16, b_lbo = (uint32_t)(kOzBChunk / 16) << 16;
-                    if (tc::elect_one()) {
+                    if (tc::elect_one() && mine) {
                         if (first) oz_issue<true>(nd, d, sa0 | a_lbo, a_step, (sa0 + b_off) | b_lbo);
                         else oz_issue<false>(nd, d, sa0 | a_lbo, a_step, (sa0 + b_off) | b_lbo);
                         tc::mma_commit(&S.empty[st0]);
@@ -852,7 +851,9 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                         }
                         if (!mask) tc::mma_commit(&S.acc_full[buf]);
                     }
-                    __syncwarp();
+                    // the lanes stay together, see mbar_wait_warp (the vote behind the MMAs: before them it took the
+                    // kernel 2% longer; what the elected lane's own waits allowed may run)
+                    ok = __all_sync(0xffffffffu, mine);
                     first = false;
                     stage += two ? 2 : 1;
                     if (stage >= kOzStages) {
@@ -862,7 +863,6 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                 }
                 ++n;
             }
-            ok = __all_sync(0xffffffffu, ok);
             if (!ok && lane == 0) oz_fail(A, S);
         }
         // every MMA has completed before the TMEM is released

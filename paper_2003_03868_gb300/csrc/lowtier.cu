@@ -195,8 +195,8 @@ std::shared_ptr<Groups> groups_of(const std::vector<int32_t>& root, const std::v
     return g;
 }
 
-std::shared_ptr<Groups> groups_of_rows(const Groups& g, const std::vector<int32_t>& rows, const std::vector<int32_t>& bs,
-                                       cudaStream_t s) {
+std::shared_ptr<Groups> groups_of_rows(const Groups& g, const std::vector<int32_t>& rows,
+                                       const std::vector<int32_t>& bs, cudaStream_t s) {
     std::vector<int32_t> first(g.ngrp, -1), root(rows.size());
     for (size_t i = 0; i < rows.size(); ++i) {
         int32_t& f = first[g.h_of[rows[i]]];
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
             const uint32_t sa_step = (uint32_t)np * 2u * ra, sb_step = (uint32_t)np * 2u * rb;
             const uint32_t idesc = tc::uniform(tc::instr_desc(1, kTileRows, ((wc + 15) >> 4) << 4));
             const uint32_t d_tmem = tc::uniform(tmem + (uint32_t)(acc * 128));
-            ok = tc::mbar_wait(&S.acc_empty[acc], acc_phase ^ 1u, kWaitLimit);
+            ok = tc::mbar_wait_warp(&S.acc_empty[acc], acc_phase ^ 1u, kWaitLimit);
             tc::fence_after_sync();
             uint32_t accumulate = 0;
             const int64_t e0 = A.s_ptr[t], e1 = A.s_ptr[t + 1];
@@ -569,12 +569,11 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                     while (mask) {
                         int len;
                         lt_next_run(mask, len);
-                        ok = tc::mbar_wait(&S.full[stage], phase, kWaitLimit);
-                        if (!ok) break;
-                        tc::fence_after_sync();
                         const uint32_t s0 = tc::uniform(s_base + (uint32_t)stage * (kStageBytesMax / 16));
                         const uint32_t n = tc::uniform((uint32_t)len);
-                        if (tc::elect_one()) {
+                        const bool mine = tc::mbar_wait(&S.full[stage], phase, kWaitLimit);
+                        tc::fence_after_sync();
+                        if (tc::elect_one() && mine) {
                             for (uint32_t j = 0; j < n; ++j) {
                                 const uint32_t ah = (s0 + j * sa_step) | (ra << 16);
                                 const uint32_t bh = (s0 + n * sa_step + j * sb_step) | (rb << 16);
@@ -586,7 +585,9 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                             }
                             tc::mma_commit(&S.empty[stage]);         // the stage is free once these MMAs ran
                         }
-                        __syncwarp();
+                        // the lanes stay together, see mbar_wait_warp (behind the MMAs, off their way)
+                        ok = __all_sync(0xffffffffu, mine);
+                        if (!ok) break;
                         accumulate = 1;
                         if (++stage == kStages) {
                             stage = 0;
@@ -595,7 +596,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                     }
                 }
             }
-            ok = __all_sync(0xffffffffu, ok) && !__shfl_sync(0xffffffffu, lt_aborted(S), 0);
+            ok = ok && !__shfl_sync(0xffffffffu, lt_aborted(S), 0);
             if (!ok && lane == 0) lt_fail(A, S);
             if (tc::elect_one()) tc::mma_commit(&S.acc_full[acc]);    // the accumulator is complete
             __syncwarp();

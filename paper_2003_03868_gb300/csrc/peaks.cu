@@ -80,9 +80,9 @@ double bench_peak(int kind, int iters, int blocks, int threads) {
     return ops / (ms * 1e-3) * 1e-9;
 }
 
-// One warp: an mbarrier of count 1, thread 0 arrives first when `arrive`, then every lane
-// waits (bounded, as the library's kernels do) for the first phase.  out[0] = 1 if the wait
-// completed, out[1] = the cycles lane 0 waited.  No asynchronous copy or TMEM is involved,
+// One warp: an mbarrier of count 1, thread 0 arrives first when `arrive`, then the warp waits (bounded, as
+// the library's kernels do) for the first phase; arrive == 2: see dbcsr_wait_selftest.  out[0] = the lanes in
+// which the wait completed, out[1] = the cycles lane 0 waited.  No asynchronous copy or TMEM is involved,
 // so giving up leaves nothing in flight.
 __global__ void k_wait_selftest(long long limit, int arrive, int64_t* out) {
     __shared__ uint64_t bar;
@@ -91,11 +91,20 @@ __global__ void k_wait_selftest(long long limit, int arrive, int64_t* out) {
         tc::fence_barrier_init();
     }
     __syncthreads();
-    if (arrive && threadIdx.x == 0) tc::mbar_arrive(&bar);
+    if (arrive && arrive != 2 && threadIdx.x == 0) tc::mbar_arrive(&bar);
     const long long t0 = clock64();
-    const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&bar, 0, limit));
+    if (threadIdx.x >= 32) {
+        // arrive == 2: after lane 0's wait ran out, before the others' would
+        if (arrive == 2 && threadIdx.x == 32) {
+            while (clock64() - t0 < 4 * limit) {}
+            tc::mbar_arrive(&bar);
+        }
+        return;
+    }
+    const bool ok = tc::mbar_wait_warp(&bar, 0, arrive == 2 && threadIdx.x ? 64 * limit : limit);
+    const int n = __popc(__ballot_sync(0xffffffffu, ok));
     if (threadIdx.x == 0) {
-        out[0] = ok ? 1 : 0;
+        out[0] = n;
         out[1] = clock64() - t0;
     }
 }
@@ -117,9 +126,10 @@ int64_t dbcsr_launch_count(void) { return dbg::g_launches.load(); }
 int32_t dbcsr_wait_selftest(int64_t limit_cycles, int32_t arrive, int64_t* waited) {
     try {
         if (limit_cycles < 0) dbg::fail(DBCSR_EINVAL, "wait_selftest: negative limit");
+        if (arrive == 2 && limit_cycles > (1ll << 32)) dbg::fail(DBCSR_EINVAL, "wait_selftest: limit too long");
         int64_t* d = nullptr;
         DBG_CK(cudaMalloc(&d, 2 * sizeof(int64_t)));
-        dbg::k_wait_selftest<<<1, 32>>>((long long)limit_cycles, arrive, d);
+        dbg::k_wait_selftest<<<1, 64>>>((long long)limit_cycles, arrive, d);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         int64_t h[2] = {0, 0};
@@ -128,6 +138,7 @@ int32_t dbcsr_wait_selftest(int64_t limit_cycles, int32_t arrive, int64_t* waite
         DBG_CK(e);
         if (waited) *waited = h[1];
         if (!h[0]) dbg::fail(DBCSR_ETIMEOUT, "wait_selftest: the wait ran out");
+        if (h[0] != 32) dbg::fail(DBCSR_ECUDA, "wait_selftest: the lanes disagree");
         dbg::set_last_error("");
         return DBCSR_OK;
     } catch (const dbg::Error& e) {

@@ -63,6 +63,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     }
 }
 
+// The same for a converged warp: false in every lane when the limit ran out in any, so that the lanes stay
+// together (the lanes' clocks and polls differ: near the limit one may give up where another sees the phase).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, long long limit) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit));
+}
+
 // ---------------------------------------------------------------- bulk copies
 // bytes (a multiple of 16) from global src to shared dst, both 16-byte aligned; completion
 // is signalled on bar as transaction bytes.

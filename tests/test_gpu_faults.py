@@ -65,3 +65,14 @@ def test_non_finite_hamiltonian_stops_the_sign_iteration(gb, bad):
     assert e.value.status in (gb._ffi.DBCSR_EINVAL, gb._ffi.DBCSR_ENAN)
     assert "not finite" in str(e.value)
 
+
+
+def test_a_warp_gives_up_a_wait_in_all_lanes_or_none(gb):
+    # a role of a kernel that waits with its whole warp must not fall apart when the limit runs out in one
+    # lane only: the lanes go on to instructions that need all of them
+    lib = gb.lib()
+    waited = C.c_int64(0)
+    limit = 500_000
+    assert lib.dbcsr_wait_selftest(limit, 2, C.byref(waited)) == gb._ffi.DBCSR_ETIMEOUT
+    assert 4 * limit <= waited.value < 64 * limit
+    assert lib.dbcsr_wait_selftest(limit, 1, C.byref(waited)) == gb._ffi.DBCSR_OK

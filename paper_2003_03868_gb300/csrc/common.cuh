@@ -301,6 +301,10 @@ void execute_plan(MultPlan* plan);
 void check_unplanned(const dbcsr_matrix_* m, const char* where);
 
 // ---- lowtier.cu
+// The groups a matrix keeps.  Products of several threads may share an operand, and the first one that
+// needs groups keeps them there: they are read and replaced as one.
+inline std::shared_ptr<Groups> kept_groups(const dbcsr_matrix_* m) { return std::atomic_load(&m->groups); }
+inline void keep_groups(dbcsr_matrix_* m, std::shared_ptr<Groups> g) { std::atomic_store(&m->groups, std::move(g)); }
 // Groups of neighbouring blocks from the strongest couplings (block norms) of m.
 std::shared_ptr<Groups> build_groups(dbcsr_matrix_* m);
 std::shared_ptr<Groups> groups_of(const std::vector<int32_t>& root, const std::vector<int32_t>& bs, cudaStream_t s);

@@ -1311,10 +1311,11 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
 
     // BF16 products run on the tensor-core tier, on groups of blocks (kept with the matrices)
     const bool bf16 = is_bf16(prec);
-    std::shared_ptr<Groups> groups = A->groups ? A->groups : B->groups;
+    std::shared_ptr<Groups> groups = kept_groups(A);
+    if (!groups) groups = kept_groups(B);
     if (bf16 && (!groups || groups->nblk != nblk)) {
         groups = build_groups(A);
-        A->groups = groups;
+        keep_groups(A, groups);
     }
     if (groups && groups->nblk != nblk) groups.reset();
 
@@ -1403,7 +1404,7 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
     progress.tc = tc;
     if (tc && !groups) {
         groups = build_groups(A);
-        A->groups = groups;
+        keep_groups(A, groups);
     }
     const int32_t* grp = (bf16 || tc) ? groups->g_of.p : nullptr;
     // which twin of a mirrored pair is computed.  In X X with X exactly symmetric both are the same
@@ -1673,7 +1674,7 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
     C->norms = std::move(c_norm);
     C->norms_valid = true;
     C->finalized = true;
-    if (groups) C->groups = groups;
+    if (groups) keep_groups(C, groups);
     C->exact_sym = sym_result != kSymNone;
 
     if (plan) {

@@ -87,6 +87,9 @@ inline void allow_dyn_smem(K kernel, size_t dyn) {
 // memory cached (release threshold = max) so that the per-product stacks and
 // matrices are not unmapped at every host synchronisation and mapped again.
 cudaMemPool_t library_pool();
+// A stream of the library's own on the current device, never destroyed: for memory that may outlive its
+// creator's stream.
+cudaStream_t library_stream();
 // Waits for the device, then returns cached pool memory above keep_bytes to the driver.
 void trim_pool(uint64_t keep_bytes);
 // Stream-ordered allocation from library_pool().  When the device is out of memory the
@@ -157,6 +160,8 @@ HostScalars& host_scalars();
 constexpr int kGroupWidth = 112;
 constexpr int kGroupMembers = 16;
 constexpr int32_t kMaxBlockRowsLt = 262144;
+// Several matrices share them, each on a stream of its own that may be gone before the others: their arrays are
+// freed on library_stream().  (Every product waits for its kernels that read them.)
 struct Groups {
     int32_t ngrp = 0, nblk = 0, max_members = 0;
     std::vector<int32_t> h_w;            // host copies of the widths and of g_of

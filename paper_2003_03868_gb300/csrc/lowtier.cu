@@ -192,6 +192,8 @@ std::shared_ptr<Groups> groups_of(const std::vector<int32_t>& root, const std::v
     DBG_CK(cudaMemcpyAsync(g->g_mem.p, g_mem.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, s));
     DBG_CK(cudaMemcpyAsync(g->g_w.p, g_w.data(), sizeof(int32_t) * ng, cudaMemcpyHostToDevice, s));
     DBG_CK(cudaStreamSynchronize(s));           // the host vectors go out of scope
+    for (DBuf<int32_t>* b : {&g->g_of, &g->g_pos, &g->g_ptr, &g->g_mem, &g->g_w, &g->g_mrec, &g->g_midx})
+        b->s = library_stream();
     return g;
 }
 

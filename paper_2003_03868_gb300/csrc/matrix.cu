@@ -158,6 +158,17 @@ void copy_with_host(const HostCopy* c, int n, bool to_host, cudaStream_t s) {
     DBG_LAUNCH_CK();
 }
 
+cudaStream_t library_stream() {
+    static std::mutex mu;
+    static auto* streams = new std::map<int, cudaStream_t>();   // (outlives every static destructor)
+    int dev = 0;
+    DBG_CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    cudaStream_t& s = (*streams)[dev];
+    if (!s) DBG_CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    return s;
+}
+
 void trim_pool(uint64_t keep_bytes) {
     int dev = 0;
     DBG_CK(cudaGetDevice(&dev));

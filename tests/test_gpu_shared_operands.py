@@ -53,3 +53,30 @@ def test_first_products_of_several_threads_on_one_operand(gb):
         ref = ref or out[0]
         for o in out:
             assert all(np.array_equal(x, y) for x, y in zip(o, ref))
+
+
+def test_results_outlive_their_operand_and_its_stream(gb):
+    # a product's result shares its operand's groups: they stay usable, and can be freed, when the operand and
+    # the stream it was made on are gone
+    import torch
+    rt = torch.cuda.cudart()
+    h = synth.build_hamiltonian(synth.small(40, seed=2501)).H
+    H = gb.Matrix.of(h)
+    for _ in range(3):
+        handle = torch.zeros(1, dtype=torch.int64)
+        assert int(rt.cudaStreamCreate(handle.data_ptr())) == 0
+        A = gb.Matrix.of(h, int(handle[0]))
+        C = gb.Matrix(H.blk_size, H.stream)
+        assert gb.multiply(1.0, A, H, 0.0, C, 1e-7).n_tiles > 0
+        A.close()
+        assert int(rt.cudaStreamDestroy(int(handle[0]))) == 0
+        D, E = gb.Matrix(H.blk_size, H.stream), gb.Matrix(H.blk_size, H.stream)
+        assert gb.multiply(1.0, C, H, 0.0, D, 1e-7).n_tiles > 0
+        fresh = gb.Matrix.from_blocks(C.blk_size, *C.export())
+        gb.multiply(1.0, fresh, H, 0.0, E, 1e-7)
+        (rp, col, x), (rp2, col2, y) = D.export(), E.export()
+        # the groups of the two differ (H's couplings and the product's): equal to the rounding of 920 terms
+        assert np.array_equal(rp, rp2) and np.array_equal(col, col2)
+        assert np.linalg.norm(x - y) <= 920 * 2.0 ** -53 * np.linalg.norm(y)
+        C.close()
+        D.close()

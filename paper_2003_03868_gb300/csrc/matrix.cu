@@ -84,24 +84,74 @@ constexpr int64_t kHostCopyPiece = 1 << 16;          // bytes a CTA copies at a 
 struct HostCopyArgs {
     HostCopy c[kHostCopies];
     int n;
+    bool to_host;
 };
+
+// 16 bytes to or from a device address that is a multiple of kGrain bytes.
+template <int kGrain>
+__device__ __forceinline__ int4 load16(const char* p) {
+    int4 v;
+    if (kGrain == 16) {
+        v = *reinterpret_cast<const int4*>(p);
+    } else if (kGrain == 8) {
+        const int2 a = *reinterpret_cast<const int2*>(p), b = *reinterpret_cast<const int2*>(p + 8);
+        v = make_int4(a.x, a.y, b.x, b.y);
+    } else {
+        const int* q = reinterpret_cast<const int*>(p);
+        v = make_int4(q[0], q[1], q[2], q[3]);
+    }
+    return v;
+}
+template <int kGrain>
+__device__ __forceinline__ void store16(char* p, int4 v) {
+    if (kGrain == 16) {
+        *reinterpret_cast<int4*>(p) = v;
+    } else if (kGrain == 8) {
+        *reinterpret_cast<int2*>(p) = make_int2(v.x, v.y);
+        *reinterpret_cast<int2*>(p + 8) = make_int2(v.z, v.w);
+    } else {
+        int* q = reinterpret_cast<int*>(p);
+        q[0] = v.x;
+        q[1] = v.y;
+        q[2] = v.z;
+        q[3] = v.w;
+    }
+}
+// bytes (a multiple of 16); the host's side on a 16-byte boundary.
+template <int kGrain>
+__device__ __forceinline__ void copy_pieces(const char* src, char* dst, int64_t bytes, bool to_host) {
+    for (int64_t p = (int64_t)blockIdx.x * kHostCopyPiece; p < bytes; p += (int64_t)gridDim.x * kHostCopyPiece) {
+        const int64_t e = min(p + kHostCopyPiece, bytes);
+        for (int64_t x = p + 16 * threadIdx.x; x < e; x += 16 * kHostCopyThreads) {
+            if (to_host) store16<16>(dst + x, load16<kGrain>(src + x));
+            else store16<kGrain>(dst + x, load16<16>(src + x));
+        }
+    }
+}
 
 // Arrays to or from pinned host memory.  Both ends run at the link's rate (193 GB/s to the host), but the
 // first access to a host page after other work waits for its translation, and the copy engine takes
 // these waits one after another: 1.1 GB of a density matrix took 28 to 52 ms after a sign iteration
 // (5.6 when repeated), this kernel, with the accesses of 152 CTAs in flight, 5.6 to 8.5 ms.
+// The host's side is taken in whole 128-byte lines, 16 bytes a thread, wherever it begins; the device's side
+// in what its alignment against that allows.
 __global__ void __launch_bounds__(kHostCopyThreads) k_host_copy(HostCopyArgs A) {
     for (int i = 0; i < A.n; ++i) {
         const char* src = static_cast<const char*>(A.c[i].src);
         char* dst = static_cast<char*>(A.c[i].dst);
         const int64_t bytes = A.c[i].bytes;                           // a multiple of 4
-        const bool wide = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
-        for (int64_t p = (int64_t)blockIdx.x * kHostCopyPiece; p < bytes; p += (int64_t)gridDim.x * kHostCopyPiece) {
-            const int64_t e = min(p + kHostCopyPiece, bytes), ew = wide ? e & ~(int64_t)15 : p;
-            for (int64_t x = p + 16 * threadIdx.x; x < ew; x += 16 * kHostCopyThreads)
-                *reinterpret_cast<int4*>(dst + x) = *reinterpret_cast<const int4*>(src + x);
-            for (int64_t x = ew + 4 * threadIdx.x; x < e; x += 4 * kHostCopyThreads)
-                *reinterpret_cast<int*>(dst + x) = *reinterpret_cast<const int*>(src + x);
+        const uintptr_t host = reinterpret_cast<uintptr_t>(A.to_host ? dst : src);
+        const int64_t head = min((int64_t)((0 - host) & 127), bytes), mid = (bytes - head) & ~(int64_t)15;
+        const uintptr_t dev = reinterpret_cast<uintptr_t>(A.to_host ? src : dst) + head;
+        if ((dev & 15) == 0) copy_pieces<16>(src + head, dst + head, mid, A.to_host);
+        else if ((dev & 7) == 0) copy_pieces<8>(src + head, dst + head, mid, A.to_host);
+        else copy_pieces<4>(src + head, dst + head, mid, A.to_host);
+        if (blockIdx.x == 0) {                                        // what lies before and after the lines
+            const int64_t rest = bytes - mid;
+            for (int64_t x = 4 * threadIdx.x; x < rest; x += 4 * kHostCopyThreads) {
+                const int64_t at = x < head ? x : mid + x;
+                *reinterpret_cast<int*>(dst + at) = *reinterpret_cast<const int*>(src + at);
+            }
         }
     }
 }
@@ -139,6 +189,7 @@ void* pinned_address(const void* p, int64_t bytes, bool write) {
 
 void copy_with_host(const HostCopy* c, int n, bool to_host, cudaStream_t s) {
     HostCopyArgs a{};
+    a.to_host = to_host;
     int64_t most = 0;
     for (int i = 0; i < n; ++i) {
         if (c[i].bytes <= 0) continue;

@@ -63,3 +63,24 @@ def test_export_and_put_values(gb, kind, nblk):
         for _, _, keep in bufs:
             if keep:
                 keep()
+
+
+# heads and tails around the 128-byte lines of the host's side: every offset of eight bytes in a line, arrays of
+# less than a line up to several
+@pytest.mark.parametrize("shift", [0, 1, 2, 7, 9, 15])
+def test_any_offset_in_a_line(gb, shift):
+    import torch
+    for nblk in (1, 2, 3, 4, 5, 9, 12, 130):
+        m = synth.random_block_matrix([1] * nblk, 1.0, 100 + nblk)
+        M = gb.Matrix.of(m)
+        rp, col, data = M.export()
+        whole = [torch.full((n + 40,), -7, dtype=t).pin_memory()
+                 for n, t in ((nblk + 1, torch.int64), (len(col), torch.int32), (len(data), torch.float64))]
+        view = [w[8 + shift:8 + shift + n] for w, n in zip(whole, (nblk + 1, len(col), len(data)))]
+        M.export_to(view[0].data_ptr(), view[1].data_ptr(), len(col), view[2].data_ptr(), len(data))
+        for w, v, ref in zip(whole, view, (rp, col, data)):
+            assert np.array_equal(v.numpy(), ref)
+            assert bool((w[:8 + shift] == -7).all()) and bool((w[8 + shift + len(ref):] == -7).all())
+        view[2].mul_(3.0)
+        M.put_values(view[2].numpy())
+        assert np.array_equal(M.export()[2], view[2].numpy())

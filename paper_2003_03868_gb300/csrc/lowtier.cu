@@ -84,62 +84,63 @@ __global__ void __launch_bounds__(256) k_top_couplings(int32_t nb, const int64_t
                                                        const int32_t* __restrict__ col,
                                                        const double* __restrict__ nrm, Coupling* __restrict__ out) {
     const int lane = threadIdx.x & 31;
-    const int32_t i = (int32_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
-    if (i >= nb) return;
     constexpr int32_t kNone = 0x7fffffff;
-    double w[kTop];
-    int32_t c[kTop];
+    const int32_t warps = (int32_t)(gridDim.x * (blockDim.x >> 5));
+    for (int32_t i = (int32_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); i < nb; i += warps) {
+        double w[kTop];
+        int32_t c[kTop];
 #pragma unroll
-    for (int k = 0; k < kTop; ++k) {
-        w[k] = -1.0;                     // below every norm
-        c[k] = kNone;
-    }
-    const int64_t q1 = rp[i + 1];
-    for (int64_t q = rp[i] + lane; q < q1; q += 32) {
-        int32_t nc = col[q];
-        if (nc == i) continue;
-        double nw = nrm[q];
-        if (!stronger(nw, nc, w[kTop - 1], c[kTop - 1])) continue;
+        for (int k = 0; k < kTop; ++k) {
+            w[k] = -1.0;                     // below every norm
+            c[k] = kNone;
+        }
+        const int64_t q1 = rp[i + 1];
+        for (int64_t q = rp[i] + lane; q < q1; q += 32) {
+            int32_t nc = col[q];
+            if (nc == i) continue;
+            double nw = nrm[q];
+            if (!stronger(nw, nc, w[kTop - 1], c[kTop - 1])) continue;
 #pragma unroll
-        for (int k = 0; k < kTop; ++k) {  // insertion: the displaced entry moves down
-            if (stronger(nw, nc, w[k], c[k])) {
-                const double tw = w[k];
-                const int32_t tc = c[k];
-                w[k] = nw;
-                c[k] = nc;
-                nw = tw;
-                nc = tc;
+            for (int k = 0; k < kTop; ++k) {  // insertion: the displaced entry moves down
+                if (stronger(nw, nc, w[k], c[k])) {
+                    const double tw = w[k];
+                    const int32_t tc = c[k];
+                    w[k] = nw;
+                    c[k] = nc;
+                    nw = tw;
+                    nc = tc;
+                }
             }
         }
-    }
-    Coupling* o = out + (size_t)i * kTop;
-    int r = 0;
-    for (; r < kTop; ++r) {
-        double bw = w[0];
-        int32_t bc = c[0];
+        Coupling* o = out + (size_t)i * kTop;
+        int r = 0;
+        for (; r < kTop; ++r) {
+            double bw = w[0];
+            int32_t bc = c[0];
 #pragma unroll
-        for (int sh = 16; sh; sh >>= 1) {
-            const double ow = __shfl_xor_sync(0xffffffffu, bw, sh);
-            const int32_t oc = __shfl_xor_sync(0xffffffffu, bc, sh);
-            if (stronger(ow, oc, bw, bc)) {
-                bw = ow;
-                bc = oc;
+            for (int sh = 16; sh; sh >>= 1) {
+                const double ow = __shfl_xor_sync(0xffffffffu, bw, sh);
+                const int32_t oc = __shfl_xor_sync(0xffffffffu, bc, sh);
+                if (stronger(ow, oc, bw, bc)) {
+                    bw = ow;
+                    bc = oc;
+                }
+            }
+            if (bc == kNone) break;          // the same on every lane
+            if (lane == 0) o[r] = Coupling{bw, min(i, bc), max(i, bc)};
+            if (c[0] == bc) {                // the one lane that held it (columns are unique in a row)
+#pragma unroll
+                for (int k = 0; k + 1 < kTop; ++k) {
+                    w[k] = w[k + 1];
+                    c[k] = c[k + 1];
+                }
+                w[kTop - 1] = -1.0;
+                c[kTop - 1] = kNone;
             }
         }
-        if (bc == kNone) break;          // the same on every lane
-        if (lane == 0) o[r] = Coupling{bw, min(i, bc), max(i, bc)};
-        if (c[0] == bc) {                // the one lane that held it (columns are unique in a row)
-#pragma unroll
-            for (int k = 0; k + 1 < kTop; ++k) {
-                w[k] = w[k + 1];
-                c[k] = c[k + 1];
-            }
-            w[kTop - 1] = -1.0;
-            c[kTop - 1] = kNone;
-        }
+        if (lane == 0)
+            for (; r < kTop; ++r) o[r] = Coupling{0.0, -1, -1};
     }
-    if (lane == 0)
-        for (; r < kTop; ++r) o[r] = Coupling{0.0, -1, -1};
 }
 
 }  // namespace

@@ -103,3 +103,17 @@ def test_groups_need_a_finalized_matrix(gb):
     with pytest.raises(gb.DbcsrError) as e:
         M.groups()
     assert e.value.status == gb._ffi.DBCSR_ESTATE
+
+
+def test_groups_of_more_rows_than_one_pass_of_the_grid(gb):
+    # the couplings' kernel runs 64 CTAs of eight rows per SM at most: 77,824 rows on 152 SMs
+    nb = 80011
+    i = np.arange(nb, dtype=np.int64)
+    rows = np.concatenate([i, i[1:], i[:-1]])
+    cols = np.concatenate([i, i[1:] - 1, i[:-1] + 1])
+    order = np.lexsort((cols, rows))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=nb))])
+    data = np.random.default_rng(9).uniform(0.1, 1.0, len(rows))
+    M = gb.Matrix.from_blocks(np.ones(nb, np.int32), rp, cols[order].astype(np.int32), data)
+    g_of = _check(gb, M, np.ones(nb, np.int32))
+    assert np.bincount(g_of)[g_of[-1]] > 1

@@ -272,6 +272,7 @@ struct F64TcPlan;
 // One-off and planned products below this many flops (counted over both triangles) stay on the FP64
 // pipe: such a product is launch-bound on either path, and the tensor cores' needs more launches.
 constexpr double kTcMinFlops = 64e6;
+constexpr double kGroupFlops = 0.5e6;
 // m <- (m + m^T) / 2 on the blocks that have a twin; blocks without one are dropped.
 void symmetrize(dbcsr_matrix_* m);
 void mark_if_symmetric(dbcsr_matrix_* m);
@@ -293,9 +294,11 @@ struct MultPlan {
     F64TcPlan* tc = nullptr;             // FP64 products: the digit tiles of the tensor-core blocks
     ~MultPlan();
 };
-// tc_min_flops: FP64 products of fewer flops do not use the tensor cores.  The iterations leave it
-// at 0: the choice then depends on each tile alone, and a system's products are the same sums in
-// a batch as on their own.
+// tc_min_flops: FP64 products of fewer flops do not use the tensor cores, nor do those whose operands
+// have no block groups yet and fewer than kGroupFlops flops a block row (grouping takes 0.3 to 0.7 us a
+// block row on the host: 60,000 blocks of 5 in a band of nine took 43 ms with it and 5.7 without).  The
+// iterations leave it at 0: the choice then depends on each tile alone, and a system's products are the same
+// sums in a batch as on their own.
 // plan: build a plan instead of a one-off product (beta = 0, C distinct from A and B, no
 // symmetric result); C then holds the formed pattern with blocks under eps zeroed.
 void multiply(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta, dbcsr_matrix_* C, double eps,
@@ -357,11 +360,12 @@ struct F64TcBlocks {
 void f64tc_delete(F64TcPlan* p);
 // Tile patterns, stacks and digit tiles of C = alpha A B and the blocks the tensor cores take;
 // null when the product does not fit them (then comp is not complete).  planned: the tiles serve later
-// values of A and B too, so nothing is taken from the values these have now.
+// values of A and B too, so nothing is taken from the values these have now.  weigh: null as well when the
+// tiles cost more than they save.
 std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A, dbcsr_matrix_* B,
                                                                std::shared_ptr<Groups> groups, int64_t nform,
                                                                const int64_t* f_rp, const F64TcBlocks& f, double alpha,
-                                                               bool planned, cudaStream_t s);
+                                                               bool planned, bool weigh, cudaStream_t s);
 // The current values into the digit tiles (f64tc_prepare has done it for its values).
 void f64tc_pack(F64TcPlan& L, const dbcsr_matrix_* A, const dbcsr_matrix_* B, cudaStream_t s);
 // After f64tc_pack of a planned product's new values: the tensor-core blocks that need the FP64 pipe with

@@ -273,15 +273,23 @@ __device__ __forceinline__ bool oz_pays(int64_t entries, int width, unsigned lon
     const int slices = (width + kSlice - 1) / kSlice;
     return (double)entries * (kGroupWidth / 16) * slices * kStepClocks * kSimtFlopsPerClock <= (double)flops;
 }
-// Tiles for which the tensor cores pay: without one nothing is packed.
+// Flops of the tiles for which the tensor cores pay.
 __global__ void k_oz_pays(int64_t nt, const int64_t* __restrict__ s_ptr, const int32_t* __restrict__ c_tcol,
                           const int32_t* __restrict__ g_w, const unsigned long long* __restrict__ flops,
-                          unsigned long long* __restrict__ count) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool pays = t < nt && oz_pays(s_ptr[t + 1] - s_ptr[t], g_w[c_tcol[t]], flops[t]);
-    const int n = __syncthreads_count(pays);
-    if (threadIdx.x == 0 && n) atomicAdd(count, (unsigned long long)n);
+                          unsigned long long* __restrict__ sum) {
+    unsigned long long f = 0;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nt; t += (int64_t)gridDim.x * blockDim.x)
+        if (oz_pays(s_ptr[t + 1] - s_ptr[t], g_w[c_tcol[t]], flops[t])) f += flops[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    if ((threadIdx.x & 31) == 0 && f) atomicAdd(sum, f);
 }
+// Without such tiles nothing is packed.  Nor is it, in a product that need not take the same path in a batch
+// (weigh), when packing the operands' tiles takes longer than the FP64 pipe needs for those blocks: tiles of a
+// pattern without neighbourhoods hold a block or two each in 200 KB of digits, of which a quarter or less (the K
+// steps in use) is written at 4 TB/s (3,000 blocks of 13 with 20 random ones a row: 16.9 ms with the tiles, for a
+// few of its 5.8 GF, 12.8 without, 11.0 if the blocks need not be grouped).
+constexpr double kPackBytesPerSecond = 16e12, kSimtFlopsPerSecond = 1e12;
 
 // A computed block runs on the tensor cores (comp = 2) unless
 //   * its tile's tensor-core time (every stack entry at full width; a rule on the tile alone, so
@@ -1169,7 +1177,7 @@ void oz_depth(F64TcPlan& L, cudaStream_t s) {
 std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A, dbcsr_matrix_* B,
                                                                std::shared_ptr<Groups> groups, int64_t nform,
                                                                const int64_t* f_rp, const F64TcBlocks& f, double alpha,
-                                                               bool planned, cudaStream_t s) {
+                                                               bool planned, bool weigh, cudaStream_t s) {
     std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> P(nullptr, f64tc_delete);
     if (groups->ngrp > kMaxBlockRowsLt || !nform) return P;
     std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> up(new F64TcPlan(), f64tc_delete);
@@ -1233,15 +1241,16 @@ std::unique_ptr<F64TcPlan, void (*)(F64TcPlan*)> f64tc_prepare(dbcsr_matrix_* A,
     DBG_LAUNCH_CK();
     L.next.alloc(1, s);
     L.next.zero();
-    k_oz_pays<<<(unsigned)ceil_div(L.cp.nt, 256), 256, 0, s>>>(L.cp.nt, L.s_ptr.p, L.cp.t_col.p, g.g_w.p, L.tile_flops.p,
-                                                               L.next.p);
+    k_oz_pays<<<grid_for(L.cp.nt, 256), 256, 0, s>>>(L.cp.nt, L.s_ptr.p, L.cp.t_col.p, g.g_w.p, L.tile_flops.p, L.next.p);
     DBG_LAUNCH_CK();
     {
         const int64_t* src[2] = {L.s_ptr.p + L.cp.nt, (const int64_t*)L.next.p};
         int64_t h[2];
         read_i64s(src, 2, h, s);
         L.nentries = h[0];
-        if (!h[1]) return P;
+        const double pays = (double)(unsigned long long)h[1];
+        const double pack = (double)(L.a.pat.nt + L.b.pat.nt) * (double)oz_tile_bytes(L);
+        if (pays == 0.0 || (weigh && pays / kSimtFlopsPerSecond < pack / kPackBytesPerSecond)) return P;
     }
     oz_tables(L, L.a, A, s);
     oz_pack(L, L.a, A, s);

@@ -1401,6 +1401,7 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
     const int64_t nform = hk[0];
     // FP64 products of at least tc_min_flops may use the tensor cores (fp64tc.cu decides per block)
     bool tc = !bf16 && nform && (double)(unsigned long long)hk[1] >= tc_min_flops;
+    if (tc_min_flops > 0 && !groups && (double)(unsigned long long)hk[1] < kGroupFlops * nblk) tc = false;
     progress.tc = tc;
     if (tc && !groups) {
         groups = build_groups(A);
@@ -1462,7 +1463,7 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
             // group tile patterns, digit tiles and the blocks the tensor cores take (f_comp = 2)
             tcp = f64tc_prepare(A, B, groups, nform, f_rp.p,
                                 F64TcBlocks{f_row.p, f_col.p, mirror.p, f_ksum.p, f_max.p, f_at.p, f_comp.p, sym_result, by_group}, alpha,
-                                plan != nullptr, s);
+                                plan != nullptr, tc_min_flops > 0, s);
             tc = tcp != nullptr;
         }
         k_form_stats<<<grid_for(nform, 256, (int64_t)num_sms() * 8), 256, 0, s>>>(nform, f_row.p, f_col.p, f_np.p, f_ksum.p, mirror.p,

@@ -249,3 +249,32 @@ def test_rows_of_subnormals(gb):
     C = gb.Matrix(A.blk_size, A.stream)
     gb.multiply(1.0, A, B, 0.0, C, 0.0)
     _check(C, bsr.Mat.of(a), bsr.Mat.of(b))
+
+
+@pytest.mark.parametrize("kind", ["band", "random"])
+def test_products_that_the_tensor_cores_would_slow_down(gb, kind):
+    # many small blocks with little work each (grouping them would take longer than the product), and a pattern
+    # without neighbourhoods (a block or two in every tile): both stay off the tensor cores
+    nb, b = (8000, 5) if kind == "band" else (1500, 13)
+    r = np.random.default_rng(1900)
+    i = np.arange(nb)
+    if kind == "band":
+        near = i[:, None] + np.arange(-4, 5)[None, :]
+        pairs = np.stack([np.repeat(i, 9), near.ravel()], 1)
+        pairs = pairs[(pairs[:, 1] >= 0) & (pairs[:, 1] < nb)]
+    else:
+        pairs = np.concatenate([np.stack([i, i], 1), r.integers(0, nb, (20 * nb, 2))])
+    key = np.unique(pairs[:, 0].astype(np.int64) * nb + pairs[:, 1])
+    rp = np.concatenate([[0], np.cumsum(np.bincount(key // nb, minlength=nb))])
+    a, c = (synth.BlockMatrix(np.full(nb, b, np.int32), rp, (key % nb).astype(np.int32),
+                              r.uniform(-1.0, 1.0, len(key) * b * b)) for _ in range(2))
+    A, B = gb.Matrix.of(a), gb.Matrix.of(c)
+    C = gb.Matrix(A.blk_size, A.stream)
+    st = gb.multiply(1.0, A, B, 0.0, C, 0.0)
+    assert st.flops >= 64e6 and st.n_tiles == 0
+    ref = bsr.multiply(1.0, bsr.Mat.of(a), bsr.Mat.of(c))
+    rp2, col, data = C.export()
+    assert np.array_equal(rp2, ref.rp) and np.array_equal(col, ref.col)
+    # terms of a block: at most the row's blocks times b; both sums are rounded
+    n = int(np.diff(rp).max()) * b
+    assert np.abs(data - ref.data).max() <= 2 * (n + 2) * U * n

@@ -838,7 +838,7 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                 // are nearly through with the ones before it, so what lies between two batches of
                 // MMAs leaves them idle
                 bool first = true;
-                while (mask && ok) {
+                while (mask) {
                     const int st0 = stage, st1 = stage + 1 == kOzStages ? 0 : stage + 1;
                     mask &= mask - 1;
                     const bool two = mask != 0;
@@ -859,9 +859,7 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                         }
                         if (!mask) tc::mma_commit(&S.acc_full[buf]);
                     }
-                    // the lanes stay together, see mbar_wait_warp (the vote behind the MMAs: before them it took the
-                    // kernel 2% longer; what the elected lane's own waits allowed may run)
-                    ok = __all_sync(0xffffffffu, mine);
+                    __syncwarp();
                     first = false;
                     stage += two ? 2 : 1;
                     if (stage >= kOzStages) {
@@ -869,6 +867,9 @@ __global__ void __maxnreg__(64) k_oz(const __grid_constant__ OzMaps maps, OzArgs
                         phase ^= 1u;
                     }
                 }
+                // the lanes stay together, see mbar_wait_warp: one whose wait ran out only stops issuing until here
+                // (a vote before the MMAs of every step took the kernel 2% longer, one behind them 1%)
+                ok = __all_sync(0xffffffffu, mine);
                 ++n;
             }
             if (!ok && lane == 0) oz_fail(A, S);

@@ -557,15 +557,15 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
             const uint32_t sa_step = (uint32_t)np * 2u * ra, sb_step = (uint32_t)np * 2u * rb;
             const uint32_t idesc = tc::uniform(tc::instr_desc(1, kTileRows, ((wc + 15) >> 4) << 4));
             const uint32_t d_tmem = tc::uniform(tmem + (uint32_t)(acc * 128));
-            ok = tc::mbar_wait_warp(&S.acc_empty[acc], acc_phase ^ 1u, kWaitLimit);
+            bool mine = tc::mbar_wait(&S.acc_empty[acc], acc_phase ^ 1u, kWaitLimit);
             tc::fence_after_sync();
             uint32_t accumulate = 0;
             const int64_t e0 = A.s_ptr[t], e1 = A.s_ptr[t + 1];
-            for (int64_t eb0 = e0; eb0 < e1 && ok; eb0 += 32) {
+            for (int64_t eb0 = e0; eb0 < e1; eb0 += 32) {
                 const int64_t my = eb0 + lane;
                 const unsigned mym = my < e1 ? (unsigned)(A.ea[my] & 255) : 0u;
                 unsigned live = __ballot_sync(0xffffffffu, mym != 0u);
-                while (live && ok) {
+                while (live) {
                     const int x = __ffs(live) - 1;
                     live &= live - 1;
                     unsigned mask = __shfl_sync(0xffffffffu, mym, x);
@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                         lt_next_run(mask, len);
                         const uint32_t s0 = tc::uniform(s_base + (uint32_t)stage * (kStageBytesMax / 16));
                         const uint32_t n = tc::uniform((uint32_t)len);
-                        const bool mine = tc::mbar_wait(&S.full[stage], phase, kWaitLimit);
+                        mine = mine && tc::mbar_wait(&S.full[stage], phase, kWaitLimit);
                         tc::fence_after_sync();
                         if (tc::elect_one() && mine) {
                             for (uint32_t j = 0; j < n; ++j) {
@@ -588,9 +588,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                             }
                             tc::mma_commit(&S.empty[stage]);         // the stage is free once these MMAs ran
                         }
-                        // the lanes stay together, see mbar_wait_warp (behind the MMAs, off their way)
-                        ok = __all_sync(0xffffffffu, mine);
-                        if (!ok) break;
+                        __syncwarp();
                         accumulate = 1;
                         if (++stage == kStages) {
                             stage = 0;
@@ -599,7 +597,8 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_lowtier(LtArgs A) {
                     }
                 }
             }
-            ok = ok && !__shfl_sync(0xffffffffu, lt_aborted(S), 0);
+            // the lanes stay together, see mbar_wait_warp: one whose wait ran out only stops issuing until here
+            ok = __all_sync(0xffffffffu, mine) && !__shfl_sync(0xffffffffu, lt_aborted(S), 0);
             if (!ok && lane == 0) lt_fail(A, S);
             if (tc::elect_one()) tc::mma_commit(&S.acc_full[acc]);    // the accumulator is complete
             __syncwarp();

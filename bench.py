@@ -36,9 +36,11 @@ NOMINAL_BF16 = 2250.0
 NOMINAL_FP64 = 1.25
 FALLBACK_BF16_BURST, FALLBACK_BF16_SUSTAINED = 1900.0, 1700.0
 
-# DRAM bytes per flop of the FP64 block-product kernels from a capture; None: not captured since the
-# products moved to the tensor cores.
-SMM_F64_BYTES_PER_FLOP = None
+# DRAM bytes per flop of the FP64 block-product kernels (k_oz and the k_smm_f64 classes): dram__bytes_read.sum +
+# dram__bytes_write.sum over one product H H of 512 waters with 23/7 blocks, divided by its executed flops:
+# 33.25 GB / 150.9 GFLOP.  A full launch's traffic is this ratio times its flops (the larger systems are assumed to
+# re-read operands at the same rate per flop).  Reset to None whenever the kernels change.
+SMM_F64_BYTES_PER_FLOP = 0.2203
 # BF16 digit products per FP64 product on the tensor cores (eight digits, the pairs of weight 0 to 7)
 DIGIT_PRODUCTS = 36
 F64_KERNELS = "k_oz beside k_smm_f64"

@@ -252,10 +252,17 @@ dbcsr_status dbcsr_add(double alpha, dbcsr_matrix A, double beta, dbcsr_matrix B
 /*
  * C = beta * C + alpha * A * B, then every block of C with Frobenius norm
  * strictly below eps_filter is removed (diagonal blocks are always kept).
- * The sum over K of each C_IJ is taken in ascending K.  C may be the same
- * handle as A and/or B.  The result is formed on the pattern of A*B (union C's
- * pattern when beta != 0) less the candidates that the exact norm-bound
- * prescreen proves would be filtered.  prec: DBCSR_FP64, DBCSR_BF16 or DBCSR_BF16X3
+ * FP64: a block C_IJ is summed by the FP64 units, in ascending K, or, from 64 million flops
+ * a product on and where it pays, by the tensor cores from eight 8-bit digits per operand
+ * element, exactly, and rounded once.  Either way an element's error is that of an FP64 sum of its
+ * terms, (n + 4) 2^-53 (|alpha| |A| |B| + |beta| |C|)_ij at most, n the matrix dimension: blocks with
+ * elements too weak for the digits' common scale stay on the FP64 units, and so does everything
+ * when an operand holds values that are not finite or outside 2^-430 to 2^430, or when the digits
+ * do not fit the free memory.  The tensor cores work on groups of neighbouring blocks; a matrix
+ * keeps its groups from its first such product on (through put_values too) and hands them to
+ * results, and the last bits of a product depend on them.  C may be the same handle as A and/or B.
+ * The result is formed on the pattern of A*B (union C's pattern when beta != 0) less the candidates
+ * that the exact norm-bound prescreen proves would be filtered.  prec: DBCSR_FP64, DBCSR_BF16 or DBCSR_BF16X3
  * (BF16 kinds: the operands are rounded to BF16 once per call; the sums run in FP32 on
  * the tensor cores; alpha, beta, C_in and the result stay FP64).  The stack of block
  * products is built on the device (section "Local multiplication": traversal and
@@ -283,7 +290,8 @@ dbcsr_status dbcsr_multiply(double alpha, dbcsr_matrix A, dbcsr_matrix B, double
  * dbcsr_multiply_execute replays it on C's stream: C = alpha * A * B on C's planned
  * pattern, with the current values of A and B (change them with dbcsr_put_values), and
  * no host synchronisation.  A block product whose prescreen bound was below eps at plan
- * time stays excluded.
+ * time stays excluded.  Blocks on the tensor cores that the current values do not suit (see
+ * dbcsr_multiply) are formed by the FP64 units in the same execution.
  *   - A, B, C: finalized (C may be empty), C distinct from A and B, equal block sizes.
  *     While the plan lives, their arrays are pinned: put_block, finalize, filter, copy into
  *     them, multiply into C and destroy fail with DBCSR_ESTATE.  Values may change.
@@ -304,7 +312,8 @@ dbcsr_status dbcsr_multiply(double alpha, dbcsr_matrix A, dbcsr_matrix B, double
  *     block's shape (K-split where m n = 32 EF + 1).  Products with a shape of more than 17
  *     element slots per lane (m n > 544) keep the per-shape launches.
  * It concerns the blocks the FP64 units compute (dbcsr_multiply).  Every C element is summed in
- * the same order either way; the block norms differ only in rounding where the per-shape schedule uses warp pairs.  Library-wide; not from the paper.
+ * the same order either way; the block norms differ only in rounding where the per-shape
+ * schedule uses warp pairs.  Library-wide; not from the paper.
  * Errors: EINVAL (unknown mode).
  */
 #define DBCSR_SCHEDULE_PER_SHAPE 0

@@ -202,9 +202,10 @@ struct dbcsr_matrix_ {
 
     int plans = 0;                       // live multiply plans that use this matrix's arrays
 
-    // groups of blocks for the tensor-core tier: computed from this matrix (or inherited from
-    // the operand of the product that formed it) at its first BF16 product; any partition
-    // gives the same products, the groups only decide how dense the tiles are
+    // groups of blocks for the tensor cores: computed from this matrix at its first product that needs
+    // them, or inherited from the operand of the product that formed it, and kept when its values change.
+    // They decide how dense the tiles are, and through the order of the BF16 tier's FP32 sums and the common
+    // scales of the FP64 digits the last bits of a product, not its accuracy
     std::shared_ptr<dbg::Groups> groups;
 
     // staging area of put_block(s) before finalize

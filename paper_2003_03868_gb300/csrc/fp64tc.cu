@@ -74,10 +74,10 @@ constexpr int16_t kNoExp = -32768;
 constexpr int kFlagRange = 0, kFlagRedo = 1, kFlagFailed = 2, kFlags = 3;
 // Clocks of one K step of one 32-column slice charged against the FP64 pipe's flops per clock and SM
 // (1.01 TFLOP/s measured on the block products) when a tile is given to one of the two.  A K step takes
-// about 768 clocks with eight digits and half of that on average (most entries run fewer); beside the
-// FP64 pipe's kernels the balance lies lower still.  Sign iteration on 512 waters: 234 ms at 430, 231 at
-// 350, 226 at 270, 227 at 200; 23/7 product 22.6 ms at 430, 22.7 at 270, 22.3 at 200; 1,024-water product
-// 28.6, 28.0, 28.0.
+// 797 clocks with eight digits (oz_mmas) and fewer on average (most entries run fewer digits); beside the
+// FP64 pipe's kernels the balance lies lower still, and hardly matters: sign iteration on 512 waters 222.4 ms at
+// 270 and 222.6 at 200, 1,024-water product 28.3 and 28.4, ragged update 3.70 and 3.70 (before k_oz_weak, which
+// sends more to the FP64 pipe, 234 ms at 430, 231 at 350, 226 at 270, 227 at 200).
 constexpr double kStepClocks = 270.0, kSimtFlopsPerClock = 3.2;
 
 // ------------------------------------------------------------------ symbolic helpers
@@ -608,9 +608,11 @@ __device__ __forceinline__ void oz_tma4(void* dst, const void* tmap, int c0, int
 // The MMAs of one K step with ND digits.  Digit s of A times digits 0 .. ND - 1 - s of the B slice
 // (the N dimension, one digit after the other) lands in accumulators s .. ND - 1.  MMAs that
 // overlap in tensor memory at another first column wait for each other (about 110 clocks each,
-// measured), so up to seven digits all MMAs write all ND accumulators, with zero digit blocks before
-// digit 0 standing in for the pairs that do not exist; with eight digits, where that costs 1,024
-// clocks, two groups (s < 4: eight accumulators, s >= 4: the last four) take 850.
+// measured), so up to six digits all MMAs write all ND accumulators, with zero digit blocks before
+// digit 0 standing in for the pairs that do not exist.  With seven and eight digits, where that would cost 784 and
+// 1,024 clocks (an MMA takes N / 2 clocks, at least 66), there are two groups, s < 4 with all accumulators and
+// s >= 4 with the last ND - 4: 776 clocks by the MMAs' own times at eight digits, 797 measured with nothing
+// beside them.
 // al, bl: the low words of the operands' descriptors at A's digit 0 and at the first zero block of B
 // (start address and chunk distance); the high words hold the constant 128 bytes between 8-row
 // groups.

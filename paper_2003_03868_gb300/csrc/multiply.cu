@@ -1618,9 +1618,9 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
         }
         // The FP64 pipe's blocks run beside the tensor cores', on other streams: k_oz hardly uses the FP64
         // pipe, and its registers are held down so that both fit an SM.  One after the other the two took
-        // 13.9 and 28.4 ms on 512 waters (13/5, 23/7), side by side 11.4 and 22.6.  With the shapes'
-        // launches side by side too (four streams): 10.9 and 22.1, and 0.78 -> 0.26 ms on 32 waters,
-        // where a shape alone does not fill the chip.
+        // 13.9 and 28.4 ms on 512 waters (13/5, 23/7), side by side 11.4 and 22.6 (with the blocks that k_oz_weak
+        // sends back 33.2 and 27.7 for 23/7).  With the shapes' launches side by side too (four streams): 10.9
+        // and 22.1, and 0.78 -> 0.26 ms on 32 waters, where a shape alone does not fill the chip.
         std::unique_ptr<SideStreams> side;
         if (n_simt >= (tc ? 1 : 2)) {
             side.reset(new SideStreams());

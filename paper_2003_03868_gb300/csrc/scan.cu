@@ -86,8 +86,8 @@ __device__ int64_t tiles_before(const T* __restrict__ in, const unsigned long lo
 }
 
 // Exclusive prefix sums, out[n] = the total, of up to kScanJobs arrays of one length (blockIdx.y), each in
-// one pass over memory: a CTA sums its tile, publishes the sum, adds up what lies before it and writes
-// its tile.  Bound by launches at the sizes of a product's lists: scanning tiles, their sums and adding
+// one pass over memory (single-pass scan with decoupled look-back; Merrill and Garland 2016): a CTA sums its
+// tile, publishes the sum, adds up what lies before it and writes its tile.  Bound by launches at the sizes of a product's lists: scanning tiles, their sums and adding
 // the offsets back took five to eight launches an array and 0.2 ms of a product on 512 waters; short
 // arrays (ONE) are a single CTA's loop without a chain.
 template <class T, bool ONE>

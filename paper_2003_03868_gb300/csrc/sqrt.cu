@@ -135,7 +135,7 @@ dbcsr_status inverse_sqrt(dbcsr_matrix_* S, const dbcsr_sign_opts* opts, dbcsr_m
     auto W = make_like(S, s);
     // the tensor-core products group the blocks by S's couplings: those of the first product's left
     // operand, Z = 1, would leave nearly every tile empty (1,024 waters: FP64 516 ms, all on the FP64 pipe,
-    // and the mixed ladder 849 ms; so 241 and 169 ms)
+    // and the mixed ladder 849 ms; so 314 and 216 ms)
     Y->groups = build_groups(Y.get());
     Z->groups = Y->groups;
     if (A) A->groups = Y->groups;

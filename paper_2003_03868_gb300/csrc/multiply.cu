@@ -1306,8 +1306,12 @@ void multiply_once(double alpha, dbcsr_matrix_* A, dbcsr_matrix_* B, double beta
     const int32_t nblk = A->nblk;
     if (nblk > kMaxBlockRows) fail(DBCSR_ECAPACITY, "multiply: more than 262144 block rows");
     cudaStream_t s = C->stream;
-    if (A->stream != s) DBG_CK(cudaStreamSynchronize(A->stream));
-    if (B->stream != s) DBG_CK(cudaStreamSynchronize(B->stream));
+    // an operand's norms are formed on its own stream: before that stream is waited for
+    for (dbcsr_matrix_* m : {A, B}) {
+        if (m->stream == s) continue;
+        ensure_norms(m);
+        DBG_CK(cudaStreamSynchronize(m->stream));
+    }
 
     // BF16 products run on the tensor-core tier, on groups of blocks (kept with the matrices)
     const bool bf16 = is_bf16(prec);

@@ -80,3 +80,40 @@ def test_results_outlive_their_operand_and_its_stream(gb):
         assert np.linalg.norm(x - y) <= 920 * 2.0 ** -53 * np.linalg.norm(y)
         C.close()
         D.close()
+
+
+@pytest.mark.parametrize("planned", [False, True])
+def test_operands_on_another_stream_whose_norms_are_not_known(gb, planned):
+    # the operands' norms are formed on their stream, the product on its own, which has the higher priority while
+    # a third keeps the GPU busy: the product waits for the norms
+    import torch
+    rows = [synth.build_hamiltonian(synth.small(40, seed=2502 + k)).H for k in range(2)]
+    s, hi = torch.cuda.Stream(priority=0), torch.cuda.Stream(priority=-1)
+    busy = torch.cuda.Stream()
+    X = [gb.Matrix.of(h) for h in rows]
+    ref = gb.Matrix(X[0].blk_size)
+    gb.multiply(1.0, X[0], X[1], 0.0, ref, 1e-5)
+    ref = ref.export()
+    w = torch.randn(8192, 8192, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(5):
+        A, B = (gb.Matrix.of(h, s.cuda_stream) for h in rows)
+        C = gb.Matrix(A.blk_size, hi.cuda_stream)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(busy):
+            for _ in range(4):
+                torch.mm(w, w)
+        if planned:
+            plan = gb.Plan(1.0, A, B, C, 1e-5)
+            plan.execute()
+            F = gb.Matrix.from_blocks(C.blk_size, *C.export())
+            F.filter(1e-5)                           # (a plan keeps the blocks below eps, as zeros)
+            out = F.export()
+            plan.close()
+        else:
+            gb.multiply(1.0, A, B, 0.0, C, 1e-5)
+            out = C.export()
+        busy.synchronize()
+        (rp, col, x), (rp2, col2, y) = out, ref
+        assert np.array_equal(rp, rp2) and np.array_equal(col, col2)
+        assert np.linalg.norm(x - y) <= 920 * 2.0 ** -53 * np.linalg.norm(y)
